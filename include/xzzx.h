@@ -103,8 +103,7 @@ typedef struct {
  * planar lattice (Sec. "The XZZX code"), G_f = X_left Z_up Z_down X_right.
  * d must be odd, 3 <= d <= 31; another layout returns XZZX_EUNSUPPORTED.
  * Planar codes run through sampling, greedy initialisation, xzzx_anneal,
- * xzzx_anneal_variant, the decision and xzzx_decode_batch; the warp-per-chain
- * kernel, batches and the server take rotated codes only (XZZX_EUNSUPPORTED).
+ * xzzx_anneal_variant, the decision and xzzx_decode_batch; xzzx_anneal_warp, batches and the server take rotated codes only (XZZX_EUNSUPPORTED).
  * Uploads the tables to the current device.  *out is owned by the caller and
  * released with xzzx_free_code. */
 xzzx_status xzzx_make_code(int d, int layout, xzzx_code** out);
@@ -228,10 +227,11 @@ xzzx_status xzzx_anneal(const xzzx_code* code, const xzzx_schedule* sched, uint6
                         int n_shots, int restarts, const uint32_t* init, int32_t* best_E, uint32_t* best_cfg,
                         int32_t* final_E, uint32_t* final_cfg, void* stream);
 
-/* xzzx_anneal with one warp per chain instead of one thread: the lanes take a
- * colour's faces in parallel (rows in shared memory, accepted moves applied
- * with shared atomics), cutting each chain's sequential work up to 32-fold
- * for latency-bound use.  Same arguments, draws and results as xzzx_anneal. */
+/* xzzx_anneal with several lanes of a warp per chain instead of one thread
+ * (each lane holds a pair of rows and takes their faces), cutting each chain's
+ * sequential work up to 16-fold for latency-bound use.  xzzx_anneal itself
+ * does this for launches too small to fill the GPU one thread per chain; this
+ * entry point always does.  Same arguments, draws and results as xzzx_anneal. */
 xzzx_status xzzx_anneal_warp(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
                              int n_shots, int restarts, const uint32_t* init, int32_t* best_E, uint32_t* best_cfg,
                              int32_t* final_E, uint32_t* final_cfg, void* stream);
@@ -306,7 +306,7 @@ typedef struct {
 
 typedef struct {
   int32_t ctas_per_sm;    /* persistent grid = SMs x this; 0 = the occupancy maximum.  Mode 2: resident
-                             CTAs (4 chains each) per SM capped at this by padding each CTA's shared memory */
+                             four-warp CTAs per SM capped at this by padding each CTA's shared memory */
   int32_t order;          /* chunk queue: 0 = longest chunks first, 1 = segment order */
   int32_t graph_mode;     /* the mode xzzx_batch_run_graph captures: 0, 3 or 4 */
   int32_t chains_per_cta; /* chains per CTA of the annealing launches (chunk size): 128 or 256; 0 = 128 */
@@ -321,7 +321,7 @@ typedef struct {
   int64_t total_shots;
   int32_t chains_per_cta, sweep_unroll;
   int32_t n_classes;     /* distance classes present (d <= 15, 17..21, 23..31): mode 4's launches */
-  int32_t warp_ctas_per_sm; /* mode 2: resident CTAs (4 chains each) per SM, fewest over the distances */
+  int32_t warp_ctas_per_sm; /* mode 2: resident four-warp CTAs per SM, fewest over the distances */
 } xzzx_batch_info;
 
 typedef struct xzzx_batch xzzx_batch;
@@ -338,8 +338,8 @@ xzzx_status xzzx_batch_create(const xzzx_segment* segs, int n_segs, uint64_t see
  * the batch has distances both up to 17 and above), one persistent annealing
  * launch whose CTAs pull chunks (longest first) from an atomic counter, one
  * decision launch.  mode 1: the three kernels once per
- * distance (the plain form).  mode 2: as mode 1 with one warp per chain
- * (xzzx_anneal_warp).  mode 3: one greedy launch, then each distance's own
+ * distance (the plain form).  mode 2: as mode 1 with several lanes
+ * per chain (xzzx_anneal_warp).  mode 3: one greedy launch, then each distance's own
  * annealing kernel on its own stream forked from this one (largest distance
  * first, so the hardware fills one distance's tail with the next one's CTAs),
  * joined back before one decision launch; the batch owns those streams.
@@ -368,9 +368,9 @@ typedef struct {
   int32_t n_slots;          /* batches in flight at once, one stream each (1..64) */
   int32_t queue_capacity;   /* pending requests before submit returns XZZX_EBUSY */
   size_t hbm_budget_bytes;  /* device memory for all slots, split evenly (0 = 256 MiB) */
-  int32_t warp_max_requests;/* a batch of at most this many requests anneals with one warp per
-                               chain (lower latency) while the warps of all batches doing so
-                               stay within 16 per SM; otherwise one thread per chain, which
+  int32_t warp_max_requests;/* a batch of at most this many requests anneals with several lanes
+                               per chain (lower latency) while the chains of all batches doing
+                               so stay within 80 per SM; otherwise one thread per chain, which
                                has the higher throughput (0 = 16, -1 = never) */
   int32_t resident_waves;   /* register budget of all batches in flight, in GPU-fulls of the
                                annealing kernels' resident CTAs (0 = 2).  1: every admitted

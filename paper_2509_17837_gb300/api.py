@@ -170,7 +170,7 @@ def greedy_init(code, noise, seed, shot0, syndromes, restarts, randomised=True, 
 
 def anneal(code, sched, seed, shot0, init, want_cfg=True, want_final=False, best_E=None, best_cfg=None,
            final_E=None, final_cfg=None, stream=None, per_warp=False, order=ORDER_COLOUR, emin=EMIN_PER_PHASE):
-    """Alg. 2 for every chain.  per_warp selects xzzx_anneal_warp; a non-default
+    """Alg. 2 for every chain.  per_warp selects xzzx_anneal_warp (several lanes per chain); a non-default
     order (ORDER_RANDOM_SITE) or emin (EMIN_PER_ATTEMPT) selects
     xzzx_anneal_variant, the literal forms of Alg. 2 / Alg. 3."""
     n, restarts = init.shape[0], init.shape[1]
@@ -185,7 +185,7 @@ def anneal(code, sched, seed, shot0, init, want_cfg=True, want_final=False, best
     assert best_E.numel() == chains
     if order != ORDER_COLOUR or emin != EMIN_PER_PHASE:
         if per_warp:
-            raise ValueError("the warp-per-chain kernel runs the colour sweep with per-phase minima only")
+            raise ValueError("the lane-parallel kernel runs the colour sweep with per-phase minima only")
         call("xzzx_anneal_variant", code.handle, sched.handle, seed, shot0, n, restarts, int(order), int(emin),
              _ptr(init), _ptr(best_E), _ptr(best_cfg), _ptr(final_E), _ptr(final_cfg), _stream(stream))
     else:
@@ -239,7 +239,7 @@ class Batch:
     restarts, and optionally randomised (default True) and true_errors.
     Output tensors (cls, E4, recovery, fail) are allocated per segment and
     exposed as ``self.outputs``.  run(mode): 0 = one persistent launch,
-    1 = one launch per distance, 2 = as 1 with one warp per chain, 3 = the
+    1 = one launch per distance, 2 = as 1 with several lanes per chain, 3 = the
     distances' own launches concurrently on forked streams, 4 = one
     persistent launch per distance class concurrently on forked streams.
     run_graph replays graph_mode (0, 3 or 4) as a captured CUDA graph.

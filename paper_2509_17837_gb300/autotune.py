@@ -5,7 +5,7 @@ It picks, for a batch shape, by timing short runs:
 * the chain-to-hardware mapping, as the launch mode of ``Batch.run``:
   0 = one persistent launch, one chain per thread, CTAs pulling chunks of
   chains from a queue; 1 = one launch per distance, one chain per thread;
-  2 = one launch per distance, one chain per warp; 3 = each distance's own
+  2 = one launch per distance, several lanes per chain; 3 = each distance's own
   launch, concurrently on forked streams; 4 = one persistent launch per
   distance class, concurrently on forked streams;
 * for mode 0, the persistent grid in CTAs per SM (how many chains are in

@@ -1,6 +1,7 @@
 // The plain annealing launch (Alg. 2 with the Metropolis step of Alg. 3):
 // one launch per distance, one chain per thread, chains of consecutive
 // (shot, restart, coset) indices.  The per-CTA work is core::anneal_cta.
+// Launches too small to fill the GPU that way go to anneal_coop.cu.
 #include "anneal_core.cuh"
 
 namespace xzzx {
@@ -97,6 +98,11 @@ xzzx_status launch_anneal_planar(const xzzx_code* code, const xzzx_schedule* sch
                                  int n_shots, int restarts, int order, int emin, const uint32_t* init, int32_t* best_E,
                                  uint32_t* best_cfg, int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream);
 
+xzzx_status coop_is_faster(int d, int64_t n_chains, bool* yes);
+xzzx_status launch_anneal_coop(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
+                               int n_shots, int restarts, const uint32_t* init, int32_t* best_E, uint32_t* best_cfg,
+                               int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream);
+
 xzzx_status launch_anneal(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
                           int n_shots, int restarts, const uint32_t* init, int32_t* best_E, uint32_t* best_cfg,
                           int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream) {
@@ -104,6 +110,12 @@ xzzx_status launch_anneal(const xzzx_code* code, const xzzx_schedule* sched, uin
   if (code->layout == kLayoutPlanar)  // colour sweep, minimum per colour phase
     return launch_anneal_planar(code, sched, seed, shot0, n_shots, restarts, 0, 0, init, best_E, best_cfg, final_E,
                                 final_cfg, stream);
+  bool coop = false;
+  xzzx_status st = coop_is_faster(code->d, (int64_t)n_shots * restarts * 4, &coop);
+  if (st) return st;
+  if (coop)
+    return launch_anneal_coop(code, sched, seed, shot0, n_shots, restarts, init, best_E, best_cfg, final_E, final_cfg,
+                              stream);
   AnnealArgs A;
   A.keys = philox_keys(seed);
   A.chain0 = shot0 * (uint64_t)restarts * 4u;

@@ -8,7 +8,7 @@
 //          group), one persistent annealing launch whose CTAs pull chunks,
 //          longest first, from an atomic counter, and one decision launch;
 //   mode 1 (plain):   the same three kernels once per distance;
-//   mode 2 (latency): as mode 1 with one warp per chain (colour-parallel lanes).
+//   mode 2 (latency): as mode 1 with several lanes per chain.
 // Every chain uses the chain id it would get from xzzx_decode_batch on its
 // segment alone, so both modes, and per-segment calls, agree bit for bit.
 //
@@ -332,7 +332,10 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
     DistanceRange r;
     r.d = segs[order[j]].code->d;
     r.seg_begin = j;
-    while (j < n_segs && segs[order[j]].code->d == r.d) ++j;
+    while (j < n_segs && segs[order[j]].code->d == r.d) {
+      r.n_classes = std::max(r.n_classes, segs[order[j]].sched->n_classes);
+      ++j;
+    }
     r.seg_end = j;
     auto by_seg = [](const ChunkDev& c, int sidx) { return c.seg < sidx; };
     r.chunk_begin = (int)(std::lower_bound(P.byd.begin(), P.byd.end(), r.seg_begin, by_seg) - P.byd.begin());
@@ -418,15 +421,16 @@ xzzx_status launch_plan(const Plan& p, const PlanDev& d, const PhiloxKeys& K, in
                          stream)))
       return st;
     if (mode == 2) {
-      WarpLaunch W;
+      CoopLaunch W;
       W.keys = K;
       W.segs = d.segs;
-      W.chain_prefix = d.chain_prefix;
-      W.n_segs = (int)p.segs.size();
-      W.chain0 = p.chain_prefix[r.seg_begin];
-      W.n_chains = p.chain_prefix[r.seg_end] - p.chain_prefix[r.seg_begin];
-      W.smem = r.warp_smem;
-      if ((st = launch_warp_chains(r.d, W, stream))) return st;
+      W.chunks = d.byd;
+      W.chunk0 = r.chunk_begin;
+      W.n_chunks = r.chunk_end - r.chunk_begin;
+      W.nt = p.nt;
+      W.n_classes = r.n_classes;
+      W.smem = r.coop_smem;
+      if ((st = launch_coop_chunks(r.d, W, stream))) return st;
     } else if ((st = launch_chunks(r.d, p.nt, p.unroll,
                                    anneal_launch(d, K, d.byd, r.chunk_begin, r.chunk_end - r.chunk_begin, nullptr), stream))) {
       return st;
@@ -452,7 +456,7 @@ struct xzzx_batch {
   cudaGraphExec_t graph_exec = nullptr;
   int graph_mode = 0;
   int class_grid[xzzx::batch::kNumClasses] = {0, 0, 0};  // mode 4: persistent grid of each class
-  int warp_per_sm = 0;  // mode 2: resident warp-kernel CTAs per SM (fewest over the distances)
+  int warp_per_sm = 0;  // mode 2: resident CTAs of the lane-parallel kernel per SM (fewest over the distances)
   // modes 3 and 4: one side stream and one completion event per distance (or
   // class), and the fork event, created on first use
   std::vector<cudaStream_t> side;
@@ -611,7 +615,7 @@ xzzx_status xzzx_batch_create(const xzzx_segment* segs, int n_segs, uint64_t see
   b->warp_per_sm = 0;
   for (DistanceRange& r : b->plan.ranges) {
     int w_per_sm = 0;
-    if ((st = configure_warp_chains(r.d, cfg ? cfg->ctas_per_sm : 0, &r.warp_smem, &w_per_sm))) {
+    if ((st = configure_coop_chunks(r.d, cfg ? cfg->ctas_per_sm : 0, r.n_classes, &r.coop_smem, &w_per_sm))) {
       free_batch(b);
       return st;
     }
@@ -630,7 +634,7 @@ xzzx_status xzzx_batch_run(xzzx_batch* b, int mode, void* stream) {
   if (!b) return fail(XZZX_EINVAL, "batch is NULL");
   if (mode < 0 || mode > 4)
     return fail(XZZX_EINVAL,
-                "mode must be 0 (batched), 1 (one launch per distance), 2 (one warp per chain), 3 (concurrent "
+                "mode must be 0 (batched), 1 (one launch per distance), 2 (several lanes per chain), 3 (concurrent "
                 "per-distance launches) or 4 (concurrent per-class persistent launches)");
   xzzx_status st = check_device(b->device);
   if (st) return st;

@@ -54,7 +54,8 @@ struct DistanceRange {
   int d;
   int seg_begin, seg_end;        // segments [begin, end) (ordered by distance)
   int chunk_begin, chunk_end;    // chunks_byd range
-  int warp_smem = 0;             // mode 2: shared memory per CTA of the warp kernel (0: its own need)
+  int n_classes = 0;             // the most thresholds per sweep of any of its schedules
+  int coop_smem = 0;             // mode 2: shared memory per CTA of the lane-parallel kernel (0: its own need)
 };
 
 // Distance classes of the persistent kernels: d <= 15, 17..21, 23..31.
@@ -107,7 +108,7 @@ size_t descriptor_bytes(const Plan& p);
 PlanDev descriptor_layout(const Plan& p, char* dev_base);
 void pack_descriptors(const Plan& p, char* host_blob);
 // Enqueue the decode of a plan (mode 0: batched, 1: one launch per distance,
-// 2: one launch per distance with one warp per chain).  Modes 3 and 4 need
+// 2: one launch per distance with several lanes per chain).  Modes 3 and 4 need
 // side streams and are issued by the batch handle.
 xzzx_status launch_plan(const Plan& p, const PlanDev& d, const PhiloxKeys& K, int grid, int mode,
                         cudaStream_t stream);
@@ -138,20 +139,20 @@ xzzx_status launch_persistent_v(const AnnealLaunch& L, int grid, cudaStream_t st
 template <int DMAX, int NT, int U>
 xzzx_status configure_persistent_v(int* ctas_per_sm);
 
-// Per-distance warp-per-chain kernel over the chains [chain0, chain0 + n).
-struct WarpLaunch {
+// Per-distance lane-parallel kernel (mode 2) over chunks [chunk0, chunk0 + n).
+struct CoopLaunch {
   PhiloxKeys keys;
   const SegDev* segs;
-  const int64_t* chain_prefix;
-  int n_segs;
-  int64_t chain0, n_chains;
-  int smem;  // dynamic shared memory per CTA; below the kernel's need means its need
+  const ChunkDev* chunks;
+  int chunk0, n_chunks, nt;
+  int n_classes;  // the most thresholds per sweep of any of the chunks' schedules
+  int smem;       // dynamic shared memory per CTA; below the kernel's need means its need
 };
-xzzx_status launch_warp_chains(int d, const WarpLaunch& L, cudaStream_t stream);
-// Configure the distance-d warp kernel for at most cap resident CTAs per SM
-// (0: no cap) by padding its shared memory: bytes per CTA to *smem, the
+xzzx_status launch_coop_chunks(int d, const CoopLaunch& L, cudaStream_t stream);
+// Configure the distance-d lane-parallel kernel for at most cap resident CTAs
+// per SM (0: no cap) by padding its shared memory: bytes per CTA to *smem, the
 // resulting resident CTAs per SM to *ctas_per_sm.
-xzzx_status configure_warp_chains(int d, int cap, int* smem, int* ctas_per_sm);
+xzzx_status configure_coop_chunks(int d, int cap, int n_classes, int* smem, int* ctas_per_sm);
 
 }  // namespace batch
 }  // namespace xzzx

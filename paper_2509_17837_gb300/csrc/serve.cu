@@ -12,7 +12,7 @@
 // under load the next batch's CTAs already wait in hardware when a batch
 // ends).  The batch is decoded by the batched plan (one greedy launch, one
 // annealing launch of the batch distance's own kernel, one decision launch;
-// small batches on a lightly loaded GPU anneal with one warp per chain
+// small batches on a lightly loaded GPU anneal with several lanes per chain
 // instead, for latency) between a
 // host-to-device
 // copy of the syndromes and a device-to-host copy of the results; batches in
@@ -66,8 +66,8 @@ struct Slot {
   char* host_in = nullptr;   // pinned: descriptors + syndromes
   char* host_out = nullptr;  // pinned: results
   bool busy = false;
-  bool warp_mode = false;  // anneal this batch with one warp per chain
-  int64_t warps = 0;       // warps it occupies while it does
+  bool coop_mode = false;   // anneal this batch with several lanes per chain
+  int64_t coop_chains = 0;  // its chains while it does
   int64_t regs = 0;
   std::vector<Req> reqs;
   size_t off_out = 0, out_stride = 0;
@@ -89,7 +89,7 @@ struct xzzx_server {
   std::vector<xzzx::serve::Slot> slots;
   size_t slot_bytes = 0, staging_bytes = 0;
   int64_t regs_total = 0, regs_in_use = 0;
-  int64_t warp_inflight = 0;  // warps of batches annealing one warp per chain
+  int64_t coop_inflight = 0;  // chains of batches annealing with several lanes per chain
   bool started = false, stop = false;
   bool blocked = false;  // pending requests wait for budget freed by a completion
   std::deque<xzzx::serve::Req> pending;
@@ -183,7 +183,7 @@ xzzx_status issue(xzzx_server* sv, Slot& slot) {
   // One distance per batch: its own chunk kernel (mode 1) runs with that
   // distance's register allocation; the persistent form's queue over distances
   // has nothing to balance here.
-  if ((st = launch_plan(plan, pd, sv->keys, (int)plan.lpt.size(), slot.warp_mode ? 2 : 1, slot.stream))) return st;
+  if ((st = launch_plan(plan, pd, sv->keys, (int)plan.lpt.size(), slot.coop_mode ? 2 : 1, slot.stream))) return st;
   XZZX_CUDA_TRY(cudaMemcpyAsync(slot.host_out, slot.dev + o_out, out_bytes, cudaMemcpyDeviceToHost, slot.stream));
   // the device error flags after this batch, read beside its results
   XZZX_CUDA_TRY(cudaMemcpyAsync(slot.host_out + (size_t)sv->cfg.max_batch * kOutStride, sv->d_err,
@@ -215,10 +215,10 @@ void harvest(xzzx_server* sv) {
     }
     sv->device_errors |= *(const uint32_t*)(s.host_out + (size_t)sv->cfg.max_batch * kOutStride);
     sv->regs_in_use -= s.regs;
-    sv->warp_inflight -= s.warps;
+    sv->coop_inflight -= s.coop_chains;
     s.reqs.clear();
     s.regs = 0;
-    s.warps = 0;
+    s.coop_chains = 0;
     s.busy = false;
   }
   if (!sv->completed_slots.empty()) sv->cv_done.notify_all();
@@ -260,15 +260,15 @@ bool form_batch(xzzx_server* sv, Slot& slot) {
   sv->pending.swap(rest);
   slot.reqs.swap(reqs);
   slot.regs = regs;
-  // A small batch anneals one warp per chain while the warps of all batches
-  // doing so stay within 16 per SM: a lightly loaded GPU has the room, and
-  // each chain's sequential work is shorter.  Past that the batch runs one
-  // thread per chain, which has the higher throughput.
+  // A small batch anneals with several lanes per chain while the chains of all
+  // batches doing so stay within 80 per SM: a lightly loaded GPU has the room,
+  // and each chain's sequential work is shorter.  Past that the batch runs one
+  // thread per chain, which has the higher throughput (coop_is_faster).
   const int warp_max = sv->cfg.warp_max_requests == 0 ? 16 : sv->cfg.warp_max_requests;
-  const int64_t warps = (int64_t)slot.reqs.size() * 4 * sv->cfg.restarts;
-  slot.warp_mode = (int)slot.reqs.size() <= warp_max && sv->warp_inflight + warps <= (int64_t)sv->n_sm * 16;
-  slot.warps = slot.warp_mode ? warps : 0;
-  sv->warp_inflight += slot.warps;
+  const int64_t chains = (int64_t)slot.reqs.size() * 4 * sv->cfg.restarts;
+  slot.coop_mode = (int)slot.reqs.size() <= warp_max && sv->coop_inflight + chains <= (int64_t)sv->n_sm * 80;
+  slot.coop_chains = slot.coop_mode ? chains : 0;
+  sv->coop_inflight += slot.coop_chains;
   slot.busy = true;
   sv->regs_in_use += regs;
   sv->dispatched += (int64_t)slot.reqs.size();
@@ -312,9 +312,9 @@ void dispatcher_main(xzzx_server* sv) {
             sv->sticky = st;
             sv->sticky_msg = std::string("dispatch failed: ") + xzzx_last_error();
             sv->regs_in_use -= s.regs;
-            sv->warp_inflight -= s.warps;
+            sv->coop_inflight -= s.coop_chains;
             s.reqs.clear();
-            s.regs = s.warps = 0;
+            s.regs = s.coop_chains = 0;
             s.busy = false;
           }
           break;
@@ -338,10 +338,10 @@ void dispatcher_main(xzzx_server* sv) {
         sv->sticky = st;
         sv->sticky_msg = std::string("dispatch failed: ") + xzzx_last_error();
         sv->regs_in_use -= s.regs;
-        sv->warp_inflight -= s.warps;
+        sv->coop_inflight -= s.coop_chains;
         s.reqs.clear();
         s.regs = 0;
-        s.warps = 0;
+        s.coop_chains = 0;
         s.busy = false;
         break;
       }
