@@ -14,7 +14,7 @@ struct AnnealArgs {
   uint64_t chain0;  // global id of local chain 0
   int64_t n_chains;
   int restarts;
-  int n_sweeps, n_classes;
+  int n_sweeps, n_classes, n_live;
   int32_t W[4];
   const uint32_t* T;
   const int2* sig;
@@ -42,6 +42,7 @@ __device__ __forceinline__ void anneal_body(const AnnealArgs& A) {
   tab.sig = A.sig;
   tab.n_sweeps = A.n_sweeps;
   tab.n_classes = A.n_classes;
+  tab.n_live = A.n_live;
   for (int k = 0; k < 4; ++k) tab.W[k] = A.W[k];
   tab.err = A.err;
   ChainOut out;
@@ -123,6 +124,7 @@ xzzx_status launch_anneal(const xzzx_code* code, const xzzx_schedule* sched, uin
   A.restarts = restarts;
   A.n_sweeps = sched->n_sweeps;
   A.n_classes = sched->n_classes;
+  A.n_live = sched->n_live[kLayoutRotated];
   for (int k = 0; k < 4; ++k) A.W[k] = sched->noise.W[k];
   A.T = sched->d_T;
   A.sig = sched->d_sig;

@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(Form<D, NC, NP>::kThreads, kMinCtas<D, NP>)
   tab.sig = ch.sig;
   tab.n_sweeps = ch.n_sweeps;
   tab.n_classes = ch.n_classes;
+  tab.n_live = ch.n_live;
   for (int j = 0; j < 4; ++j) tab.W[j] = ch.W[j];
   tab.err = sg.code.err;
   const core::ChainOut out{sg.chain_E, nullptr, nullptr, nullptr};
@@ -197,6 +198,7 @@ xzzx_status launch_anneal_coop(const xzzx_code* code, const xzzx_schedule* sched
   A.tab.sig = sched->d_sig;
   A.tab.n_sweeps = sched->n_sweeps;
   A.tab.n_classes = sched->n_classes;
+  A.tab.n_live = sched->n_live[kLayoutRotated];
   for (int k = 0; k < 4; ++k) A.tab.W[k] = sched->noise.W[k];
   A.tab.err = code->dev.err;
   A.init = init;

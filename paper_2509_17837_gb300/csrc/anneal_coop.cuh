@@ -210,10 +210,11 @@ __device__ __forceinline__ uint32_t batch_counter(uint32_t C, uint32_t first, ui
 }
 
 // One colour phase; returns the lane's energy change.  tbl: this sweep's
-// table (shared address).  STAGED: x holds the phase's draws.  Otherwise each
+// table (shared address).  kStaged: x holds the phase's draws.  kVote: each
 // batch of columns draws into x (two areas, taken in turn) when a vote finds a
-// lane that needs it.
-template <int D, int C, bool STAGED>
+// lane that needs it.  kFrozen: no threshold is above zero, nothing is drawn.
+enum Draws { kVote, kStaged, kFrozen };
+template <int D, int C, Draws MODE>
 __device__ __forceinline__ int32_t phase(uint32_t (&P)[Shape<D>::NW], uint32_t tbl, const LaneColour& lc,
                                          const core::SaDraws& dr, const PhiloxKeys& K, uint32_t* x, int lane,
                                          uint32_t* err) {
@@ -236,7 +237,20 @@ __device__ __forceinline__ int32_t phase(uint32_t (&P)[Shape<D>::NW], uint32_t t
       face_flip<D, column_of<C>(decltype(ic)::value)>(P, lc.rows);
     }
   };
-  if constexpr (STAGED) {
+  if constexpr (MODE == kFrozen) {
+    int32_t dE[Col::n];
+    for_columns<0, Col::n>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      dE[i] = (int32_t)entry(std::integral_constant<int, Col::first + i>{}).x;
+    });
+    for_columns<0, Col::n>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      if (dE[i] <= 0) {
+        dsum += dE[i];
+        face_flip<D, column_of<C>(Col::first + i)>(P, lc.rows);
+      }
+    });
+  } else if constexpr (MODE == kStaged) {
     uint2 e[Col::n];
     uint32_t u[Col::batches][4];
     for_columns<0, Col::n>([&](auto ic) {
@@ -368,7 +382,7 @@ __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ ini
   uint32_t* stage = stage_all + (tid / G) * 2 * W;                         // sweeping warps only
   uint32_t* raw = stage_all + F::kCtaChains * 2 * W;                       // NP = 0: [kSweeps][n_classes]
   const uint32_t raw_s = (uint32_t)__cvta_generic_to_shared(raw);
-  const int n_sweeps = tab.n_sweeps, ncls = tab.n_classes;
+  const int n_sweeps = tab.n_sweeps, ncls = tab.n_classes, n_live = min(tab.n_live, n_sweeps);
 
   // The energy changes are the same in every sweep; the thresholds (zero
   // where no draw can accept) follow per set of sweeps.
@@ -392,19 +406,19 @@ __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ ini
       const uint64_t ch = chain0 + (uint64_t)(first + min(w * S::kChains + lane / G, n_chains - 1));
       base[w].init((uint32_t)ch, kTagSA | ((uint32_t)(ch >> 32) << 8), K);
     }
-    for (int t0 = 0, set = 0; t0 < n_sweeps; t0 += kSweeps, set ^= 1) {
-      produce<D, NC, NP>(t0, min(kSweeps, n_sweeps - t0), base, tab, K, tables + (uint32_t)(set * kSweeps) * kTable, upd,
+    for (int t0 = 0, set = 0; t0 < n_live; t0 += kSweeps, set ^= 1) {
+      produce<D, NC, NP>(t0, min(kSweeps, n_live - t0), base, tab, K, tables + (uint32_t)(set * kSweeps) * kTable, upd,
                           n_upd, draws + set * (F::kDrawWords / 2), warp - NC, lane);
       __syncthreads();
     }
-    if (n_sweeps > 0) __syncthreads();
+    if (n_live > 0) __syncthreads();
     return;
   }
   auto fetch = [&](int t0) {  // thresholds of sweeps [t0, t0 + kSweeps) into raw, asynchronously
-    const int n = min(kSweeps, n_sweeps - t0) * ncls;
+    const int n = min(kSweeps, n_live - t0) * ncls;
     for (int j = tid; j < n; j += F::kThreads) copy_async_u32(raw_s + 4u * (uint32_t)j, tab.T + (size_t)t0 * ncls + j);
   };
-  if (NP == 0 && n_sweeps > 0) fetch(0);
+  if (NP == 0 && n_live > 0) fetch(0);
 
   const bool active = tid / G < n_chains;
   const int64_t ci = first + (active ? tid / G : n_chains - 1);
@@ -452,8 +466,39 @@ __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ ini
 #pragma unroll
   for (int j = 0; j < NW; ++j) best[j] = P[j];
 
-  for (int t0 = 0, set = 0; t0 < n_sweeps; t0 += kSweeps, set ^= (F::kSets - 1)) {
-    const int ns = min(kSweeps, n_sweeps - t0);
+  // One sweep; x: its draws (kStaged) or the warp's two areas (kVote).
+  auto sweep = [&](auto mode, uint32_t tbl, uint32_t* x) {
+    constexpr Draws M = decltype(mode)::value;
+    // The words after colours 0, 1 and 2 (even layout), for the minimum.
+    uint32_t P0[NW], P1[NW], P2[NW];
+    const int32_t d0 = phase<D, 0, M>(P, tbl, c0, dr, K, x, lane, tab.err);
+    copy_words(P, P0);
+    to_odd(P, m_up);
+    const int32_t d1 = phase<D, 1, M>(P, tbl, c1, dr, K, M == kStaged ? x + S::kB0 * kBatchWords : x, lane, tab.err);
+    to_even(P, m_dn);
+    copy_words(P, P1);
+    const int32_t d2 =
+        phase<D, 2, M>(P, tbl, c2, dr, K, M == kStaged ? x + (S::kB0 + S::kB1) * kBatchWords : x, lane, tab.err);
+    copy_words(P, P2);
+    to_odd(P, m_up);
+    const int32_t d3 =
+        phase<D, 3, M>(P, tbl, c3, dr, K, M == kStaged ? x + (S::kB0 + 2 * S::kB1) * kBatchWords : x, lane, tab.err);
+    to_even(P, m_dn);
+    if (__any_sync(0xFFFFFFFFu, (d0 < 0) | (d1 < 0) | (d2 < 0) | (d3 < 0))) {
+      const int32_t e0 = e_lane + d0, e1 = e0 + d1, e2 = e1 + d2, e3 = e2 + d3;
+      const int32_t E0 = group_sum<G>(e0), E1 = group_sum<G>(e1), E2 = group_sum<G>(e2), E3 = group_sum<G>(e3);
+      if (min(min(E0, E1), min(E2, E3)) < E_best) {  // the earliest phase with the lowest energy
+        if (E0 < E_best) E_best = E0, copy_words(P0, best);
+        if (E1 < E_best) E_best = E1, copy_words(P1, best);
+        if (E2 < E_best) E_best = E2, copy_words(P2, best);
+        if (E3 < E_best) E_best = E3, copy_words(P, best);
+      }
+    }
+    e_lane += d0 + d1 + d2 + d3;
+  };
+
+  for (int t0 = 0, set = 0; t0 < n_live; t0 += kSweeps, set ^= (F::kSets - 1)) {
+    const int ns = min(kSweeps, n_live - t0);
     if constexpr (NP == 0) {
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();  // the fetched thresholds are in, and every warp is done with the tables
@@ -466,42 +511,32 @@ __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ ini
       }
     }
     __syncthreads();  // this set is ready (NP > 0: and the producing warps may refill the other one)
-    if (NP == 0 && t0 + kSweeps < n_sweeps) fetch(t0 + kSweeps);
+    if (NP == 0 && t0 + kSweeps < n_live) fetch(t0 + kSweeps);
     for (int s = 0; s < ns; ++s) {
       const uint32_t tbl = tables + (uint32_t)(set * kSweeps + s) * kTable;
       if (NP == 0) dr.sweep((uint32_t)(t0 + s), K);
-      constexpr bool ST = NP > 0;
-      uint32_t* x = ST ? draws + set * (F::kDrawWords / 2) + (s * NC + warp) * S::kBatches * kBatchWords
+      uint32_t* x = NP ? draws + set * (F::kDrawWords / 2) + (s * NC + warp) * S::kBatches * kBatchWords
                        : draws + warp * 2 * kBatchWords;
-      // The words after colours 0, 1 and 2 (even layout), for the minimum.
-      uint32_t P0[NW], P1[NW], P2[NW];
-      const int32_t d0 = phase<D, 0, ST>(P, tbl, c0, dr, K, x, lane, tab.err);
-      copy_words(P, P0);
-      to_odd(P, m_up);
-      const int32_t d1 = phase<D, 1, ST>(P, tbl, c1, dr, K, ST ? x + S::kB0 * kBatchWords : x, lane, tab.err);
-      to_even(P, m_dn);
-      copy_words(P, P1);
-      const int32_t d2 =
-          phase<D, 2, ST>(P, tbl, c2, dr, K, ST ? x + (S::kB0 + S::kB1) * kBatchWords : x, lane, tab.err);
-      copy_words(P, P2);
-      to_odd(P, m_up);
-      const int32_t d3 =
-          phase<D, 3, ST>(P, tbl, c3, dr, K, ST ? x + (S::kB0 + 2 * S::kB1) * kBatchWords : x, lane, tab.err);
-      to_even(P, m_dn);
-      if (__any_sync(0xFFFFFFFFu, (d0 < 0) | (d1 < 0) | (d2 < 0) | (d3 < 0))) {
-        const int32_t e0 = e_lane + d0, e1 = e0 + d1, e2 = e1 + d2, e3 = e2 + d3;
-        const int32_t E0 = group_sum<G>(e0), E1 = group_sum<G>(e1), E2 = group_sum<G>(e2), E3 = group_sum<G>(e3);
-        if (min(min(E0, E1), min(E2, E3)) < E_best) {  // the earliest phase with the lowest energy
-          if (E0 < E_best) E_best = E0, copy_words(P0, best);
-          if (E1 < E_best) E_best = E1, copy_words(P1, best);
-          if (E2 < E_best) E_best = E2, copy_words(P2, best);
-          if (E3 < E_best) E_best = E3, copy_words(P, best);
-        }
-      }
-      e_lane += d0 + d1 + d2 + d3;
+      sweep(std::integral_constant<Draws, NP ? kStaged : kVote>{}, tbl, x);
     }
   }
-  if (NP > 0 && n_sweeps > 0) __syncthreads();  // pairs with the producing warps' last
+  if (NP > 0 && n_live > 0) __syncthreads();  // pairs with the producing warps' last
+  // The frozen sweeps (see anneal_core.cuh).
+  uint32_t saved[NW];
+  const bool may_stop = !out.final_E && !out.final_cfg;
+  bool done = false;
+  for (int t = n_live, i = 0; t < n_sweeps; ++t, ++i) {
+    if ((i & (i + 1)) == 0) copy_words(P, saved);
+    sweep(std::integral_constant<Draws, kFrozen>{}, tables, nullptr);
+    if (may_stop) {
+      uint32_t diff = 0;
+#pragma unroll
+      for (int j = 0; j < NW; ++j) diff |= P[j] ^ saved[j];
+      const uint32_t same = __ballot_sync(0xFFFFFFFFu, diff == 0u) >> (lane & ~(G - 1));
+      done |= (same & ((1u << G) - 1u)) == (1u << G) - 1u;
+      if (__all_sync(0xFFFFFFFFu, done)) break;
+    }
+  }
 
   const int32_t E_final = group_sum<G>(e_lane);
   if (active && k == 0) {

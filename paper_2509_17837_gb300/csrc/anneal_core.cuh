@@ -40,6 +40,17 @@
 // so a table address is the slot base OR'd with the byte offset cut from the
 // pair word.
 //
+// Frozen sweeps.  Once every threshold is zero (at beta dE/scale > 22 for the
+// smallest positive dE) a sweep is a fixed map of the configuration that takes
+// the moves with dE <= 0 and draws nothing, so the energy never rises again.  A
+// configuration that returns after some sweeps repeats from there on at one
+// energy: the minimum can no longer change, and a warp whose 32 chains have all
+// returned is finished (unless the caller wants the state after the last
+// sweep).  Each chain is compared with its configuration saved 1, 2, 4, ...
+// sweeps apart, so any period is found.  With the usual linear schedules to 20
+// times the Nishimori beta, the last third of the sweeps is frozen and the
+// chains of a warp repeat within about 60 of them.
+//
 // Minimum tracking.  The lowest energy and its configuration are recorded at
 // the start and after every colour phase (strict improvement), in shared
 // memory.
@@ -215,8 +226,9 @@ __device__ __forceinline__ void store_rows(const Row (&R)[D], uint32_t* __restri
   }
 }
 
-// One colour phase of one sweep (row layout, d > 15).
-template <int D, int C, typename Row>
+// One colour phase of one sweep (row layout, d > 15).  LIVE = false: no
+// threshold is above zero, so a move is taken iff dE <= 0 and nothing is drawn.
+template <int D, int C, bool LIVE, typename Row>
 __device__ __forceinline__ void colour_phase(Row (&R)[D], int32_t& E, const uint2* __restrict__ L, const SaDraws& dr,
                                              const PhiloxKeys& K, uint32_t* err) {
   // Rows of this colour: a = 2j + AOFF; colour 0 ends with the bottom boundary
@@ -264,7 +276,7 @@ __device__ __forceinline__ void colour_phase(Row (&R)[D], int32_t& E, const uint
         need |= e[q].y;
       }
       uint4 r = make_uint4(0u, 0u, 0u, 0u);
-      if (__any_sync(0xFFFFFFFFu, need != 0u)) r = dr.block(((uint32_t)C << 16) | (ib << 8) | (uint32_t)g, K);
+      if (LIVE && __any_sync(0xFFFFFFFFu, need != 0u)) r = dr.block(((uint32_t)C << 16) | (ib << 8) | (uint32_t)g, K);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int j = j0 + q;
@@ -272,7 +284,7 @@ __device__ __forceinline__ void colour_phase(Row (&R)[D], int32_t& E, const uint
         const int ia = j + IAOFF;
         const uint32_t u = lane_of(r, ia & 3);
         const int32_t dE = (int32_t)e[q].x;
-        const bool acc = (dE <= 0) | (u < e[q].y);
+        const bool acc = (dE <= 0) | (LIVE && u < e[q].y);
         if (acc) {
           E += dE;
           if (C == 3 && j == 0) {
@@ -315,7 +327,7 @@ __device__ __forceinline__ void colour_phase(Row (&R)[D], int32_t& E, const uint
       for (int j = 0; j < NR; ++j)
         if (((j + IAOFF) >> 2) == g) need |= e[j].y;
       r[g] = make_uint4(0u, 0u, 0u, 0u);
-      if (__any_sync(0xFFFFFFFFu, need != 0u))
+      if (LIVE && __any_sync(0xFFFFFFFFu, need != 0u))
         r[g] = dr.block(((uint32_t)C << 16) | (ibb << 8) | (uint32_t)g, K);
     }
 #pragma unroll
@@ -323,7 +335,7 @@ __device__ __forceinline__ void colour_phase(Row (&R)[D], int32_t& E, const uint
       const int ia = j + IAOFF;
       const uint32_t u = lane_of(r[ia >> 2], ia & 3);
       const int32_t dE = (int32_t)e[j].x;
-      const bool acc = (dE <= 0) | (u < e[j].y);
+      const bool acc = (dE <= 0) | (LIVE && u < e[j].y);
       if (acc) {
         E += dE;
         const int a = 2 * j + AOFF;
@@ -495,7 +507,7 @@ __device__ __forceinline__ uint2 pair_entry(uint32_t a, uint32_t Lb, uint32_t* e
 
 // One column of faces of colour C at column b (bit s of its register, as MODE
 // says).  Lb: the warp's table slot.
-template <int D, int C, int MODE>
+template <int D, int C, int MODE, bool LIVE>
 __device__ __forceinline__ void pair_column(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E,
                                             uint32_t Lb, const SaDraws& dr, const PhiloxKeys& K, int b, uint32_t s,
                                             uint32_t* err) {
@@ -525,14 +537,14 @@ __device__ __forceinline__ void pair_column(uint32_t (&P)[PairShape<D>::H][PairS
     for (int j = 0; j < NR; ++j)
       if (((j + IAOFF) >> 2) == g) need |= e[j].y;
     r[g] = make_uint4(0u, 0u, 0u, 0u);
-    if (__any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (ib << 8) | (uint32_t)g, K);
+    if (LIVE && __any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (ib << 8) | (uint32_t)g, K);
   }
 #pragma unroll
   for (int j = 0; j < NR; ++j) {
     const int ia = j + IAOFF;
     const uint32_t u = lane_of(r[ia >> 2], ia & 3);
     const int32_t dE = (int32_t)e[j].x;
-    if ((dE <= 0) | (u < e[j].y)) {
+    if ((dE <= 0) | (LIVE && u < e[j].y)) {
       E += dE;
       if (C == 3 && j == 0) pair_flip<NW, MODE>(P[0], 0x84u, s);               // Z on BL, X on BR
       else if (C == 0 && j == NR - 1) pair_flip<NW, MODE>(P[j], 0x12u, s);     // X on TL, Z on TR
@@ -544,7 +556,7 @@ __device__ __forceinline__ void pair_column(uint32_t (&P)[PairShape<D>::H][PairS
 // The columns of colour C whose bytes start in register RG of the pair
 // words: b = 8RG at bit 0 (even-b colours), then the columns inside the
 // register, then b = 8RG + 7 across registers RG and RG + 1 (odd-b colours).
-template <int D, int C, int RG>
+template <int D, int C, int RG, bool LIVE>
 __device__ __forceinline__ void pair_register_columns(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E,
                                                       uint32_t Lb, const SaDraws& dr, const PhiloxKeys& K,
                                                       uint32_t* err) {
@@ -553,15 +565,15 @@ __device__ __forceinline__ void pair_register_columns(uint32_t (&P)[PairShape<D>
     constexpr int PB = C >> 1;
     constexpr int BMAX = PB + 2 * ((D - 1) / 2 - 1);  // the colour's last bulk column
     constexpr int B0 = 8 * RG;
-    if constexpr (PB == 0 && B0 <= BMAX) pair_column<D, C, kAt0 | (RG << 4)>(P, E, Lb, dr, K, B0, 0u, err);
+    if constexpr (PB == 0 && B0 <= BMAX) pair_column<D, C, kAt0 | (RG << 4), LIVE>(P, E, Lb, dr, K, B0, 0u, err);
     constexpr int LO = B0 + (PB == 0 ? 2 : 1);
     constexpr int HI = (B0 + 6 - PB) < BMAX ? (B0 + 6 - PB) : BMAX;
 #pragma unroll 1
     for (int b = LO; b <= HI; b += 2)
-      pair_column<D, C, kIn | (RG << 4)>(P, E, Lb, dr, K, b, 4u * (uint32_t)(b - B0), err);
+      pair_column<D, C, kIn | (RG << 4), LIVE>(P, E, Lb, dr, K, b, 4u * (uint32_t)(b - B0), err);
     if constexpr (PB == 1 && B0 + 7 <= BMAX && RG + 1 < NW)
-      pair_column<D, C, kAcross | (RG << 4)>(P, E, Lb, dr, K, B0 + 7, 28u, err);
-    pair_register_columns<D, C, RG + 1>(P, E, Lb, dr, K, err);
+      pair_column<D, C, kAcross | (RG << 4), LIVE>(P, E, Lb, dr, K, B0 + 7, 28u, err);
+    pair_register_columns<D, C, RG + 1, LIVE>(P, E, Lb, dr, K, err);
   }
 }
 
@@ -574,7 +586,7 @@ __device__ __forceinline__ uint32_t pair_bits(const uint32_t (&w)[NW], uint32_t 
 
 // One column of faces of colour C at column b >= 1 of the pair words (two
 // registers at most), the column a run-time value.
-template <int D, int C>
+template <int D, int C, bool LIVE>
 __device__ __forceinline__ void pair_column_rt(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E,
                                                uint32_t Lb, const SaDraws& dr, const PhiloxKeys& K, int b,
                                                uint32_t* err) {
@@ -606,7 +618,7 @@ __device__ __forceinline__ void pair_column_rt(uint32_t (&P)[PairShape<D>::H][Pa
     for (int j = 0; j < NR; ++j)
       if (((j + IAOFF) >> 2) == g) need |= e[j].y;
     r[g] = make_uint4(0u, 0u, 0u, 0u);
-    if (__any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (ib << 8) | (uint32_t)g, K);
+    if (LIVE && __any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (ib << 8) | (uint32_t)g, K);
   }
   using M = typename std::conditional<NW == 1, uint32_t, uint64_t>::type;
   const M m_bulk = (M)0x96u << s, m_top = (M)0x84u << s, m_bottom = (M)0x12u << s;
@@ -615,7 +627,7 @@ __device__ __forceinline__ void pair_column_rt(uint32_t (&P)[PairShape<D>::H][Pa
     const int ia = j + IAOFF;
     const uint32_t u = lane_of(r[ia >> 2], ia & 3);
     const int32_t dE = (int32_t)e[j].x;
-    if ((dE <= 0) | (u < e[j].y)) {
+    if ((dE <= 0) | (LIVE && u < e[j].y)) {
       E += dE;
       const int row = (C == 3 && j == 0) ? 0 : (C == 0 && j == NR - 1) ? j : j + JOFF;
       const M m = (C == 3 && j == 0) ? m_top : (C == 0 && j == NR - 1) ? m_bottom : m_bulk;
@@ -631,25 +643,25 @@ __device__ __forceinline__ void pair_column_rt(uint32_t (&P)[PairShape<D>::H][Pa
 // about one instruction per column for the shifted masks but cuts the sweep
 // body several-fold, which pays once the body outgrows instruction fetch
 // (d = 13, 15); at d <= 11 the per-register form is faster.
-template <int D, int C>
+template <int D, int C, bool LIVE>
 __device__ __forceinline__ void pair_bulk_columns(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E,
                                                   uint32_t Lb, const SaDraws& dr, const PhiloxKeys& K,
                                                   uint32_t* err) {
   constexpr int PB = C >> 1;
   constexpr int BMAX = PB + 2 * ((D - 1) / 2 - 1);  // the colour's last bulk column
-  if constexpr (PB == 0) pair_column<D, C, kAt0>(P, E, Lb, dr, K, 0, 0u, err);
+  if constexpr (PB == 0) pair_column<D, C, kAt0, LIVE>(P, E, Lb, dr, K, 0, 0u, err);
 #pragma unroll 1
-  for (int b = PB == 0 ? 2 : 1; b <= BMAX; b += 2) pair_column_rt<D, C>(P, E, Lb, dr, K, b, err);
+  for (int b = PB == 0 ? 2 : 1; b <= BMAX; b += 2) pair_column_rt<D, C, LIVE>(P, E, Lb, dr, K, b, err);
 }
 
 // One colour phase of one sweep (pair layout: even for colours 0 and 2, odd
 // for 1 and 3).
-template <int D, int C>
+template <int D, int C, bool LIVE>
 __device__ __forceinline__ void pair_phase(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E, uint32_t Lb,
                                            const SaDraws& dr, const PhiloxKeys& K, uint32_t* err) {
   constexpr int H = PairShape<D>::H;
-  if constexpr (D >= 13) pair_bulk_columns<D, C>(P, E, Lb, dr, K, err);
-  else pair_register_columns<D, C, 0>(P, E, Lb, dr, K, err);
+  if constexpr (D >= 13) pair_bulk_columns<D, C, LIVE>(P, E, Lb, dr, K, err);
+  else pair_register_columns<D, C, 0, LIVE>(P, E, Lb, dr, K, err);
   if constexpr (C == 1 || C == 2) {
     // Boundary column: right (b = d-1: TL and BL) for colour 1, left (b = -1:
     // TR and BR) for colour 2, over the bulk rows of the colour.
@@ -680,14 +692,14 @@ __device__ __forceinline__ void pair_phase(uint32_t (&P)[PairShape<D>::H][PairSh
       for (int j = 0; j < NR; ++j)
         if (((j + IAOFF) >> 2) == g) need |= e[j].y;
       r[g] = make_uint4(0u, 0u, 0u, 0u);
-      if (__any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (ibb << 8) | (uint32_t)g, K);
+      if (LIVE && __any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (ibb << 8) | (uint32_t)g, K);
     }
 #pragma unroll
     for (int j = 0; j < NR; ++j) {
       const int ia = j + IAOFF;
       const uint32_t u = lane_of(r[ia >> 2], ia & 3);
       const int32_t dE = (int32_t)e[j].x;
-      if ((dE <= 0) | (u < e[j].y)) {
+      if ((dE <= 0) | (LIVE && u < e[j].y)) {
         E += dE;
         if constexpr (C == 1) P[j + JOFF][RW] ^= 0x6u << RS;  // X on TL, Z on BL
         else P[j][0] ^= 0x9u;                                 // Z on TR, X on BR
@@ -742,6 +754,7 @@ struct SweepTables {
   const uint32_t* T;
   const int2* sig;
   int n_sweeps, n_classes;
+  int n_live;  // sweeps whose thresholds are not all zero come before this one (xzzx_schedule::n_live)
   int32_t W[4];
   uint32_t* err;  // the code's device error area (bounds checks of the checked build)
 };
@@ -822,25 +835,30 @@ __device__ __forceinline__ void anneal_cta_rows(const uint32_t* __restrict__ ini
   int32_t W4[4] = {tab.W[0], tab.W[1], tab.W[2], tab.W[3]};
   int32_t E = energy_of<D, Row>(R, W4);
   int32_t E_best = E;
+  const bool keep = out.best_cfg != nullptr;
+  if (keep) {
 #pragma unroll
-  for (int r = 0; r < D; ++r) best_rows[r * NT + tid] = R[r];
+    for (int r = 0; r < D; ++r) best_rows[r * NT + tid] = R[r];
+  }
   __syncwarp();
 
-#pragma unroll U
-  for (int t = 0; t < n_sweeps; ++t) {
-    dr.sweep((uint32_t)t, K);
-#define XZZX_PHASE(CC)                                                              \
-  colour_phase<D, CC, Row>(R, E, L, dr, K, tab.err);                                \
-  if (E < E_best) {                                                                 \
-    E_best = E;                                                                     \
-    _Pragma("unroll") for (int r = 0; r < D; ++r) best_rows[r * NT + tid] = R[r];   \
+#define XZZX_PHASE(CC, LIVE)                                                                    \
+  colour_phase<D, CC, LIVE, Row>(R, E, L, dr, K, tab.err);                                      \
+  if (E < E_best) {                                                                             \
+    E_best = E;                                                                                 \
+    if (keep) {                                                                                 \
+      _Pragma("unroll") for (int r = 0; r < D; ++r) best_rows[r * NT + tid] = R[r];             \
+    }                                                                                           \
   }
-    XZZX_PHASE(0)
-    XZZX_PHASE(1)
-    XZZX_PHASE(2)
-    XZZX_PHASE(3)
-#undef XZZX_PHASE
-    if (t + 1 < n_sweeps) {  // next sweep's thresholds, once every lane is done with these
+  const int n_live = min(tab.n_live, n_sweeps);
+#pragma unroll U
+  for (int t = 0; t < n_live; ++t) {
+    dr.sweep((uint32_t)t, K);
+    XZZX_PHASE(0, true)
+    XZZX_PHASE(1, true)
+    XZZX_PHASE(2, true)
+    XZZX_PHASE(3, true)
+    if (t + 1 < n_live) {  // next sweep's thresholds, once every lane is done with these
       __syncwarp();
       const uint32_t* Trow = tab.T + (size_t)(t + 1) * tab.n_classes;
       for (int k = lane; k < n_upd; k += 32) {  // only the thresholds of the dE > 0 entries change
@@ -850,6 +868,29 @@ __device__ __forceinline__ void anneal_cta_rows(const uint32_t* __restrict__ ini
       __syncwarp();
     }
   }
+  // The frozen sweeps (see above).  The minimum's rows are not kept when
+  // nobody asks for them; the saved configuration then takes their place
+  // (registers for it would cost a resident CTA).
+  const bool may_stop = !out.final_E && !out.final_cfg && !keep;
+  bool done = false;
+  for (int t = n_live, i = 0; t < n_sweeps; ++t, ++i) {
+    if (may_stop && (i & (i + 1)) == 0) {
+#pragma unroll
+      for (int r = 0; r < D; ++r) best_rows[r * NT + tid] = R[r];
+    }
+    XZZX_PHASE(0, false)
+    XZZX_PHASE(1, false)
+    XZZX_PHASE(2, false)
+    XZZX_PHASE(3, false)
+    if (may_stop) {
+      Row diff = 0;
+#pragma unroll
+      for (int r = 0; r < D; ++r) diff |= R[r] ^ best_rows[r * NT + tid];
+      done |= diff == 0;
+      if (__all_sync(0xFFFFFFFFu, done)) break;
+    }
+  }
+#undef XZZX_PHASE
 
   if (!active) return;
   *out.best_E = E_best;
@@ -914,34 +955,60 @@ __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ in
     for (int k = 0; k < NW; ++k) best[(j * NW + k) * NT + tid] = P[j][k];
   __syncwarp();
 
-#pragma unroll U
-  for (int t = 0; t < n_sweeps; ++t) {
-    dr.sweep((uint32_t)t, K);
 #define XZZX_SNAPSHOT                                                                         \
   if (E < E_best) {                                                                           \
     E_best = E;                                                                               \
     _Pragma("unroll") for (int j = 0; j < H; ++j)                                             \
     _Pragma("unroll") for (int k = 0; k < NW; ++k) best[(j * NW + k) * NT + tid] = P[j][k];   \
   }
-    pair_phase<D, 0>(P, E, Lb, dr, K, tab.err);
-    XZZX_SNAPSHOT
-    even_to_odd<D>(P);
-    pair_phase<D, 1>(P, E, Lb, dr, K, tab.err);
-    odd_to_even<D>(P);
-    XZZX_SNAPSHOT
-    pair_phase<D, 2>(P, E, Lb, dr, K, tab.err);
-    XZZX_SNAPSHOT
-    even_to_odd<D>(P);
-    pair_phase<D, 3>(P, E, Lb, dr, K, tab.err);
-    odd_to_even<D>(P);
-    XZZX_SNAPSHOT
-#undef XZZX_SNAPSHOT
-    if (t + 1 < n_sweeps) {  // next sweep's thresholds, once every lane is done with these
+#define XZZX_SWEEP(LIVE)                            \
+  pair_phase<D, 0, LIVE>(P, E, Lb, dr, K, tab.err); \
+  XZZX_SNAPSHOT                                     \
+  even_to_odd<D>(P);                                \
+  pair_phase<D, 1, LIVE>(P, E, Lb, dr, K, tab.err); \
+  odd_to_even<D>(P);                                \
+  XZZX_SNAPSHOT                                     \
+  pair_phase<D, 2, LIVE>(P, E, Lb, dr, K, tab.err); \
+  XZZX_SNAPSHOT                                     \
+  even_to_odd<D>(P);                                \
+  pair_phase<D, 3, LIVE>(P, E, Lb, dr, K, tab.err); \
+  odd_to_even<D>(P);                                \
+  XZZX_SNAPSHOT
+  const int n_live = min(tab.n_live, n_sweeps);
+#pragma unroll U
+  for (int t = 0; t < n_live; ++t) {
+    dr.sweep((uint32_t)t, K);
+    XZZX_SWEEP(true)
+    if (t + 1 < n_live) {  // next sweep's thresholds, once every lane is done with these
       __syncwarp();
       update_lut_pair(Lb, upd, n_upd, tab.T + (size_t)(t + 1) * tab.n_classes, lane);
       __syncwarp();
     }
   }
+  // The frozen sweeps (see above).
+  uint32_t saved[H][NW];
+  const bool may_stop = !out.final_E && !out.final_cfg;
+  bool done = false;
+  for (int t = n_live, i = 0; t < n_sweeps; ++t, ++i) {
+    if ((i & (i + 1)) == 0) {
+#pragma unroll
+      for (int j = 0; j < H; ++j)
+#pragma unroll
+        for (int k = 0; k < NW; ++k) saved[j][k] = P[j][k];
+    }
+    XZZX_SWEEP(false)
+    if (may_stop) {
+      uint32_t diff = 0;
+#pragma unroll
+      for (int j = 0; j < H; ++j)
+#pragma unroll
+        for (int k = 0; k < NW; ++k) diff |= P[j][k] ^ saved[j][k];
+      done |= diff == 0u;
+      if (__all_sync(0xFFFFFFFFu, done)) break;
+    }
+  }
+#undef XZZX_SWEEP
+#undef XZZX_SNAPSHOT
 
   if (!active) return;
   *out.best_E = E_best;

@@ -281,6 +281,7 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
     d.sig = s.sched->d_sig;
     d.n_sweeps = s.sched->n_sweeps;
     d.n_classes = s.sched->n_classes;
+    d.n_live = s.sched->n_live[kLayoutRotated];
     for (int k = 0; k < 4; ++k) d.W[k] = s.sched->noise.W[k];
     P.cta_prefix[j + 1] = P.cta_prefix[j] + (int64_t)s.n_shots * d.greedy_groups;
     if (s.code->d <= greedy::kListMaxD) P.list_cta_end = P.cta_prefix[j + 1];
@@ -299,6 +300,7 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
       ch.sig = s.sched->d_sig;
       ch.n_sweeps = s.sched->n_sweeps;
       ch.n_classes = s.sched->n_classes;
+      ch.n_live = s.sched->n_live[kLayoutRotated];
       for (int k = 0; k < 4; ++k) ch.W[k] = s.sched->noise.W[k];
       chunks.push_back(ch);
     }

@@ -27,6 +27,7 @@ __device__ __forceinline__ void run_chunk(const ChunkDev& ch, const SegDev& sg, 
   tab.sig = ch.sig;
   tab.n_sweeps = ch.n_sweeps;
   tab.n_classes = ch.n_classes;
+  tab.n_live = ch.n_live;
   for (int k = 0; k < 4; ++k) tab.W[k] = ch.W[k];
   tab.err = sg.code.err;
   core::ChainOut out;
@@ -38,8 +39,13 @@ __device__ __forceinline__ void run_chunk(const ChunkDev& ch, const SegDev& sg, 
 }
 
 // Register bounds: kernels on the pair path (d <= 15) are held to 1024
-// threads per SM (64 registers); kernels on the row path keep the compiler's
-// choice for their CTA size.
+// threads per SM (64 registers); kernels on the row path to 640 (d <= 21, 96
+// registers), 512 (d <= 27, 128) or 384 (160), the persistent ones to 512 (up
+// to d = 21) or 384, none of which spills.  Left alone, the compiler takes 240
+// registers for the persistent kernels: two CTAs per SM.
+template <int D>
+constexpr int kRowThreads = D <= 21 ? 640 : D <= 27 ? 512 : 384;
+
 template <int D, int NT, int U>
 __global__ void __launch_bounds__(NT, (1024 / NT)) anneal_chunks_kernel(const __grid_constant__ AnnealLaunch L) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -47,7 +53,7 @@ __global__ void __launch_bounds__(NT, (1024 / NT)) anneal_chunks_kernel(const __
   run_chunk<D, NT, U>(ch, L.segs[ch.seg], L.keys, smem);
 }
 template <int D, int NT, int U>
-__global__ void __launch_bounds__(NT) anneal_chunks_kernel_rows(const __grid_constant__ AnnealLaunch L) {
+__global__ void __launch_bounds__(NT, kRowThreads<D> / NT) anneal_chunks_kernel_rows(const __grid_constant__ AnnealLaunch L) {
   extern __shared__ __align__(16) uint8_t smem[];
   const ChunkDev ch = L.chunks[L.chunk0 + blockIdx.x];
   run_chunk<D, NT, U>(ch, L.segs[ch.seg], L.keys, smem);
@@ -89,7 +95,7 @@ __global__ void __launch_bounds__(NT, (1024 / NT)) anneal_persistent_kernel(cons
   persistent_body<DMAX, NT, U>(L);
 }
 template <int DMAX, int NT, int U>
-__global__ void __launch_bounds__(NT) anneal_persistent_kernel_rows(const __grid_constant__ AnnealLaunch L) {
+__global__ void __launch_bounds__(NT, (DMAX <= 21 ? 512 : 384) / NT) anneal_persistent_kernel_rows(const __grid_constant__ AnnealLaunch L) {
   persistent_body<DMAX, NT, U>(L);
 }
 template <int DMAX, int NT, int U>

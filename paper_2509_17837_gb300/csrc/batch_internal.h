@@ -28,7 +28,7 @@ struct SegDev {
   // schedule (also carried by every chunk of the segment)
   const uint32_t* T;
   const int2* sig;
-  int n_sweeps, n_classes;
+  int n_sweeps, n_classes, n_live;
   int32_t W[4];
 };
 
@@ -38,7 +38,7 @@ struct ChunkDev {
   int seg, d, first_chain, n_chains;
   const uint32_t* T;
   const int2* sig;
-  int n_sweeps, n_classes;
+  int n_sweeps, n_classes, n_live;
   int32_t W[4];
 };
 

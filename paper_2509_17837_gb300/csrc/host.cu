@@ -433,6 +433,14 @@ xzzx_status xzzx_make_schedule(const xzzx_noise* noise, int kind, int n_sweeps, 
     for (int k = 0; k < s->n_classes; ++k)
       s->T[(size_t)t * s->n_classes + k] = threshold_of(beta, s->dE_class[k], noise->scale);
   }
+  for (int layout = 0; layout < 2; ++layout) {
+    std::vector<char> used(s->n_classes, 0);
+    for (int i = layout ? kSigRot : 0; i < (layout ? kSigTable : kSigRot); ++i)
+      if (s->sig_class[i] >= 0) used[s->sig_class[i]] = 1;
+    for (int k = 0; k < s->n_classes; ++k)
+      for (int t = n_sweeps; used[k] && t > s->n_live[layout]; --t)
+        if (s->T[(size_t)(t - 1) * s->n_classes + k]) s->n_live[layout] = t;
+  }
   std::vector<int2> sig(kSigTable);
   for (int i = 0; i < kSigTable; ++i) sig[i] = make_int2(s->sig_dE[i], s->sig_class[i]);
   if (!has_device()) {  // host tables only; launches with this handle are refused

@@ -175,6 +175,10 @@ struct xzzx_schedule {
   std::vector<uint32_t> T;              // n_sweeps x n_classes
   std::vector<int32_t> sig_dE;          // kSigTable entries
   std::vector<int32_t> sig_class;       // kSigTable entries, class index or -1 (dE <= 0)
+  // Sweeps up to the last in which a move that raises the energy can be
+  // accepted (any threshold above zero), by code layout: from there on a sweep
+  // takes the moves with dE <= 0 and no other, whatever the draws.
+  int n_live[2] = {0, 0};
   uint32_t* d_T = nullptr;              // device copy of T (at least one row)
   int2* d_sig = nullptr;                // device (dE, class) per compact signature
 };

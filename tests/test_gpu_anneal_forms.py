@@ -33,3 +33,35 @@ def test_thread_and_lane_forms_agree(env, d):
     for k in thread:
         assert torch.equal(thread[k], lanes[k]), k
         assert torch.equal(thread[k][:1], few[k]), k
+
+
+@pytest.mark.parametrize("d,eta", [(3, 10.0), (5, 100.0), (11, 100.0), (15, 1.0), (17, 100.0), (21, 1.0), (31, 1000.0)])
+def test_stopping_in_the_frozen_sweeps_changes_no_minimum(env, d, eta):
+    """Past the last sweep with a threshold above zero a warp whose chains all
+    repeat stops, unless the final states are asked for: the minima with and
+    without them are the same, in the thread form, both lane forms and a batch."""
+    X, torch = env
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    restarts = 32
+    shots = (144 * n_sm) // (4 * restarts) + 1
+    code, noise = X.Code(d), X.noise_from_eta(0.15, eta)
+    sched = X.Schedule(noise, 150, 0.1, 60.0)  # frozen from about a fifth of the sweeps
+    _, T = sched.table()
+    assert not T[-1].any() and T[0].any()
+    _, syn = X.sample_errors(code, noise, 9, 0, shots)
+    init, cbits = X.greedy_init(code, noise, 9, 0, syn, restarts)
+    full = X.anneal(code, sched, 9, 0, init, want_cfg=True, want_final=True)
+    for per_warp in (False, True):
+        got = X.anneal(code, sched, 9, 0, init, want_cfg=True, per_warp=per_warp)
+        assert torch.equal(got["best_E"], full["best_E"]) and torch.equal(got["best_cfg"], full["best_cfg"])
+        got = X.anneal(code, sched, 9, 0, init, want_cfg=False, per_warp=per_warp)
+        assert torch.equal(got["best_E"], full["best_E"])
+        few = X.anneal(code, sched, 9, 0, init[:2].contiguous(), want_cfg=True, per_warp=per_warp)
+        assert torch.equal(few["best_E"], full["best_E"][:2]) and torch.equal(few["best_cfg"], full["best_cfg"][:2])
+    want = X.decode_reduce(code, init, cbits, full["best_E"])
+    b = X.Batch([dict(code=code, noise=noise, sched=sched, shot0=0, syndromes=syn, restarts=restarts)], 9)
+    for mode in (0, 1, 2):
+        b.run(mode)
+        torch.cuda.synchronize()
+        assert all(torch.equal(b.outputs[0][k], want[k]) for k in ("cls", "E4", "recovery"))
+    b.close()
