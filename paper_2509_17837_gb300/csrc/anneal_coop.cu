@@ -2,7 +2,7 @@
 // and schedule (xzzx_anneal_warp, and xzzx_anneal when its chains do not fill
 // the GPU one per thread), and batches (batch mode 2, the server's small
 // batches).
-#include "anneal_coop.cuh"
+#include "anneal_coop_launch.cuh"
 #include "batch_internal.h"
 
 #include <algorithm>
@@ -14,39 +14,12 @@ xzzx_status check_anneal_args(const xzzx_code*, const xzzx_schedule*, int, int);
 namespace coop {
 namespace {
 
-struct Args {
-  PhiloxKeys keys;
-  uint64_t chain0;
-  int64_t n_chains;
-  core::SweepTables tab;
-  const uint32_t* init;
-  int32_t* best_E;
-  uint32_t* best_cfg;
-  int32_t* final_E;
-  uint32_t* final_cfg;
-};
-
-// Resident CTAs per SM the forms are register-bounded for (what their shared
-// memory allows).
-template <int D, int NP>
-constexpr int kMinCtas = NP ? 3 : 4;
-
-template <int D, int NC, int NP>
-__global__ void __launch_bounds__(Form<D, NC, NP>::kThreads, kMinCtas<D, NP>) anneal_coop_kernel(const __grid_constant__ Args A) {
-  constexpr int kCta = Form<D, NC, NP>::kCtaChains;
-  extern __shared__ __align__(16) uint8_t smem[];
-  const int64_t first = (int64_t)blockIdx.x * kCta;
-  const core::ChainOut out{A.best_E, A.best_cfg, A.final_E, A.final_cfg};
-  anneal_coop_cta<D, NC, NP>(A.init, A.chain0, first, (int)min((int64_t)kCta, A.n_chains - first), out, A.tab, A.keys,
-                             smem);
-}
-
 // Batched form: the chunks of one distance, each cut into CTAs of kCtaChains
 // chains (so a CTA's chains share a segment and its thresholds).
-template <int D, int NC, int NP>
-__global__ void __launch_bounds__(Form<D, NC, NP>::kThreads, kMinCtas<D, NP>)
+template <class Geo, int NC, int NP>
+__global__ void __launch_bounds__(Form<Geo, NC, NP>::kThreads, kMinCtas<NP>)
     coop_chunks_kernel(const __grid_constant__ batch::CoopLaunch L) {
-  constexpr int kCta = Form<D, NC, NP>::kCtaChains;
+  constexpr int kCta = Form<Geo, NC, NP>::kCtaChains;
   extern __shared__ __align__(16) uint8_t smem[];
   const int per_chunk = L.nt / kCta;
   const batch::ChunkDev ch = L.chunks[L.chunk0 + blockIdx.x / per_chunk];
@@ -62,95 +35,38 @@ __global__ void __launch_bounds__(Form<D, NC, NP>::kThreads, kMinCtas<D, NP>)
   for (int j = 0; j < 4; ++j) tab.W[j] = ch.W[j];
   tab.err = sg.code.err;
   const core::ChainOut out{sg.chain_E, nullptr, nullptr, nullptr};
-  anneal_coop_cta<D, NC, NP>(sg.init, sg.shot0 * (uint64_t)sg.restarts * 4u, (int64_t)ch.first_chain + first,
+  anneal_coop_cta<Geo, NC, NP>(sg.init, sg.shot0 * (uint64_t)sg.restarts * 4u, (int64_t)ch.first_chain + first,
                              min(kCta, ch.n_chains - first), out, tab, L.keys, smem);
 }
 
-xzzx_status sm_count(int* n_sm) {
-  int dev = 0;
-  XZZX_CUDA_TRY(cudaGetDevice(&dev));
-  XZZX_CUDA_TRY(cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev));
-  return XZZX_OK;
-}
-
-xzzx_status shared_limit(int* optin) {
-  int dev = 0;
-  XZZX_CUDA_TRY(cudaGetDevice(&dev));
-  XZZX_CUDA_TRY(cudaDeviceGetAttribute(optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  return XZZX_OK;
-}
-
-// Allow a kernel the device's whole shared memory (the tables of a schedule
-// with many energy classes, or an occupancy cap's padding).
-template <typename F>
-xzzx_status allow_shared(F kernel) {
-  int optin = 0;
-  xzzx_status st = shared_limit(&optin);
-  if (st) return st;
-  XZZX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-  XZZX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared));
-  return XZZX_OK;
-}
-
-template <int D, int NC, int NP>
-xzzx_status launch_form(const Args& A, cudaStream_t stream) {
-  using F = Form<D, NC, NP>;
-  static DeviceOnce once;
-  xzzx_status st = once.run([] { return allow_shared(anneal_coop_kernel<D, NC, NP>); });
-  if (st) return st;
-  const int64_t grid = (A.n_chains + F::kCtaChains - 1) / F::kCtaChains;
-  if (grid > 0x7FFFFFFF) return fail(XZZX_EINVAL, "too many chains for one launch");
-  anneal_coop_kernel<D, NC, NP><<<(unsigned)grid, F::kThreads, F::smem_bytes(A.tab.n_classes), stream>>>(A);
-  XZZX_CUDA_TRY(cudaGetLastError());
-  return XZZX_OK;
-}
-// The producing form runs while every CTA (one sweeping warp, kChains chains)
-// is resident at once, about three per SM; past that its unconditional draws
-// cost more issue slots than they save, and four sweeping warps per CTA share
-// the tables.  400 sweeps at d = 11, producing / plain form, ms: 0.24 / 0.46 at
-// 128 chains, 0.30 / 0.50 at 1024, 0.40 / 0.49 at 2048, 0.69 / 0.59 at 4096.
-template <int D>
-bool producing(int64_t n_chains, int n_sm) {
-  return n_chains <= (int64_t)3 * n_sm * Form<D, 1, 3>::kCtaChains;
-}
-
-template <int D>
-xzzx_status launch_d(const Args& A, cudaStream_t stream) {
-  int n_sm = 0;
-  xzzx_status st = sm_count(&n_sm);
-  if (st) return st;
-  return producing<D>(A.n_chains, n_sm) ? launch_form<D, 1, 3>(A, stream) : launch_form<D, 4, 0>(A, stream);
-}
-
-template <int D, int NC, int NP>
+template <class Geo, int NC, int NP>
 xzzx_status chunks_form(const batch::CoopLaunch& L, cudaStream_t stream) {
-  using F = Form<D, NC, NP>;
+  using F = Form<Geo, NC, NP>;
   static DeviceOnce once;
-  xzzx_status st = once.run([] { return allow_shared(coop_chunks_kernel<D, NC, NP>); });
+  xzzx_status st = once.run([] { return allow_shared(coop_chunks_kernel<Geo, NC, NP>); });
   if (st) return st;
   const size_t smem = std::max(F::smem_bytes(L.n_classes), (size_t)std::max(L.smem, 0));
   const int64_t grid = (int64_t)L.n_chunks * (L.nt / F::kCtaChains);
   if (grid > 0x7FFFFFFF) return fail(XZZX_EINVAL, "too many chains for one launch");
-  coop_chunks_kernel<D, NC, NP><<<(unsigned)grid, F::kThreads, smem, stream>>>(L);
+  coop_chunks_kernel<Geo, NC, NP><<<(unsigned)grid, F::kThreads, smem, stream>>>(L);
   XZZX_CUDA_TRY(cudaGetLastError());
   return XZZX_OK;
 }
-template <int D>
-xzzx_status chunks_d(const batch::CoopLaunch& L, cudaStream_t stream) {
+template <class Geo>
+xzzx_status chunks_g(const batch::CoopLaunch& L, cudaStream_t stream) {
   if (L.n_chunks <= 0) return XZZX_OK;
   int n_sm = 0;
   xzzx_status st = sm_count(&n_sm);
   if (st) return st;
   // An occupancy cap (L.smem) is one of the plain form's CTAs.
-  return L.smem == 0 && producing<D>((int64_t)L.n_chunks * L.nt, n_sm) ? chunks_form<D, 1, 3>(L, stream)
-                                                                       : chunks_form<D, 4, 0>(L, stream);
+  return L.smem == 0 && producing<Geo>((int64_t)L.n_chunks * L.nt, n_sm) ? chunks_form<Geo, 1, 3>(L, stream)
+                                                                       : chunks_form<Geo, 4, 0>(L, stream);
 }
 
-template <int D>
-xzzx_status configure_d(int cap, int n_classes, int* smem_out, int* ctas_per_sm) {
-  using F = Form<D, 4, 0>;
-  xzzx_status st = allow_shared(coop_chunks_kernel<D, 4, 0>);
+template <class Geo>
+xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm) {
+  using F = Form<Geo, 4, 0>;
+  xzzx_status st = allow_shared(coop_chunks_kernel<Geo, 4, 0>);
   if (st) return st;
   size_t smem = F::smem_bytes(n_classes);
   int dev = 0, per_sm_bytes = 0, reserved = 0, optin = 0;
@@ -162,7 +78,7 @@ xzzx_status configure_d(int cap, int n_classes, int* smem_out, int* ctas_per_sm)
     const long pad = ((long)per_sm_bytes / cap - reserved) & ~15L;
     smem = std::max(smem, (size_t)std::min<long>(pad, optin));
   }
-  XZZX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_chunks_kernel<D, 4, 0>, F::kThreads, smem));
+  XZZX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_chunks_kernel<Geo, 4, 0>, F::kThreads, smem));
   *smem_out = cap > 0 ? (int)smem : 0;
   return XZZX_OK;
 }
@@ -190,26 +106,12 @@ xzzx_status coop_is_faster(int d, int64_t n_chains, bool* yes) {
 xzzx_status launch_anneal_coop(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
                                int n_shots, int restarts, const uint32_t* init, int32_t* best_E, uint32_t* best_cfg,
                                int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream) {
-  coop::Args A;
-  A.keys = philox_keys(seed);
-  A.chain0 = shot0 * (uint64_t)restarts * 4u;
-  A.n_chains = (int64_t)n_shots * restarts * 4;
-  A.tab.T = sched->d_T;
-  A.tab.sig = sched->d_sig;
-  A.tab.n_sweeps = sched->n_sweeps;
-  A.tab.n_classes = sched->n_classes;
-  A.tab.n_live = sched->n_live[kLayoutRotated];
-  for (int k = 0; k < 4; ++k) A.tab.W[k] = sched->noise.W[k];
-  A.tab.err = code->dev.err;
-  A.init = init;
-  A.best_E = best_E;
-  A.best_cfg = best_cfg;
-  A.final_E = final_E;
-  A.final_cfg = final_cfg;
+  const coop::Args A = coop::make_args(code, sched, seed, shot0, n_shots, restarts, init, best_E, best_cfg, final_E,
+                                       final_cfg);
   switch (code->d) {
 #define XZZX_CASE(DD) \
   case DD:            \
-    return coop::launch_d<DD>(A, stream);
+    return coop::launch_g<coop::RotLanes<DD>>(A, stream);
     XZZX_ALL_D(XZZX_CASE)
 #undef XZZX_CASE
     default:
@@ -223,7 +125,7 @@ xzzx_status configure_coop_chunks(int d, int cap, int n_classes, int* smem, int*
   switch (d) {
 #define XZZX_CASE(DD) \
   case DD:            \
-    return coop::configure_d<DD>(cap, n_classes, smem, ctas_per_sm);
+    return coop::configure_g<coop::RotLanes<DD>>(cap, n_classes, smem, ctas_per_sm);
     XZZX_ALL_D(XZZX_CASE)
 #undef XZZX_CASE
     default:
@@ -235,7 +137,7 @@ xzzx_status launch_coop_chunks(int d, const CoopLaunch& L, cudaStream_t stream) 
   switch (d) {
 #define XZZX_CASE(DD) \
   case DD:            \
-    return coop::chunks_d<DD>(L, stream);
+    return coop::chunks_g<coop::RotLanes<DD>>(L, stream);
     XZZX_ALL_D(XZZX_CASE)
 #undef XZZX_CASE
     default:

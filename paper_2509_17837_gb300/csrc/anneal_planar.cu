@@ -281,19 +281,30 @@ __global__ void __launch_bounds__(kPThreads) anneal_planar_kernel(const __grid_c
 
 }  // namespace
 
+xzzx_status coop_planar_is_faster(int d, int64_t n_chains, bool* yes);
+xzzx_status launch_anneal_coop_planar(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
+                                      int n_shots, int restarts, const uint32_t* init, int32_t* best_E,
+                                      uint32_t* best_cfg, int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream);
 xzzx_status launch_anneal_planar_reg(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
                                      int n_shots, int restarts, const uint32_t* init, int32_t* best_E,
                                      uint32_t* best_cfg, int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream);
 
-// Launch for a planar code (arguments checked by the caller): the colour sweep
-// with per-phase minima runs register-resident up to d = 15, everything else
-// in the table-driven kernel below.
+// Launch for a planar code (arguments checked by the caller).  The colour sweep
+// with per-phase minima runs one thread per chain in registers, or with several
+// lanes per chain (small launches, and d > 15, where a chain's rows outgrow one
+// thread's registers); the literal forms run in the table-driven kernel above.
 xzzx_status launch_anneal_planar(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
                                  int n_shots, int restarts, int order, int emin, const uint32_t* init, int32_t* best_E,
                                  uint32_t* best_cfg, int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream) {
-  if (order == 0 && emin == 0 && code->d <= 15)
-    return launch_anneal_planar_reg(code, sched, seed, shot0, n_shots, restarts, init, best_E, best_cfg, final_E,
-                                    final_cfg, stream);
+  if (order == 0 && emin == 0) {
+    bool coop = false;
+    xzzx_status st = coop_planar_is_faster(code->d, (int64_t)n_shots * restarts * 4, &coop);
+    if (st) return st;
+    return coop ? launch_anneal_coop_planar(code, sched, seed, shot0, n_shots, restarts, init, best_E, best_cfg, final_E,
+                                            final_cfg, stream)
+                : launch_anneal_planar_reg(code, sched, seed, shot0, n_shots, restarts, init, best_E, best_cfg, final_E,
+                                           final_cfg, stream);
+  }
   PlanarArgs A;
   A.keys = philox_keys(seed);
   A.chain0 = shot0 * (uint64_t)restarts * 4u;

@@ -35,6 +35,30 @@ def test_thread_and_lane_forms_agree(env, d):
         assert torch.equal(thread[k][:1], few[k]), k
 
 
+@pytest.mark.parametrize("d", range(3, 32, 2))
+def test_planar_forms_agree(env, d):
+    """On the planar lattice (d <= 15: one thread per chain, then several lanes;
+    above: lanes with every warp sweeping, then with producing warps)."""
+    X, torch = env
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    restarts = 37
+    shots = (128 * n_sm) // (4 * restarts) + 2
+    code, noise = X.Code(d, X.LAYOUT_PLANAR), X.noise_from_eta(0.13, 5.0, X.CONVENTION_PAPER)
+    _, syn = X.sample_errors(code, noise, 5, 7, shots)
+    init, _ = X.greedy_init(code, noise, 5, 7, syn, restarts)
+    for n, b0, b1 in ((11, 0.9, 1.0), (60, 0.1, 60.0)):  # the second freezes
+        sched = X.Schedule(noise, n, b0, b1)
+        many = X.anneal(code, sched, 5, 7, init, want_cfg=True, want_final=True)
+        no_final = X.anneal(code, sched, 5, 7, init, want_cfg=True)
+        assert torch.equal(no_final["best_E"], many["best_E"]) and torch.equal(no_final["best_cfg"], many["best_cfg"])
+        for take in (1, 1 + 40 * n_sm // (4 * restarts)):
+            few = X.anneal(code, sched, 5, 7, init[:take].contiguous(), want_cfg=True, want_final=True)
+            for k in many:
+                assert torch.equal(many[k][:take], few[k]), (k, take)
+            few = X.anneal(code, sched, 5, 7, init[:take].contiguous(), want_cfg=False)
+            assert torch.equal(many["best_E"][:take], few["best_E"])
+
+
 @pytest.mark.parametrize("d,eta", [(3, 10.0), (5, 100.0), (11, 100.0), (15, 1.0), (17, 100.0), (21, 1.0), (31, 1000.0)])
 def test_stopping_in_the_frozen_sweeps_changes_no_minimum(env, d, eta):
     """Past the last sweep with a threshold above zero a warp whose chains all
