@@ -70,9 +70,9 @@ xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm)
   if (st) return st;
   size_t smem = F::smem_bytes(n_classes);
   int dev = 0, per_sm_bytes = 0, reserved = 0, optin = 0;
-  if ((st = shared_limit(&optin))) return st;
   XZZX_CUDA_TRY(cudaGetDevice(&dev));
   XZZX_CUDA_TRY(cudaDeviceGetAttribute(&per_sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+  XZZX_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   XZZX_CUDA_TRY(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
   if (cap > 0) {
     const long pad = ((long)per_sm_bytes / cap - reserved) & ~15L;

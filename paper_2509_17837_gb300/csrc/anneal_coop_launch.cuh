@@ -64,26 +64,6 @@ xzzx_status sm_count(int* n_sm) {
   return XZZX_OK;
 }
 
-xzzx_status shared_limit(int* optin) {
-  int dev = 0;
-  XZZX_CUDA_TRY(cudaGetDevice(&dev));
-  XZZX_CUDA_TRY(cudaDeviceGetAttribute(optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  return XZZX_OK;
-}
-
-// Allow a kernel the device's whole shared memory (the tables of a schedule
-// with many energy classes, or an occupancy cap's padding).
-template <typename F>
-xzzx_status allow_shared(F kernel) {
-  int optin = 0;
-  xzzx_status st = shared_limit(&optin);
-  if (st) return st;
-  XZZX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-  XZZX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared));
-  return XZZX_OK;
-}
-
 template <class Geo, int NC, int NP>
 xzzx_status launch_form(const Args& A, cudaStream_t stream) {
   using F = Form<Geo, NC, NP>;

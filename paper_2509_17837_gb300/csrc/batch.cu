@@ -90,7 +90,6 @@ xzzx_status configure_persistent(int dmax, int nt, int unroll, int* ctas_per_sm)
 
 namespace {
 
-constexpr int kGreedyWarps = greedy::kWarps;
 constexpr int kReduceWarps = 4;
 
 // Index of the segment whose [prefix[s], prefix[s+1]) range holds x.
@@ -112,20 +111,20 @@ struct GreedyLaunch {
   int64_t cta0;
 };
 
-template <bool L>
-__global__ void __launch_bounds__(kGreedyWarps * 32, L ? greedy::RotGeo::kMinCtasLists : 1)
+template <int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, 32 / kWarps)
     greedy_batch_kernel(const __grid_constant__ GreedyLaunch G) {
-  __shared__ greedy::SharedT<greedy::RotGeo, L> S;
+  extern __shared__ __align__(16) uint8_t smem[];
   const int64_t b = G.cta0 + blockIdx.x;
   const int s = find_segment(G.cta_prefix, G.n_segs, b);
   const SegDev& sg = G.segs[s];
   const int64_t local = b - G.cta_prefix[s];
   const int64_t k = local / sg.greedy_groups;
   const int group = (int)(local % sg.greedy_groups);
-  greedy::greedy_cta<greedy::RotGeo, L>(sg.code, G.keys, sg.shot0 + (uint64_t)k, group, sg.restarts, sg.greedy_rpw,
-                                        sg.randomised, sg.Wt_x, sg.Wt_z, sg.syndromes + (size_t)k * sg.code.sw,
-                                        sg.init + (size_t)k * sg.restarts * 2 * sg.code.w,
-                                        sg.cbits + (size_t)k * sg.restarts, S);
+  greedy::greedy_cta<greedy::RotGeo, kWarps>(sg.code, G.keys, sg.shot0 + (uint64_t)k, group, sg.greedy_groups, sg.greedy_cols, sg.restarts,
+                                     sg.randomised, sg.Wt_x, sg.Wt_z, sg.syndromes + (size_t)k * sg.code.sw,
+                                     sg.init + (size_t)k * sg.restarts * 2 * sg.code.w, sg.cbits + (size_t)k * sg.restarts,
+                                     smem);
 }
 
 struct ReduceLaunch {
@@ -160,16 +159,24 @@ xzzx_status run_greedy(const Plan& p, const PlanDev& d, const PhiloxKeys& K, int
   G.segs = d.segs;
   G.cta_prefix = d.cta_prefix;
   G.n_segs = (int)p.segs.size();
-  // Segments are ordered by distance: CTAs before list_cta_end (d <= 17) run
-  // the kernel with candidate lists, the rest the one without.
-  const int64_t end = cta0 + n_ctas, split = std::min(std::max(p.list_cta_end, cta0), end);
+  static DeviceOnce once;
+  xzzx_status st = once.run([]() -> xzzx_status {
+    xzzx_status e = allow_shared(greedy_batch_kernel<greedy::kSmallWarps>);
+    return e ? e : allow_shared(greedy_batch_kernel<greedy::kLargeWarps>);
+  });
+  if (st) return st;
+  // Segments are ordered by distance: CTAs before small_cta_end (d <= 17) run
+  // the kernel of the small codes, the rest that of the large.
+  const int64_t end = cta0 + n_ctas, split = std::min(std::max(p.small_cta_end, cta0), end);
   if (split > cta0) {
     G.cta0 = cta0;
-    greedy_batch_kernel<true><<<(unsigned)(split - cta0), kGreedyWarps * 32, 0, stream>>>(G);
+    greedy_batch_kernel<greedy::kSmallWarps>
+        <<<(unsigned)(split - cta0), greedy::kSmallWarps * 32, p.greedy_smem[0], stream>>>(G);
   }
   if (end > split) {
     G.cta0 = split;
-    greedy_batch_kernel<false><<<(unsigned)(end - split), kGreedyWarps * 32, 0, stream>>>(G);
+    greedy_batch_kernel<greedy::kLargeWarps>
+        <<<(unsigned)(end - split), greedy::kLargeWarps * 32, p.greedy_smem[1], stream>>>(G);
   }
   XZZX_CUDA_TRY(cudaGetLastError());
   return XZZX_OK;
@@ -242,15 +249,22 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
   P.chain_prefix.assign(n_segs + 1, 0);
   size_t ws = 0;
   std::vector<ChunkDev> chunks;
-  // Restarts per greedy warp: the largest count that leaves the whole greedy
-  // launch enough CTAs.
-  int rpw = 1;
-  for (int r = greedy::kMaxRestartsPerWarp; r > 1 && rpw == 1; r >>= 1) {
-    int64_t ctas = 0;
-    for (int j = 0; j < n_segs; ++j)
-      ctas += (int64_t)segs[j].n_shots *
-              greedy::greedy_groups(segs[j].restarts, segs[j].code->d <= greedy::kListMaxD ? r : 1);
-    if (ctas >= greedy::kMinGreedyCtas) rpw = r;
+  // Restarts per greedy warp of the small and of the large distances: the
+  // largest count that leaves each launch enough CTAs.
+  int rpw[2] = {1, 1};
+  bool few[2];
+  for (int big = 0; big < 2; ++big) {
+    auto ctas = [&](int r) {
+      int64_t n = 0;
+      for (int j = 0; j < n_segs; ++j)
+        if (greedy::is_large(segs[j].code->dev) == (big == 1))
+          n += (int64_t)segs[j].n_shots *
+               greedy::greedy_groups(segs[j].restarts, big ? greedy::kLargeWarps : greedy::kSmallWarps, r);
+      return n;
+    };
+    for (int r = greedy::kMaxRestartsPerWarp; r > 1 && rpw[big] == 1; r >>= 1)
+      if (ctas(r) >= greedy::min_ctas(big == 1)) rpw[big] = r;
+    few[big] = 2 * ctas(1) <= greedy::kFewCtas;
   }
   for (int j = 0; j < n_segs; ++j) {
     const xzzx_segment& s = segs[order[j]];
@@ -261,8 +275,11 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
     d.n_shots = s.n_shots;
     d.restarts = s.restarts;
     d.randomised = s.randomised;
-    d.greedy_rpw = s.code->d <= greedy::kListMaxD ? rpw : 1;  // several per warp only with candidate lists
-    d.greedy_groups = greedy::greedy_groups(s.restarts, d.greedy_rpw);
+    const int big = greedy::is_large(d.code);
+    const greedy::Cut cut = greedy::cut_of<greedy::RotGeo>(d.code, s.restarts, rpw[big], few[big]);
+    d.greedy_groups = cut.groups;
+    d.greedy_cols = cut.cols;
+    P.greedy_smem[big] = std::max(P.greedy_smem[big], cut.smem);
     d.Wt_x = s.noise->Wt_x;
     d.Wt_z = s.noise->Wt_z;
     d.syndromes = s.syndromes;
@@ -284,7 +301,7 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
     d.n_live = s.sched->n_live[kLayoutRotated];
     for (int k = 0; k < 4; ++k) d.W[k] = s.sched->noise.W[k];
     P.cta_prefix[j + 1] = P.cta_prefix[j] + (int64_t)s.n_shots * d.greedy_groups;
-    if (s.code->d <= greedy::kListMaxD) P.list_cta_end = P.cta_prefix[j + 1];
+    if (!big) P.small_cta_end = P.cta_prefix[j + 1];
     P.shot_prefix[j + 1] = P.shot_prefix[j] + s.n_shots;
     P.chain_prefix[j + 1] = P.chain_prefix[j] + (int64_t)s.n_shots * s.restarts * 4;
     P.dmax = std::max(P.dmax, s.code->d);
@@ -678,8 +695,8 @@ xzzx_status xzzx_batch_get_info(const xzzx_batch* b, xzzx_batch_info* out) {
   out->n_chunks = (int)b->plan.lpt.size();
   out->n_distances = (int)b->plan.ranges.size();
   out->persistent_grid = std::min(b->grid, std::max((int)b->plan.lpt.size(), 1));
-  // Mode 0: greedy (one launch per side of d = 15 present), the persistent anneal, the decision.
-  out->launches_batched = 2 + (b->plan.list_cta_end > 0 ? 1 : 0) + (b->plan.list_cta_end < b->plan.total_ctas ? 1 : 0);
+  // Mode 0: greedy (one launch for d <= 17, one above, where present), the persistent anneal, the decision.
+  out->launches_batched = 2 + (b->plan.small_cta_end > 0 ? 1 : 0) + (b->plan.small_cta_end < b->plan.total_ctas ? 1 : 0);
   out->n_classes = (int)b->plan.classes.size();
   out->launches_plain = 3 * (int)b->plan.ranges.size();
   out->workspace_bytes = b->plan.workspace_bytes;

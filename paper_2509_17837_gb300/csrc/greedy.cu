@@ -11,21 +11,30 @@ struct GreedyArgs {
   DevCode code;
   PhiloxKeys keys;
   uint64_t shot0;
-  int n_shots, restarts, randomised, groups, rpw;
+  int n_shots, restarts, randomised, groups, cols;
   int32_t Wt_x, Wt_z;
   const uint32_t* syndromes;
   uint32_t* init;
   uint8_t* cbits;
 };
 
-template <class G, bool L>
-__global__ void __launch_bounds__(kWarps * 32, L ? G::kMinCtasLists : 1)
-    greedy_kernel(const __grid_constant__ GreedyArgs A) {
-  __shared__ SharedT<G, L> S;
+template <class G, int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, 32 / kWarps) greedy_kernel(const __grid_constant__ GreedyArgs A) {
+  extern __shared__ __align__(16) uint8_t smem[];
   const int k = blockIdx.x / A.groups;
-  greedy_cta<G, L>(A.code, A.keys, A.shot0 + (uint64_t)k, blockIdx.x % A.groups, A.restarts, A.rpw, A.randomised,
-                   A.Wt_x, A.Wt_z, A.syndromes + (size_t)k * A.code.sw,
-                   A.init + (size_t)k * A.restarts * 2 * A.code.w, A.cbits + (size_t)k * A.restarts, S);
+  greedy_cta<G, kWarps>(A.code, A.keys, A.shot0 + (uint64_t)k, blockIdx.x % A.groups, A.groups, A.cols, A.restarts,
+                        A.randomised, A.Wt_x, A.Wt_z, A.syndromes + (size_t)k * A.code.sw,
+                        A.init + (size_t)k * A.restarts * 2 * A.code.w, A.cbits + (size_t)k * A.restarts, smem);
+}
+
+template <class G, int kWarps>
+xzzx_status launch_g(const GreedyArgs& A, unsigned grid, size_t smem, cudaStream_t stream) {
+  static DeviceOnce once;
+  xzzx_status st = once.run([] { return allow_shared(greedy_kernel<G, kWarps>); });
+  if (st) return st;
+  greedy_kernel<G, kWarps><<<grid, kWarps * 32, smem, stream>>>(A);
+  XZZX_CUDA_TRY(cudaGetLastError());
+  return XZZX_OK;
 }
 
 }  // namespace
@@ -41,13 +50,16 @@ xzzx_status launch_greedy(const xzzx_code* code, const xzzx_noise* noise, uint64
   A.n_shots = n_shots;
   A.restarts = restarts;
   A.randomised = randomised;
-  A.rpw = 1;  // several restarts per warp only with candidate lists (d <= 17)
-  for (int r = kMaxRestartsPerWarp; r > 1 && code->layout != kLayoutPlanar && code->d <= kListMaxD; r >>= 1)
-    if ((int64_t)n_shots * greedy_groups(restarts, r) >= kMinGreedyCtas) {
-      A.rpw = r;
-      break;
-    }
-  A.groups = greedy_groups(restarts, A.rpw);
+  const bool large = is_large(code->dev);
+  const int warps = large ? kLargeWarps : kSmallWarps;
+  int rpw = 1;
+  for (int r = kMaxRestartsPerWarp; r > 1 && rpw == 1; r >>= 1)
+    if ((int64_t)n_shots * greedy_groups(restarts, warps, r) >= min_ctas(large)) rpw = r;
+  const bool few = 2 * (int64_t)n_shots * greedy_groups(restarts, warps, 1) <= kFewCtas;
+  const Cut cut = code->layout == kLayoutPlanar ? cut_of<PlanarGeo>(A.code, restarts, rpw, few)
+                                                : cut_of<RotGeo>(A.code, restarts, rpw, few);
+  A.groups = cut.groups;
+  A.cols = cut.cols;
   A.Wt_x = noise->Wt_x;
   A.Wt_z = noise->Wt_z;
   A.syndromes = syndromes;
@@ -56,13 +68,10 @@ xzzx_status launch_greedy(const xzzx_code* code, const xzzx_noise* noise, uint64
   const uint64_t grid = (uint64_t)n_shots * A.groups;
   if (grid > 0x7FFFFFFFull) return fail(XZZX_EINVAL, "too many shots x restarts for one launch");
   if (code->layout == kLayoutPlanar)
-    greedy_kernel<PlanarGeo, false><<<(unsigned)grid, kWarps * 32, 0, stream>>>(A);
-  else if (code->d <= kListMaxD)
-    greedy_kernel<RotGeo, true><<<(unsigned)grid, kWarps * 32, 0, stream>>>(A);
-  else
-    greedy_kernel<RotGeo, false><<<(unsigned)grid, kWarps * 32, 0, stream>>>(A);
-  XZZX_CUDA_TRY(cudaGetLastError());
-  return XZZX_OK;
+    return large ? launch_g<PlanarGeo, kLargeWarps>(A, (unsigned)grid, cut.smem, stream)
+                 : launch_g<PlanarGeo, kSmallWarps>(A, (unsigned)grid, cut.smem, stream);
+  return large ? launch_g<RotGeo, kLargeWarps>(A, (unsigned)grid, cut.smem, stream)
+               : launch_g<RotGeo, kSmallWarps>(A, (unsigned)grid, cut.smem, stream);
 }
 
 }  // namespace xzzx

@@ -1,13 +1,12 @@
 // Randomised greedy matching (Algs. 5 and 6) on the GPU.
 //
-// One CTA per (shot, group of kWarps*rpw restarts); each warp takes rpw
-// restarts in turn (for d <= 17 rpw = 4, 2 or 1, the most that still leaves
-// the launch several waves of CTAs; 1 above).  The CTA first computes, in
-// shared memory, each face's shortest distance to the open boundary of its
-// decoding graph (w(u,b) of Eq. distance_u_boundary) by Bellman-Ford
-// relaxation, and the defect list of each decoding-graph colour; for d <= 17,
-// also every vertex's candidate list (below).  All of it depends on the shot
-// only, so it serves every restart of the CTA.
+// One CTA per (shot, group of restarts); its warps take the group's restarts in
+// turn.  The CTA first computes, in shared memory, each face's shortest distance
+// to the open boundary of its decoding graph (w(u,b) of Eq.
+// distance_u_boundary) by Bellman-Ford relaxation with the first step of its
+// canonical walk there, and the defect list of each decoding-graph colour.  Then,
+// colour by colour, every vertex's candidate list (below), which serves all the
+// restarts of the CTA.  All of it depends on the shot only.
 //
 // Matching.  All candidate pairs are totally ordered by (w, key, u, v): w the
 // pair weight of Eq. distance_u_v_def_new, key a Philox draw per pair (Alg. 6)
@@ -16,42 +15,52 @@
 // the same matching as repeatedly matching every pair that is the best
 // remaining pair of both its ends ("locally dominant" pairs), which is what
 // the warp does, round by round, in parallel over vertices.  A vertex's best
-// free partner is found from its candidate list when the colour has at most
-// 64 vertices: the other vertices sorted by (w, index), so the first free
-// entry has the lowest weight and, among equal weights, the lowest (u, v);
-// with random keys only the free entries tied with it at that weight are
-// compared further.  Larger colours scan all candidates.
+// free partner is found from its candidate list: the other vertices sorted by
+// (w, index), so the first free entry has the lowest weight and, among equal
+// weights, the lowest (u, v); with random keys only the free entries tied with
+// it at that weight are compared further.  Colours with more vertices than the
+// CTA has list space for scan all candidates.
 //
 // Paths.  Every kept pair is joined by a canonical shortest path (a Z step
 // toward the target whenever one is needed and possible, else an X step; to
 // the boundary, the first of Z(+1,+1), Z(-1,-1), X(+1,-1), X(-1,+1) that lowers
-// the boundary distance by its weight), added modulo two into the warp's
+// the boundary distance by its weight), added modulo two into the restart's
 // configuration.  A walk that could not complete (never expected on a valid
 // code) sets bit 7 of cbits and raises XZZX_DEVERR_GREEDY_WALK in the code's
 // error area.
+//
+// What bounds it: dependent shared-memory loads of a few active lanes (walking
+// lists, drawing tied keys), so occupancy; hence shared memory is carved to the
+// code's own size, and one list buffer serves the two colours of a large code in
+// turn.  Against lists for rotated d <= 17 only and a fixed carve for d = 31
+// (identical references): 76 shots x 256 restarts at d = 31, p = 0.24 13.6 -> 2.85
+// ms; 4000 x 100 planar d = 9 7.59 -> 2.54 ms; 100 x 100 planar d = 21 3.82 ->
+// 1.24 ms; 4000 x 64 at d = 11 1.94 -> 1.77 ms; one shot x 32 at d = 25 0.58 -> 0.13
+// ms.
 #pragma once
 
-#include <type_traits>
-
+#include "anneal_core.cuh"
 #include "internal.h"
 #include "philox.cuh"
 
 namespace xzzx {
 namespace greedy {
 
-constexpr int kWarps = 4;
-// A launch with candidate lists takes the largest restarts-per-warp count (4,
-// 2 or 1) that still gives it this many CTAs (several waves on a 152-SM GPU):
-// large launches then share each CTA's setup across more restarts, small ones
-// keep their CTAs.  Without lists (d > 17) a warp takes one restart: the scan
-// dominates there, and longer CTAs only lengthen the launch's tail.
-constexpr int64_t kMinGreedyCtas = 4096;
-constexpr int kMaxRestartsPerWarp = 4;
-
+// Warps of a CTA: 8 for codes of up to 150 faces per decoding-graph colour
+// (rotated d <= 17, planar d <= 11), 16 above, where the lists take long to build
+// and most of the shared memory.
+constexpr int kSmallWarps = 8, kLargeWarps = 16, kSmallFaces = 150;
+// A launch of no more CTAs than this gives each restart two warps, one per colour.
+constexpr int64_t kFewCtas = 152;
+// A launch takes the largest restarts-per-warp count (8, 4, 2 or 1) that still
+// gives it enough CTAs: large launches then share each CTA's setup across more
+// restarts, small ones keep their CTAs.  Lists of small codes cost little next
+// to a restart, and several waves of CTAs fill the launch's tail; the lists of
+// larger codes cost about as much as one restart, so two CTAs per SM are enough.
+constexpr int kMaxRestartsPerWarp = 8;
+inline int64_t min_ctas(bool large) { return large ? 304 : 2048; }
 // CTAs of a shot's restarts at rpw restarts per warp.
-__host__ __device__ inline int greedy_groups(int restarts, int rpw) {
-  return (restarts + kWarps * rpw - 1) / (kWarps * rpw);
-}
+inline int greedy_groups(int restarts, int warps, int rpw) { return (restarts + warps * rpw - 1) / (warps * rpw); }
 // Reference modes: greedy matching with lexicographic ties (Alg. 5), with
 // random ties (Alg. 6), or every defect joined to its nearer boundary.
 constexpr int kInitGreedy = 0, kInitGreedyRandom = 1, kInitBoundary = 2;
@@ -61,14 +70,6 @@ constexpr int32_t kInf = 0x3FFFFFFF;
 // (r, c) = r*d + c.  The four edges of a face in walking order: Z(+1,+1),
 // Z(-1,-1), X(+1,-1), X(-1,+1), crossing the qubit (max a, max b).
 struct RotGeo {
-  static constexpr bool kSortedLists = true;
-  // Resident CTAs per SM the kernel with candidate lists is register-bounded
-  // for (64 registers; its shared memory allows 7).
-  static constexpr int kMinCtasLists = 8;
-  static constexpr int kMaxFaces = kMaxD * kMaxD - 1;
-  static constexpr int kMaxAt = (kMaxD + 1) * (kMaxD + 1);
-  static constexpr int kMaxWords = (kMaxD * kMaxD + 31) / 32;
-  __device__ static int at_size(int d) { return (d + 1) * (d + 1); }
   __device__ static int face(const int16_t* at, int d, int a, int b) {
     if (a < -1 || a > d - 1 || b < -1 || b > d - 1) return -1;
     return at[(a + 1) * (d + 1) + (b + 1)];
@@ -80,22 +81,15 @@ struct RotGeo {
     qr = max(a, na);
     qc = max(b, nb);
   }
-  // Eq. distance_u_v_internal in rotated coordinates.
-  __device__ static int32_t w_int(int au, int bu, int av, int bv, int32_t Wt_x, int32_t Wt_z) {
-    return Wt_z * (abs((au + bu) - (av + bv)) >> 1) + Wt_x * (abs((au - bu) - (av - bv)) >> 1);
-  }
+  // Coordinates that a Z step (edge 0: +2) and an X step (edge 2: +2) move.
+  __device__ static int zpos(int a, int b) { return a + b; }
+  __device__ static int xpos(int a, int b) { return a - b; }
 };
 
 // Geometry of the planar layout: faces (i, j), i + j odd, of the (2d-1)^2
 // grid; qubits on the sites with r + c even.  Edges in walking order: Z right
 // and Z left (crossing (i, j+-1)), X down and X up (crossing (i+-1, j)).
 struct PlanarGeo {
-  static constexpr bool kSortedLists = false;
-  static constexpr int kMinCtasLists = 1;
-  static constexpr int kMaxFaces = 2 * kMaxD * (kMaxD - 1);
-  static constexpr int kMaxAt = (2 * kMaxD - 1) * (2 * kMaxD - 1);
-  static constexpr int kMaxWords = (kMaxD * kMaxD + (kMaxD - 1) * (kMaxD - 1) + 31) / 32;
-  __device__ static int at_size(int d) { return (2 * d - 1) * (2 * d - 1); }
   __device__ static int face(const int16_t* at, int d, int a, int b) {
     const int g = 2 * d - 1;
     if (a < 0 || a >= g || b < 0 || b >= g) return -1;
@@ -114,61 +108,77 @@ struct PlanarGeo {
     qr = a + di;
     qc = b + dj;
   }
-  // Eq. distance_u_v_internal: a Z step moves j by 2, an X step moves i by 2.
-  __device__ static int32_t w_int(int au, int bu, int av, int bv, int32_t Wt_x, int32_t Wt_z) {
-    return Wt_z * (abs(bu - bv) >> 1) + Wt_x * (abs(au - av) >> 1);
-  }
+  __device__ static int zpos(int, int b) { return b; }
+  __device__ static int xpos(int a, int) { return a; }
 };
 
-// Sorted candidate lists of one CTA (rotated codes): for each colour with at
-// most kListMax vertices and each vertex x, the other vertices y in
-// increasing (w(x, y), y), one byte each: y, plus 0x80 when w(x, y) equals the
-// previous entry's weight.  cur: each warp's first possibly-free entry.
-constexpr int kListMax = 64;
-struct CandidateLists {
-  uint8_t l[2][kListMax][kListMax];
-  uint8_t cur[kWarps][kListMax];
-  int usable[2];
+// Vertices a colour's candidate lists have room for: half of the colour's faces
+// and a little (defect density stays below one half under independent noise),
+// at least 64 and at most 256 (list entries are bytes).  None for colours of
+// more than 800 faces (planar d >= 29), which mostly hold more than 256 defects:
+// the lists' memory would only lower the occupancy of the scan that then runs
+// (d = 31, p = 0.12: 4.96 against 4.26 ms).
+__host__ __device__ inline int list_room(int faces_per_colour) {
+  const int n = (faces_per_colour * 35 / 64 + 31) / 32 * 32;
+  return faces_per_colour > 800 ? 0 : n < 64 ? 64 : n > 256 ? 256 : n;
+}
+
+inline bool is_large(const DevCode& C) { return C.ns / 2 > kSmallFaces && list_room(C.ns / 2) > 0; }
+
+// Shared memory of a CTA: offsets in bytes; cols: colours whose lists are held at
+// once (1 or 2), each in a buffer of list_bytes and tie_bytes.
+struct Carve {
+  int wb, nb, fa, fb, step, syn, defects, pq, wd, lists, ties, cur, pairs, free_, cfg, misc, total;
+  int room, list_stride, list_bytes, tie_stride, tie_bytes, vmax;
 };
-struct NoLists {};
+__host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int cols, int restarts_per_cta) {
+  Carve c;
+  int o = 0;
+  auto take = [&](int bytes) {
+    const int at = o;
+    o = (o + bytes + 15) & ~15;
+    return at;
+  };
+  const int half = ns / 2;      // faces per colour
+  c.vmax = (half + 2 + 31) & ~31;  // vertices per colour, the virtual one too
+  c.room = list_room(half);
+  c.list_stride = c.room + 4;   // an odd number of words: lanes on different lists hit different banks
+  c.tie_stride = c.room / 32 + 1;
+  c.wb = take(4 * ns);
+  c.nb = take(4 * 2 * ns);
+  c.fa = take(ns);
+  c.fb = take(ns);
+  c.step = take(ns);
+  c.syn = take(4 * sw);
+  c.defects = take(2 * 2 * c.vmax);
+  c.pq = take(2 * 4 * c.vmax);
+  c.wd = take(2 * 4 * c.vmax);
+  // best and partner of each warp: beside the lists, or in their place when
+  // the colour is scanned.
+  const int scan = c.vmax > c.room ? 4 * warps * c.vmax : 0, list = c.room * c.list_stride;
+  c.list_bytes = ((list > scan ? list : scan) + 15) & ~15;
+  c.tie_bytes = (4 * c.room * c.tie_stride + 15) & ~15;
+  c.lists = take(cols * c.list_bytes);
+  c.ties = take(cols * c.tie_bytes);
+  c.cur = take(warps * c.room);
+  c.pairs = take(4 * warps * c.room);
+  c.free_ = take(4 * warps * (c.vmax / 32));
+  c.cfg = take(4 * restarts_per_cta * 2 * w);
+  c.misc = take(4 * (4 + restarts_per_cta));  // n_def[2], usable[2], walk_error[]
+  c.total = o;
+  return c;
+}
 
-// Largest distance whose greedy launches carry candidate lists.  At d = 17
-// colours still fit kListMax vertices for p up to about 0.2 (2-3x faster
-// references); past it most colours hold more, and the lists' shared memory
-// would only lower the occupancy of the scan that runs.
-constexpr int kListMaxD = 17;
+constexpr int kOut = -1, kNone = -2;
 
-template <class G>
-struct SharedBase {
-  int16_t fa[G::kMaxFaces], fb[G::kMaxFaces];
-  int16_t at[G::kMaxAt];
-  int32_t wb[G::kMaxFaces];
-  int16_t defects[2][G::kMaxFaces / 2];
-  int n_def[2];
-  uint32_t syn[(G::kMaxFaces + 31) / 32];
-  int16_t best[kWarps][G::kMaxFaces / 2 + 1];
-  int16_t partner[kWarps][G::kMaxFaces / 2 + 1];
-  uint32_t cfg[kWarps][2 * G::kMaxWords];
-  int walk_error[kWarps];
-};
-
-// A CTA's shared state, with candidate lists when L (rotated codes only).
-template <class G, bool L>
-struct SharedT : SharedBase<G> {
-  static constexpr bool kLists = G::kSortedLists && L;
-  typename std::conditional<kLists, CandidateLists, NoLists>::type lists;
-};
-
+// A CTA's view of its shot.
 template <class G>
 struct Ctx {
-  const SharedBase<G>& S;
-  int d, w;
-  int32_t Wt_x, Wt_z;
-  uint32_t* err;  // the code's device error area
-  int nq;
-  __device__ int face(int a, int b) const { return G::face(S.at, d, a, b); }
-  __device__ int qubit(int r, int c) const { return G::qubit(d, r, c); }
-  __device__ int32_t w_int(int u, int v) const { return G::w_int(S.fa[u], S.fb[u], S.fa[v], S.fb[v], Wt_x, Wt_z); }
+  const int16_t* nb;    // [4][ns]: the face across edge e of a face; kOut: a boundary edge; kNone: no qubit there
+  const int8_t *fa, *fb;
+  const uint8_t* step;  // of a face: first edge of its walk to the boundary; 0xFF: none
+  int d, w, nq, ns;
+  uint32_t* err;        // the code's device error area
 };
 
 template <class G>
@@ -177,467 +187,504 @@ __device__ __forceinline__ void toggle(const Ctx<G>& X, uint32_t* cfg, int q, bo
   atomicXor(&cfg[(z_step ? X.w : 0) + (q >> 5)], 1u << (q & 31));
 }
 
+// Toggles the qubit that edge e of face f crosses.
+template <class G>
+__device__ __forceinline__ void cross(const Ctx<G>& X, int f, int e, uint32_t* cfg) {
+  int na, nb, qr, qc;
+  G::step(X.fa[f], X.fb[f], e, na, nb, qr, qc);
+  toggle(X, cfg, G::qubit(X.d, qr, qc), e < 2);
+}
+
 // Canonical internal walk: a Z step toward v whenever one is still needed and
 // both the next face and the crossed qubit exist, else an X step.
 template <class G>
 __device__ bool walk_internal(const Ctx<G>& X, int u, int v, uint32_t* cfg) {
-  int a = X.S.fa[u], b = X.S.fb[u];
-  const int ta = X.S.fa[v], tb = X.S.fb[v];
-  for (int guard = 0; guard < 8 * X.d * X.d + 8; ++guard) {
-    if (a == ta && b == tb) return true;
-    bool moved = false;
-    for (int e = 0; e < 4 && !moved; ++e) {
-      int na, nb, qr, qc;
-      G::step(a, b, e, na, nb, qr, qc);
-      const bool z_step = e < 2;
-      // the step must lower the remaining distance of its own kind
-      const int32_t before = G::w_int(a, b, ta, tb, z_step ? 0 : 1, z_step ? 1 : 0);
-      const int32_t after = G::w_int(na, nb, ta, tb, z_step ? 0 : 1, z_step ? 1 : 0);
-      if (after != before - 1) continue;
-      const int q = X.qubit(qr, qc);
-      if (X.face(na, nb) < 0 || q < 0) continue;
-      toggle(X, cfg, q, z_step);
-      a = na;
-      b = nb;
-      moved = true;
+  int nz = G::zpos(X.fa[v], X.fb[v]) - G::zpos(X.fa[u], X.fb[u]);  // what is left, two a step
+  int nx = G::xpos(X.fa[v], X.fb[v]) - G::xpos(X.fa[u], X.fb[u]);
+  int cur = u;
+  while (nz | nx) {
+    int e = nz < 0 ? 1 : 0, next = nz ? X.nb[e * X.ns + cur] : kNone;
+    if (next < 0 && nx) {
+      e = nx < 0 ? 3 : 2;
+      next = X.nb[e * X.ns + cur];
     }
-    if (!moved) return false;
+    if (next < 0) return false;
+    cross(X, cur, e, cfg);
+    const int done = (e & 1) ? -2 : 2;
+    if (e < 2) nz -= done;
+    else nx -= done;
+    cur = next;
   }
-  return false;
+  return true;
 }
 
-// Walk to the open boundary: at each face the first edge, in walking order,
-// that lowers the boundary distance by exactly its own weight.
+// Walk to the open boundary: at each face the edge that the setup chose.
 template <class G>
 __device__ bool walk_boundary(const Ctx<G>& X, int u, uint32_t* cfg) {
   int cur = u;
-  for (int guard = 0; guard < 8 * X.d * X.d + 8; ++guard) {
-    const int a = X.S.fa[cur], b = X.S.fb[cur];
-    const int32_t here = X.S.wb[cur];
-    bool moved = false;
-    for (int e = 0; e < 4; ++e) {
-      int na, nb, qr, qc;
-      G::step(a, b, e, na, nb, qr, qc);
-      const int q = X.qubit(qr, qc);
-      if (q < 0) continue;
-      const bool z_step = e < 2;
-      const int32_t w = z_step ? X.Wt_z : X.Wt_x;
-      const int nf = X.face(na, nb);
-      if (nf < 0) {
-        if (w == here) {
-          toggle(X, cfg, q, z_step);
-          return true;
-        }
-      } else if (X.S.wb[nf] + w == here) {
-        toggle(X, cfg, q, z_step);
-        cur = nf;
-        moved = true;
-        break;
-      }
-    }
-    if (!moved) return false;
+  for (int guard = 0; guard < X.nq; ++guard) {
+    const int e = X.step[cur];
+    if (e == 0xFF) return false;
+    cross(X, cur, e, cfg);
+    cur = X.nb[e * X.ns + cur];
+    if (cur < 0) return true;
   }
   return false;
 }
 
-// Pair weight of vertices x != y of a colour with nd defects (vertex nd is the
-// virtual boundary vertex).
-template <class G>
-__device__ __forceinline__ int32_t pair_weight(const Ctx<G>& X, const int16_t* D, int nd, int x, int y) {
-  if (x == nd) return X.S.wb[D[y]];
-  if (y == nd) return X.S.wb[D[x]];
-  return min(X.w_int(D[x], D[y]), X.S.wb[D[x]] + X.S.wb[D[y]]);
+// One colour of a shot: its defects as positions and boundary distances.
+struct Vertices {
+  const int16_t* D;   // face of vertex x < nd
+  const int32_t* pq;  // zpos + 256 | (xpos + 256) << 16
+  const int32_t* wd;  // w(u, b)
+  int nd, nv;         // vertex nd (when nd is odd) is the virtual boundary vertex
+};
+
+__device__ __forceinline__ int32_t internal_weight(int32_t pu, int32_t pv, int32_t Wt_x, int32_t Wt_z) {
+  return Wt_z * (abs((pu & 0xFFFF) - (pv & 0xFFFF)) >> 1) + Wt_x * (abs((pu >> 16) - (pv >> 16)) >> 1);
+}
+// Pair weight of vertices x != y.
+__device__ __forceinline__ int32_t pair_weight(const Vertices& V, int x, int y, int32_t Wt_x, int32_t Wt_z) {
+  if (x == V.nd) return V.wd[y];
+  if (y == V.nd) return V.wd[x];
+  return min(internal_weight(V.pq[x], V.pq[y], Wt_x, Wt_z), V.wd[x] + V.wd[y]);
 }
 
-// Keep the smaller (keep_min) or larger of v and the value of lane ^ j.
-__device__ __forceinline__ uint32_t bitonic_step(uint32_t v, int j, bool keep_min) {
-  const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, v, j);
-  return keep_min ? min(v, o) : max(v, o);
-}
-
-// Ascending bitonic sort across the warp of the values at positions lane (a)
-// and, when N64, lane + 32 (b).
-template <bool N64>
-__device__ __forceinline__ void warp_sort(uint32_t& a, uint32_t& b, int lane) {
+// Ascending bitonic sort across the warp of 32 NK keys, element h * 32 + lane
+// in key[h].
+template <int NK>
+__device__ __forceinline__ void warp_sort(uint32_t (&key)[NK], int lane) {
 #pragma unroll
-  for (int k = 2; k <= (N64 ? 64 : 32); k <<= 1) {
+  for (int k = 2; k <= 32 * NK; k <<= 1) {
 #pragma unroll
     for (int j = k >> 1; j > 0; j >>= 1) {
-      if (j == 32) {
-        const uint32_t lo = min(a, b), hi = max(a, b);
-        a = lo;
-        b = hi;
-        continue;
+      if (j >= 32) {
+#pragma unroll
+        for (int h = 0; h < NK; ++h) {
+          const int o = h ^ (j >> 5);
+          if (o < h) continue;
+          const bool up = ((32 * h) & k) == 0;
+          const uint32_t lo = min(key[h], key[o]), hi = max(key[h], key[o]);
+          key[h] = up ? lo : hi;
+          key[o] = up ? hi : lo;
+        }
+      } else {
+        const bool lower = (lane & j) == 0;
+#pragma unroll
+        for (int h = 0; h < NK; ++h) {
+          const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, key[h], j);
+          const bool up = ((32 * h + lane) & k) == 0;
+          key[h] = lower == up ? min(key[h], o) : max(key[h], o);
+        }
       }
-      const bool lower = (lane & j) == 0;
-      a = bitonic_step(a, j, lower == ((lane & k) == 0));
-      if (N64) b = bitonic_step(b, j, lower == (((lane + 32) & k) == 0));
     }
   }
 }
 
-// Candidate list of vertex x (nv <= kListMax vertices), built by one warp.
-// Returns false if a weight does not fit the 26 bits of the sort key.
-template <class G, bool N64>
-__device__ __forceinline__ bool build_list(const Ctx<G>& X, const int16_t* D, int nd, int nv, int x, uint8_t* out,
-                                           int lane) {
+// Candidate list of vertex x, built by one warp: out[pos] the vertex, bit pos of
+// ties set when its weight equals the previous entry's.  Returns false if a
+// weight does not fit the 24 bits of the sort key.
+template <int NK>
+__device__ __forceinline__ bool build_list(const Vertices& V, int x, int32_t Wt_x, int32_t Wt_z, uint8_t* out,
+                                           uint32_t* ties, int lane) {
   bool fits = true;
-  uint32_t key[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+  uint32_t key[NK];
 #pragma unroll
-  for (int h = 0; h < (N64 ? 2 : 1); ++h) {
+  for (int h = 0; h < NK; ++h) {
     const int y = lane + 32 * h;
-    if (y < nv && y != x) {
-      const int32_t w = pair_weight(X, D, nd, x, y);
-      fits = fits && w >= 0 && w < (1 << 26) - 1;  // keys stay below the 0xFFFFFFFF filler
-      key[h] = ((uint32_t)w << 6) | (uint32_t)y;
+    key[h] = 0xFFFFFFFFu;
+    if (y < V.nv && y != x) {
+      const int32_t w = pair_weight(V, x, y, Wt_x, Wt_z);
+      fits = fits && w >= 0 && w < (1 << 24) - 1;  // keys stay below the 0xFFFFFFFF filler
+      key[h] = ((uint32_t)w << 8) | (uint32_t)y;
     }
   }
-  warp_sort<N64>(key[0], key[1], lane);
-  const uint32_t prev0 = __shfl_up_sync(0xFFFFFFFFu, key[0], 1);
-  const uint32_t last0 = __shfl_sync(0xFFFFFFFFu, key[0], 31);
-  uint32_t prev1 = 0u;
-  if (N64) {
-    const uint32_t up1 = __shfl_up_sync(0xFFFFFFFFu, key[1], 1);
-    prev1 = lane == 0 ? last0 : up1;
-  }
+  warp_sort<NK>(key, lane);
+  uint32_t last = 0xFFFFFFFFu;  // the element before this block's first
 #pragma unroll
-  for (int h = 0; h < (N64 ? 2 : 1); ++h) {
-    const int pos = lane + 32 * h;
-    const uint32_t k = key[h], pk = h ? prev1 : prev0;
-    if (pos < nv - 1) out[pos] = (uint8_t)((k & 63u) | ((pos > 0 && (k >> 6) == (pk >> 6)) ? 0x80u : 0u));
+  for (int h = 0; h < NK; ++h) {
+    uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, key[h], 1);
+    if (lane == 0) prev = last;
+    last = __shfl_sync(0xFFFFFFFFu, key[h], 31);
+    const int pos = 32 * h + lane;
+    const bool on = pos < V.nv - 1;
+    if (on) out[pos] = (uint8_t)(key[h] & 255u);
+    const uint32_t t = __ballot_sync(0xFFFFFFFFu, on && pos > 0 && (key[h] >> 8) == (prev >> 8));
+    if (lane == 0 && 32 * h < V.nv - 1) ties[h] = t;
   }
   return __all_sync(0xFFFFFFFFu, fits);
 }
 
-// The reference of restart i of the CTA's shot, by one warp, after the CTA
-// has set up the boundary distances, defect lists and candidate lists.
-template <class G, bool L>
-__device__ __forceinline__ void greedy_restart(const Ctx<G>& X, const DevCode& C, const PhiloxKeys& K, uint64_t shot,
-                                               int i, int mode, uint32_t* __restrict__ init,
-                                               uint8_t* __restrict__ cbits, SharedT<G, L>& S, int warp, int lane) {
-  const int w = C.w;
-
-  uint32_t* cfg = S.cfg[warp];
-  for (int j = lane; j < 2 * w; j += 32) cfg[j] = 0u;
-  if (lane == 0) S.walk_error[warp] = 0;
-  int16_t* best = S.best[warp];
-  int16_t* partner = S.partner[warp];
-  __syncwarp();
-
-  if (mode == kInitBoundary) {
-    // Each defect joined to the nearer boundary of its decoding graph.
-    for (int colour = 0; colour < 2; ++colour)
-      for (int x = lane; x < S.n_def[colour]; x += 32)
-        if (!walk_boundary(X, S.defects[colour][x], cfg)) S.walk_error[warp] = 1;
-    __syncwarp();
+// The keys of Alg. 6: word 0 of Philox(seed; u | v << 16, restart, shot_lo, 2 |
+// shot_hi << 8), the parts that depend on the shot or the restart taken once.
+struct PairKeys {
+  core::SaDraws dr;
+  __device__ __forceinline__ PairKeys(uint64_t shot, const PhiloxKeys& K) {
+    dr.init((uint32_t)shot, kTagGreedy | ((uint32_t)(shot >> 32) << 8), K);
   }
-  for (int colour = 0; colour < 2 && mode != kInitBoundary; ++colour) {
-    const int nd = S.n_def[colour];
-    const int nv = nd + (nd & 1);  // vertex nd is the virtual boundary vertex when nd is odd
-    const int16_t* D = S.defects[colour];
+  __device__ __forceinline__ void restart(int i, const PhiloxKeys& K) { dr.sweep((uint32_t)i, K); }
+  __device__ __forceinline__ uint32_t key(uint32_t u, uint32_t v, const PhiloxKeys& K) const {
+    return dr.block(u | (v << 16), K).x;
+  }
+};
+
+// Per-warp state of one matching.
+struct Work {
+  int16_t *best, *partner;
+  uint32_t* free_;  // bit x: vertex x is free
+  uint8_t* cur;     // first possibly-free entry of each list
+};
+__device__ __forceinline__ bool is_free(const Work& W, int x) { return (W.free_[x >> 5] >> (x & 31)) & 1u; }
+
+// Greedy matching of one colour for one restart, by one warp: partner[].
+// Returns false if a round could not complete (never expected).
+template <bool LISTED>
+__device__ __forceinline__ bool match(const Vertices& V, const Carve& c, const uint8_t* lists, const uint32_t* ties,
+                                      const Work& W, bool random, const PairKeys& pk, const PhiloxKeys& K, int32_t Wt_x,
+                                      int32_t Wt_z, uint32_t* err, int lane) {
+  const int nd = V.nd, nv = V.nv;
+  bool good = true;
+  for (int x = lane; x < nv; x += 32) {
+    W.partner[x] = -1;
+    W.best[x] = -1;
+    if (LISTED) W.cur[x] = 0;
+  }
+  for (int b = 0; b < nv; b += 32)
+    if (lane == 0) W.free_[b >> 5] = nv - b >= 32 ? 0xFFFFFFFFu : (1u << (nv - b)) - 1u;
+  __syncwarp();
+  int unmatched = nv;
+  while (unmatched > 0) {
+    // A best partner that is still free stays the best (removing other vertices
+    // cannot put one ahead of it), so only vertices whose best was matched in
+    // the last round search again.
     for (int x = lane; x < nv; x += 32) {
-      partner[x] = -1;
-      best[x] = -1;
-    }
-    bool listed = false;
-    if constexpr (SharedT<G, L>::kLists) {
-      listed = nv >= 2 && nv <= kListMax && S.lists.usable[colour];
-      if (listed)
-        for (int x = lane; x < nv; x += 32) S.lists.cur[warp][x] = 0;
-    }
-    __syncwarp();
-    int unmatched = nv;
-    while (unmatched > 0 && listed) {
-      if constexpr (SharedT<G, L>::kLists) {
-        // Each free vertex whose best partner was taken walks its sorted list
-        // from its cursor to the first free entry: the lowest weight among
-        // free vertices, and the lowest (u, v) at that weight.  Keys order
-        // the free entries tied at that weight (Alg. 6).
-        for (int x = lane; x < nv; x += 32) {
-          if (partner[x] >= 0) {
-            best[x] = -1;
-            continue;
-          }
-          const int bx = best[x];
-          if (bx >= 0 && partner[bx] < 0) continue;
-          const uint8_t* Lx = S.lists.l[colour][x];
-          int c = S.lists.cur[warp][x];
-          while (c < nv - 1 && partner[Lx[c] & 63] >= 0) ++c;
-          S.lists.cur[warp][x] = (uint8_t)c;
-          if (c >= nv - 1) {  // no free vertex left for x: impossible with an even count
-            best[x] = -1;
-            S.walk_error[warp] = 1;
-            continue;
-          }
-          int bestv = Lx[c] & 63;
-          if (mode == kInitGreedyRandom) {
-            const uint32_t sx = x == nd ? kBoundary : (uint32_t)D[x];
-            const uint32_t s0 = bestv == nd ? kBoundary : (uint32_t)D[bestv];
-            uint32_t bu = min(sx, s0), bvv = max(sx, s0), bkey = 0;
-            bool bkey_ok = false;
-            const uint32_t c3 = kTagGreedy | ((uint32_t)(shot >> 32) << 8);
-            for (int k = c + 1; k < nv - 1; ++k) {
-              const uint32_t ent = Lx[k];
-              if (!(ent & 0x80u)) break;
-              const int y = (int)(ent & 63u);
-              if (partner[y] >= 0) continue;
-              const uint32_t sy = y == nd ? kBoundary : (uint32_t)D[y];
-              const uint32_t u = min(sx, sy), v = max(sx, sy);
-              if (!bkey_ok) {
-                bkey = philox4x32_10(bu | (bvv << 16), (uint32_t)i, (uint32_t)shot, c3, K).x;
-                bkey_ok = true;
-              }
-              const uint32_t key = philox4x32_10(u | (v << 16), (uint32_t)i, (uint32_t)shot, c3, K).x;
-              if (key < bkey || (key == bkey && (u < bu || (u == bu && v < bvv)))) {
-                bestv = y;
-                bkey = key;
-                bu = u;
-                bvv = v;
-              }
-            }
-          }
-          best[x] = (int16_t)bestv;
-        }
-        __syncwarp();
-        int made = 0;
-        for (int x = lane; x < nv; x += 32) {
-          const int y = best[x];
-          if (y > x && XZZX_CHECK(C.err, y < nv) && best[y] == x) {
-            partner[x] = (int16_t)y;
-            partner[y] = (int16_t)x;
-            made += 2;
-          }
-        }
-        __syncwarp();
-        for (int off = 16; off > 0; off >>= 1) made += __shfl_xor_sync(0xFFFFFFFFu, made, off);
-        if (made == 0) {
-          if (lane == 0) S.walk_error[warp] = 1;
-          break;
-        }
-        unmatched -= made;
+      if (!is_free(W, x)) {
+        W.best[x] = -1;
+        continue;
       }
-    }
-    while (unmatched > 0 && !listed) {
-      // Each free vertex finds its best free partner in the order (w, key, u, v),
-      // in one pass: a candidate's key is drawn only when its weight ties the
-      // best so far.  A best partner that is still free stays the best (removing
-      // other vertices cannot put one ahead of it), so only vertices whose best
-      // was matched in the last round search again.
-      for (int x = lane; x < nv; x += 32) {
-        if (partner[x] >= 0) {
-          best[x] = -1;
+      const int bx = W.best[x];
+      if (bx >= 0 && is_free(W, bx)) continue;
+      const uint32_t sx = x == nd ? kBoundary : (uint32_t)V.D[x];
+      int bestv = -1;
+      if (LISTED) {
+        // From the vertex's cursor to the first free entry: the lowest weight
+        // among free vertices, and the lowest (u, v) at that weight.  Keys
+        // order the free entries tied at that weight (Alg. 6).
+        const uint8_t* Lx = lists + x * c.list_stride;
+        const uint32_t* Tx = ties + x * c.tie_stride;
+        int k = W.cur[x];
+        while (k < nv - 1 && !is_free(W, Lx[k])) ++k;
+        W.cur[x] = (uint8_t)k;
+        if (k >= nv - 1) {  // no free vertex left for x: impossible with an even count
+          W.best[x] = -1;
+          good = false;
           continue;
         }
-        const int bx = best[x];
-        if (bx >= 0 && partner[bx] < 0) continue;
-        const bool xb = x == nd;
-        const int fx = xb ? 0 : D[x];
-        const uint32_t sx = xb ? kBoundary : (uint32_t)fx;
-        int bestv = -1;
-        int32_t bw = kInf;
-        uint32_t bkey = 0, bu = 0, bvv = 0;
-        bool bkey_ok = false;
-        for (int y = 0; y < nv; ++y) {
-          if (y == x || partner[y] >= 0) continue;
-          int32_t wxy;
-          if (xb) wxy = S.wb[D[y]];
-          else if (y == nd) wxy = S.wb[fx];
-          else wxy = min(X.w_int(fx, D[y]), S.wb[fx] + S.wb[D[y]]);
-          if (wxy > bw) continue;
-          const uint32_t sy = (y == nd) ? kBoundary : (uint32_t)D[y];
-          const uint32_t u = min(sx, sy), v = max(sx, sy);
-          if (wxy < bw) {
-            bestv = y;
-            bw = wxy;
-            bu = u;
-            bvv = v;
-            bkey_ok = false;
-            continue;
-          }
-          uint32_t key = 0;
-          if (mode == kInitGreedyRandom) {
-            const uint32_t c3 = kTagGreedy | ((uint32_t)(shot >> 32) << 8);
-            if (!bkey_ok) {
-              bkey = philox4x32_10(bu | (bvv << 16), (uint32_t)i, (uint32_t)shot, c3, K).x;
-              bkey_ok = true;
+        bestv = Lx[k];
+        if (random) {
+          uint32_t bu = 0, bv = 0, bkey = 0;
+          bool drawn = false;
+          for (++k; k < nv - 1 && ((Tx[k >> 5] >> (k & 31)) & 1u); ++k) {
+            const int y = Lx[k];
+            if (!is_free(W, y)) continue;
+            if (!drawn) {
+              const uint32_t s0 = bestv == nd ? kBoundary : (uint32_t)V.D[bestv];
+              bu = min(sx, s0);
+              bv = max(sx, s0);
+              bkey = pk.key(bu, bv, K);
+              drawn = true;
             }
-            key = philox4x32_10(u | (v << 16), (uint32_t)i, (uint32_t)shot, c3, K).x;
-          }
-          if (key < bkey || (key == bkey && (u < bu || (u == bu && v < bvv)))) {
-            bestv = y;
-            bkey = key;
-            bu = u;
-            bvv = v;
+            const uint32_t sy = y == nd ? kBoundary : (uint32_t)V.D[y];
+            const uint32_t u = min(sx, sy), v = max(sx, sy), key = pk.key(u, v, K);
+            if (key < bkey || (key == bkey && (u < bu || (u == bu && v < bv)))) {
+              bestv = y;
+              bkey = key;
+              bu = u;
+              bv = v;
+            }
           }
         }
-        best[x] = (int16_t)bestv;
-      }
-      __syncwarp();
-      // Matching phase: reads only best[], writes only partner[].
-      int made = 0;
-      for (int x = lane; x < nv; x += 32) {
-        const int y = best[x];
-        if (y > x && XZZX_CHECK(C.err, y < nv) && best[y] == x) {
-          partner[x] = (int16_t)y;
-          partner[y] = (int16_t)x;
-          made += 2;
-        }
-      }
-      __syncwarp();
-      for (int off = 16; off > 0; off >>= 1) made += __shfl_xor_sync(0xFFFFFFFFu, made, off);
-      if (made == 0) {  // impossible for a strict total order; keep the warp from spinning
-        if (lane == 0) S.walk_error[warp] = 1;
-        break;
-      }
-      unmatched -= made;
-    }
-    // Join every kept pair.
-    for (int x = lane; x < nv; x += 32) {
-      const int y = partner[x];
-      if (y <= x || x == nd) continue;
-      bool ok;
-      const int fx = D[x];
-      if (y == nd) {
-        ok = walk_boundary(X, fx, cfg);
       } else {
-        const int fy = D[y];
-        if (X.w_int(fx, fy) <= S.wb[fx] + S.wb[fy]) ok = walk_internal(X, fx, fy, cfg);
-        else ok = walk_boundary(X, fx, cfg) && walk_boundary(X, fy, cfg);
+        // One pass over all candidates: a key is drawn only when a weight ties
+        // the best so far.
+        int32_t bw = kInf;
+        uint32_t bkey = 0, bu = 0, bv = 0;
+        bool drawn = false;
+        for (int y = 0; y < nv; ++y) {
+          if (y == x || !is_free(W, y)) continue;
+          const int32_t w = pair_weight(V, x, y, Wt_x, Wt_z);
+          if (w > bw) continue;
+          const uint32_t sy = y == nd ? kBoundary : (uint32_t)V.D[y];
+          const uint32_t u = min(sx, sy), v = max(sx, sy);
+          uint32_t key = 0;
+          if (w == bw) {
+            if (random) {
+              if (!drawn) {
+                bkey = pk.key(bu, bv, K);
+                drawn = true;
+              }
+              key = pk.key(u, v, K);
+            }
+            if (!(key < bkey || (key == bkey && (u < bu || (u == bu && v < bv))))) continue;
+          } else {
+            drawn = false;
+          }
+          bestv = y;
+          bw = w;
+          bkey = key;
+          bu = u;
+          bv = v;
+        }
       }
-      if (!ok) S.walk_error[warp] = 1;
+      W.best[x] = (int16_t)bestv;
     }
     __syncwarp();
+    // Matching phase: reads only best[], writes only partner[].
+    for (int x = lane; x < nv; x += 32) {
+      const int y = W.best[x];
+      if (y > x && XZZX_CHECK(err, y < nv) && W.best[y] == x) {
+        W.partner[x] = (int16_t)y;
+        W.partner[y] = (int16_t)x;
+      }
+    }
+    __syncwarp();
+    int left = 0;
+    for (int b = 0; b < nv; b += 32) {
+      const uint32_t m = __ballot_sync(0xFFFFFFFFu, b + lane < nv && W.partner[b + lane] < 0);
+      if (lane == 0) W.free_[b >> 5] = m;
+      left += __popc(m);
+    }
+    __syncwarp();
+    if (left == unmatched) {  // impossible for a strict total order; keep the warp from spinning
+      good = false;
+      break;
+    }
+    unmatched = left;
   }
-
-  // Output R_i and its commutation bits with L_Z (bit 0) and L_X (bit 1).
-  uint32_t* out = init + (size_t)i * 2 * w;
-  const uint32_t* LX = C.logical;
-  const uint32_t* LZ = C.logical + 2 * w;
-  int par_z = 0, par_x = 0;
-  for (int j = lane; j < w; j += 32) {
-    const uint32_t ex = cfg[j], ez = cfg[w + j];
-    out[j] = ex;
-    out[w + j] = ez;
-    par_z ^= __popc((ex & LZ[w + j]) ^ (ez & LZ[j])) & 1;
-    par_x ^= __popc((ex & LX[w + j]) ^ (ez & LX[j])) & 1;
-  }
-  for (int off = 16; off > 0; off >>= 1) {
-    par_z ^= __shfl_xor_sync(0xFFFFFFFFu, par_z, off);
-    par_x ^= __shfl_xor_sync(0xFFFFFFFFu, par_x, off);
-  }
-  if (lane == 0) {
-    // A walk that could not complete is recorded in the code's error area
-    // (XZZX_DEVERR_GREEDY_WALK) and in bit 7 of the restart's class byte.
-    const bool bad = S.walk_error[warp] != 0 || (i == 0 && injected(C.err, XZZX_DEVERR_GREEDY_WALK));
-    if (bad) raise_device_error(C.err, XZZX_DEVERR_GREEDY_WALK);
-    cbits[i] = (uint8_t)(par_z | (par_x << 1) | (bad ? 0x80 : 0));
-  }
+  return good;
 }
 
-// One CTA: references of restarts [group*kWarps*rpw, (group+1)*kWarps*rpw)
-// of one shot, each warp taking rpw of them in turn, so the CTA's setup serves
-// kWarps*rpw restarts.  syn: the shot's syndrome words; init / cbits: the
-// shot's rows (restarts x 2w words, restarts bytes).
-template <class G, bool L>
-__device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K, uint64_t shot, int group, int restarts,
-                                           int rpw, int mode, int32_t Wt_x, int32_t Wt_z, const uint32_t* __restrict__ syn,
-                                           uint32_t* __restrict__ init, uint8_t* __restrict__ cbits, SharedT<G, L>& S) {
+// One CTA: references of restarts [group * restarts / groups, (group + 1) *
+// restarts / groups) of one shot.  syn: the shot's syndrome words; init / cbits:
+// the shot's rows (restarts x 2w words, restarts bytes).  smem: carve().total
+// bytes for at least that many restarts.
+template <class G, int kWarps>
+__device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K, uint64_t shot, int group, int groups,
+                                           int cols, int restarts, int mode, int32_t Wt_x, int32_t Wt_z,
+                                           const uint32_t* __restrict__ syn, uint32_t* __restrict__ init,
+                                           uint8_t* __restrict__ cbits, uint8_t* smem) {
   const int d = C.d, ns = C.ns, w = C.w;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int lo = (int)((int64_t)group * restarts / groups), hi = (int)((int64_t)(group + 1) * restarts / groups);
+  const Carve c = carve(ns, C.sw, w, kWarps, cols, hi - lo);
+  int32_t* wb = reinterpret_cast<int32_t*>(smem + c.wb);
+  int16_t* nb = reinterpret_cast<int16_t*>(smem + c.nb);            // [4][ns]
+  int8_t* fa = reinterpret_cast<int8_t*>(smem + c.fa);
+  int8_t* fb = reinterpret_cast<int8_t*>(smem + c.fb);
+  uint8_t* step = smem + c.step;
+  uint32_t* s_syn = reinterpret_cast<uint32_t*>(smem + c.syn);
+  int16_t* defects = reinterpret_cast<int16_t*>(smem + c.defects);  // [2][vmax]
+  int32_t* pq = reinterpret_cast<int32_t*>(smem + c.pq);            // [2][vmax]
+  int32_t* wd = reinterpret_cast<int32_t*>(smem + c.wd);            // [2][vmax]
+  uint32_t* cfgs = reinterpret_cast<uint32_t*>(smem + c.cfg);       // [hi - lo][2w]
+  int* n_def = reinterpret_cast<int*>(smem + c.misc);               // [2]
+  int* usable = n_def + 2;                                          // [2]
+  int* walk_error = n_def + 4;                                      // [hi - lo]
+  Work W;
+  W.free_ = reinterpret_cast<uint32_t*>(smem + c.free_) + warp * (c.vmax / 32);
+  W.cur = smem + c.cur + warp * c.room;
 
+  // Faces, their neighbours, and distances over the boundary edges alone.
   for (int f = tid; f < ns; f += blockDim.x) {
-    S.fa[f] = C.face_a[f];
-    S.fb[f] = C.face_b[f];
-  }
-  for (int j = tid; j < G::at_size(d); j += blockDim.x) S.at[j] = C.face_at[j];
-  for (int j = tid; j < C.sw; j += blockDim.x) S.syn[j] = syn[j];
-  if constexpr (SharedT<G, L>::kLists) {
-    if (tid < 2) S.lists.usable[tid] = 1;
-  }
-  __syncthreads();
-  Ctx<G> X{S, d, w, Wt_x, Wt_z, C.err, C.nq};
-
-  // Boundary distances: start from the boundary edges, relax until stable.
-  for (int f = tid; f < ns; f += blockDim.x) {
-    const int a = S.fa[f], b = S.fb[f];
+    const int a = C.face_a[f], b = C.face_b[f];
+    fa[f] = (int8_t)a;
+    fb[f] = (int8_t)b;
+    step[f] = C.face_c2[f];  // until the defects are listed
     int32_t best = kInf;
     for (int e = 0; e < 4; ++e) {
-      int na, nb, qr, qc;
-      G::step(a, b, e, na, nb, qr, qc);
-      if (X.qubit(qr, qc) < 0 || X.face(na, nb) >= 0) continue;
-      best = min(best, e < 2 ? Wt_z : Wt_x);
+      int na, nb_, qr, qc;
+      G::step(a, b, e, na, nb_, qr, qc);
+      int to = kNone;
+      if (G::qubit(d, qr, qc) >= 0) {
+        to = G::face(C.face_at, d, na, nb_);
+        if (to < 0) {
+          to = kOut;
+          best = min(best, e < 2 ? Wt_z : Wt_x);
+        }
+      }
+      nb[e * ns + f] = (int16_t)to;
     }
-    S.wb[f] = best;
+    wb[f] = best;
   }
+  for (int j = tid; j < C.sw; j += blockDim.x) s_syn[j] = syn[j];
+  for (int j = tid; j < (hi - lo) * 2 * w; j += blockDim.x) cfgs[j] = 0u;
+  for (int j = tid; j < hi - lo; j += blockDim.x) walk_error[j] = 0;
   __syncthreads();
+  Ctx<G> X{nb, fa, fb, step, d, w, C.nq, ns, C.err};
+
+  // Defect lists of both colours, in stabilizer-index order, a warp each.
+  if (warp < 2) {
+    int cnt = 0;
+    for (int base = 0; base < ns; base += 32) {
+      const int f = base + lane;
+      const bool on = f < ns && ((s_syn[f >> 5] >> (f & 31)) & 1) && step[f] == warp;
+      const uint32_t m = __ballot_sync(0xFFFFFFFFu, on);
+      const int slot = cnt + __popc(m & ((1u << lane) - 1));
+      if (on && XZZX_CHECK(C.err, slot < c.vmax)) defects[warp * c.vmax + slot] = (int16_t)f;
+      cnt += __popc(m);
+    }
+    if (lane == 0) n_def[warp] = cnt;
+  }
+  // Boundary distances: relax until stable.
   for (int iter = 0; iter < ns + 1; ++iter) {
     int changed = 0;
     for (int f = tid; f < ns; f += blockDim.x) {
-      const int a = S.fa[f], b = S.fb[f];
-      int32_t cur = S.wb[f];
+      const int32_t was = wb[f];
+      int32_t cur = was;
+#pragma unroll
       for (int e = 0; e < 4; ++e) {
-        int na, nb, qr, qc;
-        G::step(a, b, e, na, nb, qr, qc);
-        if (X.qubit(qr, qc) < 0) continue;
-        const int nf = X.face(na, nb);
-        if (nf < 0) continue;
-        const int32_t cand = S.wb[nf] + (e < 2 ? Wt_z : Wt_x);
-        if (cand < cur) {
-          cur = cand;
-          changed = 1;
-        }
+        const int nf = nb[e * ns + f];
+        if (nf >= 0) cur = min(cur, wb[nf] + (e < 2 ? Wt_z : Wt_x));
       }
-      S.wb[f] = cur;
+      wb[f] = cur;
+      changed |= cur != was;
     }
     if (!__syncthreads_or(changed)) break;
   }
-
-  // Defect lists of both colours, in stabilizer-index order.
-  if (warp == 0) {
-    int cnt[2] = {0, 0};
-    for (int base = 0; base < ns; base += 32) {
-      const int f = base + lane;
-      const bool on = f < ns && ((S.syn[f >> 5] >> (f & 31)) & 1);
-      const int c2 = f < ns ? C.face_c2[f] : 0;
-      for (int c = 0; c < 2; ++c) {
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, on && c2 == c);
-        const int slot = cnt[c] + __popc(m & ((1u << lane) - 1));
-        if (on && c2 == c && XZZX_CHECK(C.err, slot < G::kMaxFaces / 2)) S.defects[c][slot] = (int16_t)f;
-        cnt[c] += __popc(m);
-      }
+  // The first edge, in walking order, that lowers the distance by its own weight.
+  for (int f = tid; f < ns; f += blockDim.x) {
+    int st = 0xFF;
+#pragma unroll
+    for (int e = 3; e >= 0; --e) {
+      const int nf = nb[e * ns + f];
+      const int32_t we = e < 2 ? Wt_z : Wt_x;
+      if (nf == kOut ? we == wb[f] : nf >= 0 && wb[nf] + we == wb[f]) st = e;
     }
-    if (lane == 0) {
-      S.n_def[0] = cnt[0];
-      S.n_def[1] = cnt[1];
-    }
+    step[f] = (uint8_t)st;
   }
   __syncthreads();
-  if constexpr (SharedT<G, L>::kLists) {
-    // Candidate lists of both colours, every warp of the CTA building some.
-    if (mode != kInitBoundary) {
+
+  auto vertices = [&](int colour) {
+    Vertices V;
+    V.D = defects + colour * c.vmax;
+    V.pq = pq + colour * c.vmax;
+    V.wd = wd + colour * c.vmax;
+    V.nd = n_def[colour];
+    V.nv = V.nd + (V.nd & 1);
+    return V;
+  };
+  if (mode == kInitBoundary) {
+    // Each defect joined to the nearer boundary of its decoding graph.
+    for (int i = lo + warp; i < hi; i += kWarps)
       for (int colour = 0; colour < 2; ++colour) {
-        const int nd = S.n_def[colour], nv = nd + (nd & 1);
-        if (nv < 2 || nv > kListMax) continue;
-        bool fits = true;
-        for (int x = warp; x < nv; x += kWarps)
-          fits = (nv > 32 ? build_list<G, true>(X, S.defects[colour], nd, nv, x, S.lists.l[colour][x], lane)
-                          : build_list<G, false>(X, S.defects[colour], nd, nv, x, S.lists.l[colour][x], lane)) && fits;
-        if (lane == 0 && !fits) S.lists.usable[colour] = 0;
+        const Vertices V = vertices(colour);
+        for (int x = lane; x < V.nd; x += 32)
+          if (!walk_boundary(X, V.D[x], cfgs + (i - lo) * 2 * w)) walk_error[i - lo] = 1;
       }
-    }
+    __syncthreads();
+  } else {
+    for (int colour = 0; colour < 2; ++colour)
+      for (int x = tid; x < n_def[colour]; x += blockDim.x) {
+        const int f = defects[colour * c.vmax + x];
+        pq[colour * c.vmax + x] = (G::zpos(fa[f], fb[f]) + 256) | ((G::xpos(fa[f], fb[f]) + 256) << 16);
+        wd[colour * c.vmax + x] = wb[f];
+      }
+    if (tid < 2) usable[tid] = n_def[tid] + (n_def[tid] & 1) <= c.room;
     __syncthreads();
   }
-  if constexpr (SharedT<G, L>::kLists) {
-    for (int r = 0; r < rpw; ++r) {
-      const int i = (group * rpw + r) * kWarps + warp;
-      if (i >= restarts) break;
-      __syncwarp();  // the warp's previous reference is written out
-      greedy_restart<G, L>(X, C, K, shot, i, mode, init, cbits, S, warp, lane);
+  PairKeys pk(shot, K);
+  for (int first = 0; first < 2 && mode != kInitBoundary; first += cols) {
+    for (int slot = 0; slot < cols; ++slot) {  // candidate lists, every warp of the CTA building some
+      const Vertices V = vertices(first + slot);
+      if (V.nv > c.room) continue;
+      bool fits = true;
+      for (int x = warp; x < V.nv; x += kWarps) {
+        uint8_t* Lx = smem + c.lists + slot * c.list_bytes + x * c.list_stride;
+        uint32_t* Tx = reinterpret_cast<uint32_t*>(smem + c.ties + slot * c.tie_bytes) + x * c.tie_stride;
+        fits = (V.nv <= 32   ? build_list<1>(V, x, Wt_x, Wt_z, Lx, Tx, lane)
+                : V.nv <= 64 ? build_list<2>(V, x, Wt_x, Wt_z, Lx, Tx, lane)
+                : V.nv <= 128 ? build_list<4>(V, x, Wt_x, Wt_z, Lx, Tx, lane)
+                              : build_list<8>(V, x, Wt_x, Wt_z, Lx, Tx, lane)) && fits;
+      }
+      if (lane == 0 && !fits) usable[first + slot] = 0;
     }
-  } else {  // one restart per warp (rpw is 1 without lists)
-    const int i = group * kWarps + warp;
-    if (i < restarts) greedy_restart<G, L>(X, C, K, shot, i, mode, init, cbits, S, warp, lane);
+    __syncthreads();
+    for (int it = warp; it < cols * (hi - lo); it += kWarps) {
+      const int slot = it % cols, i = lo + it / cols;
+      const Vertices V = vertices(first + slot);
+      if (V.nv == 0) continue;
+      const bool listed = usable[first + slot] != 0;
+      const uint8_t* lists = smem + c.lists + slot * c.list_bytes;
+      const uint32_t* ties = reinterpret_cast<const uint32_t*>(smem + c.ties + slot * c.tie_bytes);
+      const int len = listed ? c.room : c.vmax;  // per warp: best, then partner
+      W.best = reinterpret_cast<int16_t*>(smem + (listed ? c.pairs : c.lists + slot * c.list_bytes)) + warp * 2 * len;
+      W.partner = W.best + len;
+      __syncwarp();  // the warp's previous matching is walked
+      if (mode == kInitGreedyRandom) pk.restart(i, K);
+      const bool good =
+          listed ? match<true>(V, c, lists, ties, W, mode == kInitGreedyRandom, pk, K, Wt_x, Wt_z, C.err, lane)
+                 : match<false>(V, c, lists, ties, W, mode == kInitGreedyRandom, pk, K, Wt_x, Wt_z, C.err, lane);
+      uint32_t* cfg = cfgs + (i - lo) * 2 * w;
+      bool ok = good;
+      // Join every kept pair.
+      for (int x = lane; x < V.nd; x += 32) {
+        const int y = W.partner[x];
+        if (y <= x) continue;
+        const int fx = V.D[x];
+        if (y == V.nd) {
+          ok = walk_boundary(X, fx, cfg) && ok;
+        } else {
+          const int fy = V.D[y];
+          if (internal_weight(V.pq[x], V.pq[y], Wt_x, Wt_z) <= V.wd[x] + V.wd[y]) ok = walk_internal(X, fx, fy, cfg) && ok;
+          else ok = walk_boundary(X, fx, cfg) && walk_boundary(X, fy, cfg) && ok;
+        }
+      }
+      if (!ok) walk_error[i - lo] = 1;
+    }
+    __syncthreads();  // the lists are free for the other colour, the configurations complete
   }
+
+  // Output R_i and its commutation bits with L_Z (bit 0) and L_X (bit 1).
+  const uint32_t* LX = C.logical;
+  const uint32_t* LZ = C.logical + 2 * w;
+  for (int i = lo + warp; i < hi; i += kWarps) {
+    const uint32_t* cfg = cfgs + (i - lo) * 2 * w;
+    uint32_t* out = init + (size_t)i * 2 * w;
+    uint32_t par = 0;  // bit 0: with L_Z, bit 1: with L_X
+    for (int j = lane; j < w; j += 32) {
+      const uint32_t ex = cfg[j], ez = cfg[w + j];
+      out[j] = ex;
+      out[w + j] = ez;
+      par ^= (uint32_t)(__popc((ex & LZ[w + j]) ^ (ez & LZ[j])) & 1) |
+             ((uint32_t)(__popc((ex & LX[w + j]) ^ (ez & LX[j])) & 1) << 1);
+    }
+    par = __reduce_xor_sync(0xFFFFFFFFu, par);
+    if (lane == 0) {
+      // A walk that could not complete is recorded in the code's error area
+      // (XZZX_DEVERR_GREEDY_WALK) and in bit 7 of the restart's class byte.
+      const bool bad = walk_error[i - lo] != 0 || (i == 0 && injected(C.err, XZZX_DEVERR_GREEDY_WALK));
+      if (bad) raise_device_error(C.err, XZZX_DEVERR_GREEDY_WALK);
+      cbits[i] = (uint8_t)(par | (bad ? 0x80 : 0));
+    }
+  }
+}
+
+// How a launch of n_shots x restarts of one code is cut: CTAs per shot, colours
+// held at once, shared memory.  n_ctas(r): the CTAs of the whole launch at r
+// restarts per warp (other segments' included).
+struct Cut {
+  int groups = 1, cols = 2;
+  size_t smem = 0;
+};
+template <class G>
+inline Cut cut_of(const DevCode& C, int restarts, int rpw, bool few) {
+  const bool large = is_large(C);
+  const int warps = large ? kLargeWarps : kSmallWarps;
+  Cut k;
+  k.groups = few ? (restarts + warps / 2 - 1) / (warps / 2) : greedy_groups(restarts, warps, rpw);
+  k.cols = C.ns / 2 > kSmallFaces && !few ? 1 : 2;
+  k.smem = (size_t)carve(C.ns, C.sw, C.w, warps, k.cols, (restarts + k.groups - 1) / k.groups).total;
+  return k;
 }
 
 }  // namespace greedy

@@ -43,6 +43,21 @@ class DeviceOnce {
   std::atomic<uint64_t> done_{0};
 };
 
+#ifdef __CUDACC__
+// Allow a kernel the device's whole shared memory per CTA, and let its CTAs
+// have as much of an SM's as they need.
+template <typename F>
+xzzx_status allow_shared(F kernel) {
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  return e == cudaSuccess ? XZZX_OK : cuda_fail(e, "shared memory limit of a kernel");
+}
+#endif
+
 // NVTX range around the host-side enqueue of one step of the path, so a
 // timeline tool shows greedy (K1), annealing (K2) and decision (K3) launches by
 // name.  Costs a few nanoseconds when no tool is attached.
