@@ -96,8 +96,8 @@ xzzx_status launch_d(const AnnealArgs& A, cudaStream_t stream) {
 }  // namespace
 
 xzzx_status launch_anneal_planar(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
-                                 int n_shots, int restarts, int order, int emin, const uint32_t* init, int32_t* best_E,
-                                 uint32_t* best_cfg, int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream);
+                                 int n_shots, int restarts, const uint32_t* init, int32_t* best_E, uint32_t* best_cfg,
+                                 int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream);
 
 xzzx_status coop_is_faster(int d, int64_t n_chains, bool* yes);
 xzzx_status launch_anneal_coop(const xzzx_code* code, const xzzx_schedule* sched, uint64_t seed, uint64_t shot0,
@@ -109,8 +109,8 @@ xzzx_status launch_anneal(const xzzx_code* code, const xzzx_schedule* sched, uin
                           int32_t* final_E, uint32_t* final_cfg, cudaStream_t stream) {
   NvtxRange nvtx_range("xzzx K2 anneal");
   if (code->layout == kLayoutPlanar)  // colour sweep, minimum per colour phase
-    return launch_anneal_planar(code, sched, seed, shot0, n_shots, restarts, 0, 0, init, best_E, best_cfg, final_E,
-                                final_cfg, stream);
+    return launch_anneal_planar(code, sched, seed, shot0, n_shots, restarts, init, best_E, best_cfg, final_E, final_cfg,
+                                stream);
   bool coop = false;
   xzzx_status st = coop_is_faster(code->d, (int64_t)n_shots * restarts * 4, &coop);
   if (st) return st;

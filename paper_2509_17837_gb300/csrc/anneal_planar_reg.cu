@@ -15,7 +15,7 @@
 // time with the rows unrolled; the edge steps of the odd-row class (left
 // boundary at t = 0, right boundary at the last step) are peeled.
 //
-// Results equal anneal_planar_kernel in order 0 / emin 0 (same draws, same
+// Results equal the lane-parallel kernel (same draws, same
 // acceptance, same per-phase minimum), which the parity tests check.
 #include "anneal_core.cuh"
 
