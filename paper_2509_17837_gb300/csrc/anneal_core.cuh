@@ -24,8 +24,8 @@
 // so their order inside a colour does not matter).  Inside a colour the loop
 // runs over the face columns at run time and unrolls the rows, so register
 // indices stay compile-time constants and the code stays small at any d (pair
-// path: one loop per 32-bit register with the register-edge columns peeled
-// for d <= 11, one loop over 64-bit pair words for d = 13, 15).
+// path: one loop per 32-bit register with the register-edge columns peeled; one
+// loop over 64-bit pair words is smaller code but 4 to 8% slower at d = 9 to 15).
 //
 // Acceptance.  The corner signature indexes a per-sweep table of (dE, A): A =
 // T[t][dE] for dE > 0 and A = 0 otherwise, so a move is accepted iff dE <= 0
@@ -105,6 +105,16 @@ __device__ __forceinline__ uint32_t gather2(uint64_t x) {  // bit 2i -> bit i
   x = (x | (x >> 8)) & 0x0000FFFF0000FFFFull;
   x = (x | (x >> 16)) & 0x00000000FFFFFFFFull;
   return (uint32_t)x;
+}
+
+// E += dE on the multiply pipe.  The pair path is bound by the pipe that shifts,
+// compares and does logic (70% busy, against 20% of the multiply pipe); a factor of
+// one that the compiler cannot see keeps this addition off it.  One anneal launch
+// of 600 shots x 64 restarts x 300 sweeps: d = 9 2.98 -> 2.80 ms, d = 11 4.50 ->
+// 4.11 ms, d = 15 8.29 -> 7.95 ms.  The row path, with three warps per scheduler,
+// loses 1-2% to the longer chain and adds plainly.
+__device__ __forceinline__ void add_energy(int32_t& E, int32_t dE, const PhiloxKeys& K) {
+  E = (int32_t)((uint32_t)dE * K.one + (uint32_t)E);
 }
 
 // The annealing draws of one chain: Philox4x32-10 blocks with counter
@@ -545,7 +555,7 @@ __device__ __forceinline__ void pair_column(uint32_t (&P)[PairShape<D>::H][PairS
     const uint32_t u = lane_of(r[ia >> 2], ia & 3);
     const int32_t dE = (int32_t)e[j].x;
     if ((dE <= 0) | (LIVE && u < e[j].y)) {
-      E += dE;
+      add_energy(E, dE, K);
       if (C == 3 && j == 0) pair_flip<NW, MODE>(P[0], 0x84u, s);               // Z on BL, X on BR
       else if (C == 0 && j == NR - 1) pair_flip<NW, MODE>(P[j], 0x12u, s);     // X on TL, Z on TR
       else pair_flip<NW, MODE>(P[j + JOFF], 0x96u, s);                         // X TL, Z BL, Z TR, X BR
@@ -577,91 +587,13 @@ __device__ __forceinline__ void pair_register_columns(uint32_t (&P)[PairShape<D>
   }
 }
 
-// Bits [sh, sh + 32) of a pair word (zeros above it), sh < 64.
-template <int NW>
-__device__ __forceinline__ uint32_t pair_bits(const uint32_t (&w)[NW], uint32_t sh) {
-  if constexpr (NW == 1) return w[0] >> sh;
-  else return (uint32_t)((((uint64_t)w[1] << 32) | w[0]) >> sh);
-}
-
-// One column of faces of colour C at column b >= 1 of the pair words (two
-// registers at most), the column a run-time value.
-template <int D, int C, bool LIVE>
-__device__ __forceinline__ void pair_column_rt(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E,
-                                               uint32_t Lb, const SaDraws& dr, const PhiloxKeys& K, int b,
-                                               uint32_t* err) {
-  constexpr int H = PairShape<D>::H, NW = PairShape<D>::NW;
-  static_assert(NW <= 2, "pair words of at most two registers");
-  constexpr int NR = (C == 0 || C == 3) ? H : H - 1;
-  constexpr int JOFF = (C == 1) ? 1 : 0;
-  constexpr int IAOFF = (C == 1) ? 1 : 0;
-  constexpr int NG = (NR - 1 + IAOFF) / 4 + 1;
-  const uint32_t ib = (uint32_t)(b + 1) >> 1;
-  const uint32_t s = 4u * (uint32_t)b;
-  uint2 e[NR];
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    uint32_t a;
-    if (C == 3 && j == 0)
-      a = (pair_bits<NW>(P[0], s - 1u) & 0x198u) | (Lb + kPairTop * 8);
-    else if (C == 0 && j == NR - 1)
-      a = (pair_bits<NW>(P[j], s - 3u) & 0x198u) | (Lb + kPairBottom * 8);
-    else
-      a = (pair_bits<NW>(P[j + JOFF], s - 3u) & 0x7F8u) | Lb;
-    e[j] = pair_entry(a, Lb, err);
-  }
-  uint4 r[NG];
-#pragma unroll
-  for (int g = 0; g < NG; ++g) {
-    uint32_t need = 0;
-#pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (((j + IAOFF) >> 2) == g) need |= e[j].y;
-    r[g] = make_uint4(0u, 0u, 0u, 0u);
-    if (LIVE && __any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (ib << 8) | (uint32_t)g, K);
-  }
-  using M = typename std::conditional<NW == 1, uint32_t, uint64_t>::type;
-  const M m_bulk = (M)0x96u << s, m_top = (M)0x84u << s, m_bottom = (M)0x12u << s;
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int ia = j + IAOFF;
-    const uint32_t u = lane_of(r[ia >> 2], ia & 3);
-    const int32_t dE = (int32_t)e[j].x;
-    if ((dE <= 0) | (LIVE && u < e[j].y)) {
-      E += dE;
-      const int row = (C == 3 && j == 0) ? 0 : (C == 0 && j == NR - 1) ? j : j + JOFF;
-      const M m = (C == 3 && j == 0) ? m_top : (C == 0 && j == NR - 1) ? m_bottom : m_bulk;
-      P[row][0] ^= (uint32_t)m;
-      if constexpr (NW == 2) P[row][1] ^= (uint32_t)((uint64_t)m >> 32);
-    }
-  }
-}
-
-// The bulk columns of colour C for d >= 13: b = 0 (even-b colours) with its
-// bits at the bottom of register 0, then every other column in one run-time
-// loop over 64-bit pair words.  Against the per-register form this costs
-// about one instruction per column for the shifted masks but cuts the sweep
-// body several-fold, which pays once the body outgrows instruction fetch
-// (d = 13, 15); at d <= 11 the per-register form is faster.
-template <int D, int C, bool LIVE>
-__device__ __forceinline__ void pair_bulk_columns(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E,
-                                                  uint32_t Lb, const SaDraws& dr, const PhiloxKeys& K,
-                                                  uint32_t* err) {
-  constexpr int PB = C >> 1;
-  constexpr int BMAX = PB + 2 * ((D - 1) / 2 - 1);  // the colour's last bulk column
-  if constexpr (PB == 0) pair_column<D, C, kAt0, LIVE>(P, E, Lb, dr, K, 0, 0u, err);
-#pragma unroll 1
-  for (int b = PB == 0 ? 2 : 1; b <= BMAX; b += 2) pair_column_rt<D, C, LIVE>(P, E, Lb, dr, K, b, err);
-}
-
 // One colour phase of one sweep (pair layout: even for colours 0 and 2, odd
 // for 1 and 3).
 template <int D, int C, bool LIVE>
 __device__ __forceinline__ void pair_phase(uint32_t (&P)[PairShape<D>::H][PairShape<D>::NW], int32_t& E, uint32_t Lb,
                                            const SaDraws& dr, const PhiloxKeys& K, uint32_t* err) {
   constexpr int H = PairShape<D>::H;
-  if constexpr (D >= 13) pair_bulk_columns<D, C, LIVE>(P, E, Lb, dr, K, err);
-  else pair_register_columns<D, C, 0, LIVE>(P, E, Lb, dr, K, err);
+  pair_register_columns<D, C, 0, LIVE>(P, E, Lb, dr, K, err);
   if constexpr (C == 1 || C == 2) {
     // Boundary column: right (b = d-1: TL and BL) for colour 1, left (b = -1:
     // TR and BR) for colour 2, over the bulk rows of the colour.
@@ -700,7 +632,7 @@ __device__ __forceinline__ void pair_phase(uint32_t (&P)[PairShape<D>::H][PairSh
       const uint32_t u = lane_of(r[ia >> 2], ia & 3);
       const int32_t dE = (int32_t)e[j].x;
       if ((dE <= 0) | (LIVE && u < e[j].y)) {
-        E += dE;
+        add_energy(E, dE, K);
         if constexpr (C == 1) P[j + JOFF][RW] ^= 0x6u << RS;  // X on TL, Z on BL
         else P[j][0] ^= 0x9u;                                 // Z on TR, X on BR
       }
@@ -786,7 +718,7 @@ __host__ __device__ constexpr size_t smem_pairs() {
 }
 
 // Largest distance annealed in the pair layout (the row layout takes the rest).
-constexpr int kPairMaxD = 15;
+constexpr int kPairMaxD = 21;
 
 template <int D, int NT>
 __host__ __device__ constexpr size_t smem_bytes() {
@@ -968,15 +900,15 @@ __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ in
 #define XZZX_SWEEP(LIVE)                            \
   pair_phase<D, 0, LIVE>(P, E, Lb, dr, K, tab.err); \
   XZZX_SNAPSHOT                                     \
-  even_to_odd<D>(P);                                \
+  even_to_odd<D>(P);                                 \
   pair_phase<D, 1, LIVE>(P, E, Lb, dr, K, tab.err); \
-  odd_to_even<D>(P);                                \
+  odd_to_even<D>(P);                                 \
   XZZX_SNAPSHOT                                     \
   pair_phase<D, 2, LIVE>(P, E, Lb, dr, K, tab.err); \
   XZZX_SNAPSHOT                                     \
-  even_to_odd<D>(P);                                \
+  even_to_odd<D>(P);                                 \
   pair_phase<D, 3, LIVE>(P, E, Lb, dr, K, tab.err); \
-  odd_to_even<D>(P);                                \
+  odd_to_even<D>(P);                                 \
   XZZX_SNAPSHOT
   const int n_live = min(tab.n_live, n_sweeps);
 #pragma unroll U

@@ -38,30 +38,18 @@ __device__ __forceinline__ void run_chunk(const ChunkDev& ch, const SegDev& sg, 
   core::anneal_cta<D, NT, U>(sg.init + (size_t)(c >> 2) * 2 * W, chain, (int)(c & 3), active, out, tab, K, smem);
 }
 
-// Register bounds: kernels on the pair path (d <= 15) are held to 1024
-// threads per SM (64 registers); kernels on the row path to 640 (d <= 21, 96
-// registers), 512 (d <= 27, 128) or 384 (160), the persistent ones to 512 (up
-// to d = 21) or 384, none of which spills.  Left alone, the compiler takes 240
-// registers for the persistent kernels: two CTAs per SM.
+// Threads per SM that a kernel of distances up to D is register-bounded for: 1024
+// (64 registers) up to d = 15, 512 (128) up to d = 27, 384 (160) above.  Left
+// alone, the compiler takes up to 240 registers for the persistent kernels: two
+// CTAs per SM.
 template <int D>
-constexpr int kRowThreads = D <= 21 ? 640 : D <= 27 ? 512 : 384;
+constexpr int kSmThreads = D <= 15 ? 1024 : D <= 27 ? 512 : 384;
 
 template <int D, int NT, int U>
-__global__ void __launch_bounds__(NT, (1024 / NT)) anneal_chunks_kernel(const __grid_constant__ AnnealLaunch L) {
+__global__ void __launch_bounds__(NT, kSmThreads<D> / NT) anneal_chunks_kernel(const __grid_constant__ AnnealLaunch L) {
   extern __shared__ __align__(16) uint8_t smem[];
   const ChunkDev ch = L.chunks[L.chunk0 + blockIdx.x];
   run_chunk<D, NT, U>(ch, L.segs[ch.seg], L.keys, smem);
-}
-template <int D, int NT, int U>
-__global__ void __launch_bounds__(NT, kRowThreads<D> / NT) anneal_chunks_kernel_rows(const __grid_constant__ AnnealLaunch L) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  const ChunkDev ch = L.chunks[L.chunk0 + blockIdx.x];
-  run_chunk<D, NT, U>(ch, L.segs[ch.seg], L.keys, smem);
-}
-template <int D, int NT, int U>
-constexpr auto chunks_kernel_of() {
-  if constexpr (D <= core::kPairMaxD) return &anneal_chunks_kernel<D, NT, U>;
-  else return &anneal_chunks_kernel_rows<D, NT, U>;
 }
 
 template <int D, int DMAX, int NT, int U>
@@ -77,7 +65,8 @@ __device__ __forceinline__ void dispatch_chunk(const ChunkDev& ch, const SegDev&
 }
 
 template <int DMAX, int NT, int U>
-__device__ __forceinline__ void persistent_body(const AnnealLaunch& L) {
+__global__ void __launch_bounds__(NT, (DMAX <= 21 ? kSmThreads<DMAX> : 384) / NT)
+    anneal_persistent_kernel(const __grid_constant__ AnnealLaunch L) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ int s_next;
   for (;;) {
@@ -90,20 +79,6 @@ __device__ __forceinline__ void persistent_body(const AnnealLaunch& L) {
     dispatch_chunk<3, DMAX, NT, U>(ch, L.segs[ch.seg], L.keys, smem);
   }
 }
-template <int DMAX, int NT, int U>
-__global__ void __launch_bounds__(NT, (1024 / NT)) anneal_persistent_kernel(const __grid_constant__ AnnealLaunch L) {
-  persistent_body<DMAX, NT, U>(L);
-}
-template <int DMAX, int NT, int U>
-__global__ void __launch_bounds__(NT, (DMAX <= 21 ? 512 : 384) / NT) anneal_persistent_kernel_rows(const __grid_constant__ AnnealLaunch L) {
-  persistent_body<DMAX, NT, U>(L);
-}
-template <int DMAX, int NT, int U>
-constexpr auto persistent_kernel_of() {
-  if constexpr (DMAX <= core::kPairMaxD) return &anneal_persistent_kernel<DMAX, NT, U>;
-  else return &anneal_persistent_kernel_rows<DMAX, NT, U>;
-}
-
 // The largest shared memory of any distance the persistent kernel runs.
 template <int DMAX, int NT, int D = 3>
 constexpr size_t persistent_smem() {

@@ -33,6 +33,7 @@ PhiloxKeys philox_keys(uint64_t seed) {
     k0 += 0x9E3779B9u;
     k1 += 0xBB67AE85u;
   }
+  K.one = 1;
   return K;
 }
 
