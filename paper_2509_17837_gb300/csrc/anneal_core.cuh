@@ -4,15 +4,15 @@
 // multi-distance kernel all call anneal_cta<D, NT>, so every launch form runs
 // the same instruction stream on the same state and gives identical results.
 //
-// State, d > 15 ("rows").  A chain lives in registers as one 64-bit word per
+// State, d > 21 ("rows").  A chain lives in registers as one 64-bit word per
 // lattice row, two bits per qubit (bit 2c = Z bit, bit 2c+1 = X bit of column
 // c).  The four corners of face (a, b) are then the 4-bit fields at bit 2b of
 // rows a and a+1, and applying G_f is two XORs with fixed masks.
 //
-// State, d <= 15 ("pairs").  Two lattice rows share one pair word, four bits
+// State, d <= 21 ("pairs").  Two lattice rows share one pair word, four bits
 // per column: bits [4c, 4c+2) hold (z, x) of column c of the first row, bits
 // [4c+2, 4c+4) those of the second row; a pair word takes two 32-bit registers
-// for d >= 9.  The even layout pairs rows (2j, 2j+1), the odd layout rows
+// for d = 9 to 15 and three above.  The even layout pairs rows (2j, 2j+1), the odd layout rows
 // (2j-1, 2j) (row -1 and row d are empty).  Faces of colours 0 and 2 sit on
 // even rows a, faces of colours 1 and 3 on odd ones, so in the layout of its
 // colour the 8-bit signature of face (a, b) is one byte of one pair word, at
@@ -236,7 +236,7 @@ __device__ __forceinline__ void store_rows(const Row (&R)[D], uint32_t* __restri
   }
 }
 
-// One colour phase of one sweep (row layout, d > 15).  LIVE = false: no
+// One colour phase of one sweep (row layout, d > 21).  LIVE = false: no
 // threshold is above zero, so a move is taken iff dE <= 0 and nothing is drawn.
 template <int D, int C, bool LIVE, typename Row>
 __device__ __forceinline__ void colour_phase(Row (&R)[D], int32_t& E, const uint2* __restrict__ L, const SaDraws& dr,
@@ -373,7 +373,7 @@ __device__ __forceinline__ void build_lut_warp(uint2* __restrict__ dst, const in
 }
 
 // ---------------------------------------------------------------------------
-// Pair layout (d <= 15).
+// Pair layout (d <= 21).
 // ---------------------------------------------------------------------------
 
 template <int D>
@@ -660,6 +660,17 @@ __device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v));
 }
 
+// Appends v to a shared list where on is set, in any order, one shared-memory
+// atomic per warp; the whole warp calls this.
+__device__ __forceinline__ void append_entry(bool on, uint32_t v, uint32_t* __restrict__ list, int* __restrict__ n) {
+  const uint32_t m = __ballot_sync(0xFFFFFFFFu, on);
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  if (lane == 0 && m) base = atomicAdd(n, __popc(m));
+  base = __shfl_sync(0xFFFFFFFFu, base, 0);
+  if (on) list[base + __popc(m & ((1u << lane) - 1u))] = v;
+}
+
 // Pair table of one warp (slot at shared address Lb) for the first sweep, in
 // full, from the CTA's static (dE, class) table in pair order.
 __device__ __forceinline__ void build_lut_pair(uint32_t Lb, const int2* __restrict__ sig_pair,
@@ -725,7 +736,7 @@ __host__ __device__ constexpr size_t smem_bytes() {
   return D <= kPairMaxD ? smem_pairs<D, NT>() : smem_rows<D, NT>();
 }
 
-// Row path (d > 15).  Arguments as anneal_cta.
+// Row path (d > 21).  Arguments as anneal_cta.
 template <int D, int NT, int U>
 __device__ __forceinline__ void anneal_cta_rows(const uint32_t* __restrict__ init, uint64_t chain, int P, bool active,
                                                 const ChainOut& out, const SweepTables& tab, const PhiloxKeys& K,

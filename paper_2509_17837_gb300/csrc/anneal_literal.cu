@@ -250,12 +250,13 @@ __global__ void __launch_bounds__(kThreads) anneal_literal_kernel(const __grid_c
     faces[f] = descriptor<PLANAR, Row>(A.face_a[f], A.face_b[f], d);
     if (ORDER == 0) places[f] = draw_place<PLANAR>(A.face_a[f], A.face_b[f]);
   }
+  static_assert(kEntries % kThreads == 0, "whole warps in every pass");
   for (int k = tid; k < kEntries; k += kThreads) {
     const int src = sig_source<PLANAR>(k);
     const int2 sg = src >= 0 ? __ldg(&A.sig[src]) : make_int2(1, -1);
 #pragma unroll
     for (int b = 0; b < 2; ++b) core::sts_u2(s0 + c.tables + 8u * (uint32_t)(b * kEntries + k), make_uint2((uint32_t)sg.x, 0u));
-    if (sg.y >= 0) upd[atomicAdd(n_upd_s, 1)] = ((uint32_t)k << 16) | (uint32_t)sg.y;
+    core::append_entry(sg.y >= 0, ((uint32_t)k << 16) | (uint32_t)sg.y, upd, n_upd_s);
   }
   __syncthreads();
   const int n_upd = *n_upd_s;

@@ -2,9 +2,10 @@
 // colour phase): the planar counterpart of anneal_cta, for d <= 15.
 //
 // State.  One chain per thread, one 32-bit word per grid row in registers
-// (row r holds its 2d-1 or d-1 qubits as two bits per slot k, column
-// c = 2k + (r&1)), so a face's corners are fields of rows i-1, i and i+1 at
-// shifts fixed by the column step.
+// (row r holds its d or d-1 qubits as two bits per slot k, column c = 2k +
+// (r&1)).  A phase packs the up and down corners of each of its rows' faces into
+// one word first (Packed), so a face is two nibbles at shifts fixed by the column
+// step, and a move two XORs.
 //
 // Sweep.  Colour C holds the faces (i, j) with i & 1 = C & 1 and
 // ((i+j-1)/2) & 1 = C >> 1.  With m = i >> 1 (the row inside the class) and
@@ -43,7 +44,7 @@ struct RegArgs {
   PhiloxKeys keys;
   uint64_t chain0;
   int64_t n_chains;
-  int n_sweeps, n_classes;
+  int n_sweeps, n_classes, n_live;
   int32_t W[4];
   const uint32_t* T;
   const int2* sig;
@@ -52,6 +53,7 @@ struct RegArgs {
   uint32_t* best_cfg;
   int32_t* final_E;
   uint32_t* final_cfg;
+  uint32_t* err;
 };
 
 template <int D>
@@ -108,38 +110,53 @@ __host__ __device__ constexpr int kind_of(int m) {
                                              : (kl0_of<C>(m) == -1 ? kKNoRight : kKNone));
 }
 
-// All faces of colour C at column step `step` (POS as kind_of) of sweep `sweep`.
-template <int D, int C, int POS>
-__device__ __forceinline__ void pstep(uint32_t (&R)[PShape<D>::G], int32_t& E, const uint2* __restrict__ L,
-                                      uint32_t step, uint32_t sweep, uint32_t c2, uint32_t c3, const PhiloxKeys& K) {
+// The up and down corners of the faces of one row and colour, packed for the
+// phase.  Their faces use every second slot of the rows above and below (slots of
+// parity KL + CL, KL the row's first slot in the colour); U holds the upper row's
+// at those slots and the lower row's at the slots between, so that a face's up and
+// down bits are a nibble at the bit of its left corner (CL: one slot on).
+template <int KL, int CL>
+struct Packed {
+  static constexpr int P = (KL + CL) & 1;
+  static constexpr uint32_t kMask = P ? 0xCCCCCCCCu : 0x33333333u;  // slots of parity P
+  __device__ static uint32_t pack(uint32_t up, uint32_t down) {
+    return P ? ((up & kMask) >> 2) | (down & kMask) : (up & kMask) | ((down & kMask) << 2);
+  }
+  // The row above's slots of parity P, and the row below's, from U.
+  __device__ static uint32_t up(uint32_t U) { return P ? (U & 0x33333333u) << 2 : U & 0x33333333u; }
+  __device__ static uint32_t down(uint32_t U) { return P ? U & 0xCCCCCCCCu : (U & 0xCCCCCCCCu) >> 2; }
+};
+
+// All faces of colour C at column step `step` (POS as kind_of) of a sweep; U: the
+// packed corners of the class's rows.  A face (row m, slot kl = 2 step + kl0(m))
+// has its left and right corners at bit 2 kl of row i = 2m + CL, its up and down
+// ones at bit 4 step of U[m] when kl0 + CL is 0 or 1, which the packing arranges.
+template <int D, int C, int POS, bool LIVE>
+__device__ __forceinline__ void pstep(uint32_t (&R)[PShape<D>::G], uint32_t (&U)[D], int32_t& E, uint32_t Lb,
+                                      uint32_t step, const core::SaDraws& dr, const PhiloxKeys& K, uint32_t* err) {
   constexpr int CL = C & 1;
   constexpr int M = CL ? D - 1 : D;
   constexpr int NG = (M + 3) / 4;
-  constexpr int G = PShape<D>::G;
   uint2 e[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) {
     const int i = 2 * m + CL;
     const int kind = kind_of<D, C, POS>(m);
-    // slot kl = 2 step + kl0: left corner at bit 2kl of row i, up/down at 2(kl + CL) of rows i -+ 1
     const int sm = 4 * (int)step + 2 * kl0_of<C>(m);
-    const uint32_t smid = (uint32_t)(sm < 0 ? 0 : sm), sud = (uint32_t)(sm + 2 * CL);
+    const uint32_t smid = (uint32_t)(sm < 0 ? 0 : sm);
     e[m] = make_uint2(0u, 0u);
     if (kind == kKNone) continue;
-    const uint32_t up = (kind != kKNoUp) ? (R[i > 0 ? i - 1 : 0] >> sud) & 3u : 0u;
-    const uint32_t dn = (kind != kKNoDown) ? (R[i + 1 < G ? i + 1 : i] >> sud) & 3u : 0u;
-    uint32_t idx;
-    if (kind == kKNoLeft) {
-      idx = kPOffNoLeft + ((R[i] & 3u) | (up << 2) | (dn << 4));
-    } else if (kind == kKNoRight) {
-      idx = kPOffNoRight + (((R[i] >> smid) & 3u) | (up << 2) | (dn << 4));
-    } else {
-      const uint32_t lr = (R[i] >> smid) & 0xFu;
-      if (kind == kKNoUp) idx = kPOffNoUp + (lr | (dn << 4));
-      else if (kind == kKNoDown) idx = kPOffNoDown + (lr | (up << 4));
-      else idx = lr | (up << 4) | (dn << 6);
-    }
-    e[m] = L[idx];
+    const uint32_t ud = (U[m] >> (4 * (int)step)) & (kind == kKNoUp ? 0xCu : kind == kKNoDown ? 0x3u : 0xFu);
+    uint32_t a;
+    // Entry address: 8 (lr | ud << 4), a missing corner closed up; the bulk's
+    // products by factors the compiler cannot see, on the multiply pipe.
+    if (kind == kKNoLeft) a = ud * 32u + ((R[i] & 3u) * 8u + (Lb + 8u * kPOffNoLeft));
+    else if (kind == kKNoRight) a = ud * 32u + (((R[i] >> smid) & 3u) * 8u + (Lb + 8u * kPOffNoRight));
+    else if (kind == kKNoUp) a = ud * 32u + (((R[i] >> smid) & 0xFu) * 8u + (Lb + 8u * kPOffNoUp));
+    else if (kind == kKNoDown) a = ud * 128u + (((R[i] >> smid) & 0xFu) * 8u + (Lb + 8u * kPOffNoDown));
+    else a = ud * K.c128 + (((R[i] >> smid) & 0xFu) * K.c8 + Lb);
+    e[m] = XZZX_CHECK(err, a - Lb <= 8u * (kRLut - 1) && !injected(err, XZZX_DEVERR_BOUNDS)) ? core::lds_u2(a)
+                                                                                           : make_uint2(0u, 0u);
   }
   uint4 r[NG];
 #pragma unroll
@@ -149,8 +166,7 @@ __device__ __forceinline__ void pstep(uint32_t (&R)[PShape<D>::G], int32_t& E, c
     for (int m = 0; m < M; ++m)
       if ((m >> 2) == g) need |= e[m].y;
     r[g] = make_uint4(0u, 0u, 0u, 0u);
-    if (__any_sync(0xFFFFFFFFu, need != 0u))
-      r[g] = philox4x32_10(((uint32_t)C << 16) | (step << 8) | (uint32_t)g, sweep, c2, c3, K);
+    if (LIVE && __any_sync(0xFFFFFFFFu, need != 0u)) r[g] = dr.block(((uint32_t)C << 16) | (step << 8) | (uint32_t)g, K);
   }
 #pragma unroll
   for (int m = 0; m < M; ++m) {
@@ -158,72 +174,98 @@ __device__ __forceinline__ void pstep(uint32_t (&R)[PShape<D>::G], int32_t& E, c
     if (kind == kKNone) continue;
     const int i = 2 * m + CL;
     const int sm = 4 * (int)step + 2 * kl0_of<C>(m);
-    const uint32_t smid = (uint32_t)(sm < 0 ? 0 : sm), sud = (uint32_t)(sm + 2 * CL);
+    const uint32_t smid = (uint32_t)(sm < 0 ? 0 : sm);
     const uint32_t u = lane_of(r[m >> 2], m & 3);
     const int32_t dE = (int32_t)e[m].x;
-    if ((dE <= 0) | (u < e[m].y)) {
-      E += dE;
+    if ((dE <= 0) | (LIVE && u < e[m].y)) {
+      core::add_energy(E, dE, K);
       if (kind == kKNoLeft) R[i] ^= 2u;
       else if (kind == kKNoRight) R[i] ^= 2u << smid;
       else R[i] ^= 0xAu << smid;
-      const uint32_t mud = 1u << sud;
-      if (kind != kKNoUp) R[i > 0 ? i - 1 : 0] ^= mud;
-      if (kind != kKNoDown) R[i + 1 < G ? i + 1 : i] ^= mud;
+      U[m] ^= (kind == kKNoUp ? 0x4u : kind == kKNoDown ? 0x1u : 0x5u) << (4 * (int)step);
     }
   }
 }
 
-// One colour phase: the column steps of colour C.
-template <int D, int C>
-__device__ __forceinline__ void pphase(uint32_t (&R)[PShape<D>::G], int32_t& E, const uint2* __restrict__ L,
-                                       uint32_t sweep, uint32_t c2, uint32_t c3, const PhiloxKeys& K) {
+// One colour phase: pack the class's neighbours, its column steps, unpack.
+template <int D, int C, bool LIVE>
+__device__ __forceinline__ void pphase(uint32_t (&R)[PShape<D>::G], int32_t& E, uint32_t Lb, const core::SaDraws& dr,
+                                       const PhiloxKeys& K, uint32_t* err) {
+  constexpr int CL = C & 1, M = CL ? D - 1 : D, G = PShape<D>::G;
   constexpr int NS = (D - 1) / 2;  // column steps of the even-row class; the odd-row class has NS + 1
-  if ((C & 1) == 0) {
+  constexpr int K0 = kl0_of<C>(0), K1 = kl0_of<C>(1);  // even and odd m
+  uint32_t U[D];
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const int i = 2 * m + CL;
+    const uint32_t up = i > 0 ? R[i > 0 ? i - 1 : 0] : 0u, dn = i + 1 < G ? R[i + 1 < G ? i + 1 : i] : 0u;
+    U[m] = (m & 1) ? Packed<K1, CL>::pack(up, dn) : Packed<K0, CL>::pack(up, dn);
+  }
+  if (CL == 0) {
 #pragma unroll 1
-    for (int s = 0; s < NS; ++s) pstep<D, C, 0>(R, E, L, (uint32_t)s, sweep, c2, c3, K);
+    for (int s = 0; s < NS; ++s) pstep<D, C, 0, LIVE>(R, U, E, Lb, (uint32_t)s, dr, K, err);
   } else {
-    pstep<D, C, 1>(R, E, L, 0u, sweep, c2, c3, K);
+    pstep<D, C, 1, LIVE>(R, U, E, Lb, 0u, dr, K, err);
 #pragma unroll 1
-    for (int s = 1; s < NS; ++s) pstep<D, C, 0>(R, E, L, (uint32_t)s, sweep, c2, c3, K);
-    pstep<D, C, 2>(R, E, L, (uint32_t)NS, sweep, c2, c3, K);
+    for (int s = 1; s < NS; ++s) pstep<D, C, 0, LIVE>(R, U, E, Lb, (uint32_t)s, dr, K, err);
+    pstep<D, C, 2, LIVE>(R, U, E, Lb, (uint32_t)NS, dr, K, err);
+  }
+  // The row between face rows m and m + 1: m's lower corners and m + 1's upper ones.
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const int i = 2 * m + CL;
+    if (m == 0 && i > 0)  // the row above the class's first: its other slots are untouched
+      R[i - 1] = (R[i - 1] & ~Packed<K0, CL>::kMask) | Packed<K0, CL>::up(U[0]);
+    if (i + 1 >= G) continue;
+    const uint32_t dn = (m & 1) ? Packed<K1, CL>::down(U[m]) : Packed<K0, CL>::down(U[m]);
+    if (m + 1 < M) R[i + 1] = dn | ((m & 1) ? Packed<K0, CL>::up(U[m + 1]) : Packed<K1, CL>::up(U[m + 1]));
+    else R[i + 1] = (R[i + 1] & ~((m & 1) ? Packed<K1, CL>::kMask : Packed<K0, CL>::kMask)) | dn;
   }
 }
 
-__device__ __forceinline__ void build_lut_planar(uint2* __restrict__ dst, const int2* __restrict__ sig_static,
-                                                 const uint32_t* __restrict__ Trow, int lane) {
-  for (int idx = lane; idx < kRLut; idx += 32) {
-    const int2 s = sig_static[idx];
-    dst[idx] = make_uint2((uint32_t)s.x, s.y >= 0 ? __ldg(&Trow[s.y]) : 0u);
-  }
-}
-
+// Shared memory: one table per warp, the list of entries whose threshold changes
+// per sweep, one configuration per chain.
 template <int D>
 constexpr size_t reg_smem_bytes() {
-  return kRLut * sizeof(int2) + (kRThreads / 32) * kRLut * sizeof(uint2) +
+  return (kRThreads / 32) * kRLut * sizeof(uint2) + kRLut * sizeof(uint32_t) + 16 +
          (size_t)PShape<D>::G * kRThreads * sizeof(uint32_t);
 }
 
+// Bound by the pipe of shifts and logic together with the wide multiplies of the
+// draws.  600 shots x 64 restarts, against three-row faces, a table rebuilt every
+// sweep and no frozen sweeps: 50 sweeps near the Nishimori temperature d = 9 1.65 ->
+// 1.53 ms, d = 15 5.58 -> 4.37 ms; 200 sweeps to 20 times it d = 9 4.95 -> 4.17 ms, d =
+// 15 18.7 -> 14.9 ms.  Held to seven CTAs per SM (72 registers) d = 9 takes 1.56 ms.
 template <int D>
-__global__ void __launch_bounds__(kRThreads) anneal_planar_reg_kernel(const __grid_constant__ RegArgs A) {
+__global__ void __launch_bounds__(kRThreads, 1) anneal_planar_reg_kernel(const __grid_constant__ RegArgs A) {
   constexpr int G = PShape<D>::G;
   constexpr int W = PShape<D>::kW;
   extern __shared__ __align__(16) uint8_t smem[];
-  int2* sig_static = reinterpret_cast<int2*>(smem);
-  uint2* lut_all = reinterpret_cast<uint2*>(smem + kRLut * sizeof(int2));
-  uint32_t* best_rows = reinterpret_cast<uint32_t*>(smem + kRLut * sizeof(int2) + (kRThreads / 32) * kRLut * sizeof(uint2));
   const int tid = threadIdx.x, lane = tid & 31;
-  uint2* L = lut_all + (tid >> 5) * kRLut;
+  uint32_t* upd = reinterpret_cast<uint32_t*>(smem + (kRThreads / 32) * kRLut * sizeof(uint2));
+  int* n_upd_s = reinterpret_cast<int*>(upd + kRLut);
+  uint32_t* kept = reinterpret_cast<uint32_t*>(n_upd_s + 4);  // [G][kRThreads]
+  const uint32_t L0 = (uint32_t)__cvta_generic_to_shared(smem), Lb = L0 + (uint32_t)(tid >> 5) * kRLut * 8u;
   const int64_t c_raw = (int64_t)blockIdx.x * kRThreads + tid;
   const bool active = c_raw < A.n_chains;
   const int64_t c = active ? c_raw : A.n_chains - 1;  // inactive threads shadow a real chain
   const uint64_t chain = A.chain0 + (uint64_t)c;
-  const uint32_t c2 = (uint32_t)chain;
-  const uint32_t c3 = kTagSA | ((uint32_t)(chain >> 32) << 8);
   const int P = (int)(c & 3);
 
-  for (int k = tid; k < kRLut; k += kRThreads) sig_static[k] = __ldg(&A.sig[kSigRot + k]);
+  // Every warp's table for the first sweep, in full, and the list of the entries
+  // whose threshold changes.
+  if (tid == 0) n_upd_s[0] = 0;
   __syncthreads();
-  if (A.n_sweeps > 0) build_lut_planar(L, sig_static, A.T, lane);
+  static_assert(kRLut % kRThreads == 0, "whole warps in every pass");
+  for (int k = tid; k < kRLut; k += kRThreads) {
+    const int2 sg = __ldg(&A.sig[kSigRot + k]);
+    const uint2 entry = make_uint2((uint32_t)sg.x, sg.y >= 0 && A.n_sweeps > 0 ? __ldg(&A.T[sg.y]) : 0u);
+#pragma unroll
+    for (int w = 0; w < kRThreads / 32; ++w) core::sts_u2(L0 + (uint32_t)(w * kRLut + k) * 8u, entry);
+    core::append_entry(sg.y >= 0, ((uint32_t)k << 16) | (uint32_t)sg.y, upd, n_upd_s);
+  }
+  __syncthreads();  // the last CTA barrier: warps then sweep independently
+  const int n_upd = n_upd_s[0];
 
   uint32_t R[G];
   pload<D>(A.init + (size_t)(c >> 2) * 2 * W, R);
@@ -243,36 +285,60 @@ __global__ void __launch_bounds__(kRThreads) anneal_planar_reg_kernel(const __gr
   }
   int32_t E = nx * A.W[2] + ny * A.W[3] + nz * A.W[1];
   int32_t E_best = E;
+  const bool keep = A.best_cfg != nullptr;
+  auto save = [&] {
 #pragma unroll
-  for (int r = 0; r < G; ++r) best_rows[r * kRThreads + tid] = R[r];
+    for (int r = 0; r < G; ++r) kept[r * kRThreads + tid] = R[r];
+  };
+  if (keep) save();
 
-  for (int t = 0; t < A.n_sweeps; ++t) {
-    const uint32_t tt = (uint32_t)t;
-#define XZZX_PPHASE(CC)                                                              \
-  pphase<D, CC>(R, E, L, tt, c2, c3, A.keys);                                        \
-  if (E < E_best) {                                                                  \
-    E_best = E;                                                                      \
-    _Pragma("unroll") for (int r = 0; r < G; ++r) best_rows[r * kRThreads + tid] = R[r]; \
+  core::SaDraws dr;
+  dr.init((uint32_t)chain, kTagSA | ((uint32_t)(chain >> 32) << 8), A.keys);
+#define XZZX_PPHASE(CC, LIVE)                               \
+  pphase<D, CC, LIVE>(R, E, Lb, dr, A.keys, A.err);         \
+  if (E < E_best) {                                         \
+    E_best = E;                                             \
+    if (keep) save();                                       \
   }
-    XZZX_PPHASE(0)
-    XZZX_PPHASE(1)
-    XZZX_PPHASE(2)
-    XZZX_PPHASE(3)
-#undef XZZX_PPHASE
-    if (t + 1 < A.n_sweeps) {
+  for (int t = 0; t < A.n_live; ++t) {
+    dr.sweep((uint32_t)t, A.keys);
+    XZZX_PPHASE(0, true)
+    XZZX_PPHASE(1, true)
+    XZZX_PPHASE(2, true)
+    XZZX_PPHASE(3, true)
+    if (t + 1 < A.n_live) {  // next sweep's thresholds, once every lane is done with these
       __syncwarp();
-      build_lut_planar(L, sig_static, A.T + (size_t)(t + 1) * A.n_classes, lane);
+      core::update_lut_pair(Lb, upd, n_upd, A.T + (size_t)(t + 1) * A.n_classes, lane);
       __syncwarp();
     }
   }
+  // The frozen sweeps (see anneal_core.cuh); the saved configuration takes the
+  // place of the minimum's when nobody asks for that.
+  const bool may_stop = !A.final_E && !A.final_cfg && !keep;
+  bool done = false;
+  for (int t = A.n_live, i = 0; t < A.n_sweeps; ++t, ++i) {
+    if (may_stop && (i & (i + 1)) == 0) save();
+    XZZX_PPHASE(0, false)
+    XZZX_PPHASE(1, false)
+    XZZX_PPHASE(2, false)
+    XZZX_PPHASE(3, false)
+    if (may_stop) {
+      uint32_t diff = 0;
+#pragma unroll
+      for (int r = 0; r < G; ++r) diff |= R[r] ^ kept[r * kRThreads + tid];
+      done |= diff == 0u;
+      if (__all_sync(0xFFFFFFFFu, done)) break;
+    }
+  }
+#undef XZZX_PPHASE
 
   if (!active) return;
   A.best_E[c] = E_best;
   if (A.final_E) A.final_E[c] = E;
   if (A.final_cfg) pstore<D>(R, A.final_cfg + (size_t)c * 2 * W);
-  if (A.best_cfg) {
+  if (keep) {
 #pragma unroll
-    for (int r = 0; r < G; ++r) R[r] = best_rows[r * kRThreads + tid];
+    for (int r = 0; r < G; ++r) R[r] = kept[r * kRThreads + tid];
     pstore<D>(R, A.best_cfg + (size_t)c * 2 * W);
   }
 }
@@ -307,6 +373,7 @@ xzzx_status launch_anneal_planar_reg(const xzzx_code* code, const xzzx_schedule*
   A.n_chains = (int64_t)n_shots * restarts * 4;
   A.n_sweeps = sched->n_sweeps;
   A.n_classes = sched->n_classes;
+  A.n_live = sched->n_live[kLayoutPlanar];
   for (int k = 0; k < 4; ++k) A.W[k] = sched->noise.W[k];
   A.T = sched->d_T;
   A.sig = sched->d_sig;
@@ -315,6 +382,7 @@ xzzx_status launch_anneal_planar_reg(const xzzx_code* code, const xzzx_schedule*
   A.best_cfg = best_cfg;
   A.final_E = final_E;
   A.final_cfg = final_cfg;
+  A.err = code->dev.err;
   switch (code->d) {
     case 3: return launch_d<3>(A, stream);
     case 5: return launch_d<5>(A, stream);

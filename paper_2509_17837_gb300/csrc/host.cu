@@ -34,6 +34,8 @@ PhiloxKeys philox_keys(uint64_t seed) {
     k1 += 0xBB67AE85u;
   }
   K.one = 1;
+  K.c8 = 8;
+  K.c128 = 128;
   return K;
 }
 

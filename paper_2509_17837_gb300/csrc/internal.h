@@ -117,7 +117,7 @@ constexpr int kSigTable = kSigRot + kSigPlanar;
 // Round keys of Philox4x32-10 for one seed, in kernel-parameter space.
 struct PhiloxKeys {
   uint32_t k0[10], k1[10];
-  uint32_t one;  // 1 (see add_energy in anneal_core.cuh)
+  uint32_t one, c8, c128;  // 1, 8 and 128: factors the compiler cannot see (add_energy in anneal_core.cuh)
 };
 PhiloxKeys philox_keys(uint64_t seed);
 
