@@ -16,10 +16,10 @@ namespace {
 
 // Batched form: the chunks of one distance, each cut into CTAs of kCtaChains
 // chains (so a CTA's chains share a segment and its thresholds).
-template <class Geo, int NC, int NP>
-__global__ void __launch_bounds__(Form<Geo, NC, NP>::kThreads, kMinCtas<NP>)
+template <class Geo, int NC, int NP, int KB>
+__global__ void __launch_bounds__(Form<Geo, NC, NP, KB>::kThreads, kMinCtas<NP, KB>)
     coop_chunks_kernel(const __grid_constant__ batch::CoopLaunch L) {
-  constexpr int kCta = Form<Geo, NC, NP>::kCtaChains;
+  constexpr int kCta = Form<Geo, NC, NP, KB>::kCtaChains;
   extern __shared__ __align__(16) uint8_t smem[];
   const int per_chunk = L.nt / kCta;
   const batch::ChunkDev ch = L.chunks[L.chunk0 + blockIdx.x / per_chunk];
@@ -35,20 +35,20 @@ __global__ void __launch_bounds__(Form<Geo, NC, NP>::kThreads, kMinCtas<NP>)
   for (int j = 0; j < 4; ++j) tab.W[j] = ch.W[j];
   tab.err = sg.code.err;
   const core::ChainOut out{sg.chain_E, nullptr, nullptr, nullptr};
-  anneal_coop_cta<Geo, NC, NP>(sg.init, sg.shot0 * (uint64_t)sg.restarts * 4u, (int64_t)ch.first_chain + first,
+  anneal_coop_cta<Geo, NC, NP, KB>(sg.init, sg.shot0 * (uint64_t)sg.restarts * 4u, (int64_t)ch.first_chain + first,
                              min(kCta, ch.n_chains - first), out, tab, L.keys, smem);
 }
 
-template <class Geo, int NC, int NP>
+template <class Geo, int NC, int NP, int KB>
 xzzx_status chunks_form(const batch::CoopLaunch& L, cudaStream_t stream) {
-  using F = Form<Geo, NC, NP>;
+  using F = Form<Geo, NC, NP, KB>;
   static DeviceOnce once;
-  xzzx_status st = once.run([] { return allow_shared(coop_chunks_kernel<Geo, NC, NP>); });
+  xzzx_status st = once.run([] { return allow_shared(coop_chunks_kernel<Geo, NC, NP, KB>); });
   if (st) return st;
   const size_t smem = std::max(F::smem_bytes(L.n_classes), (size_t)std::max(L.smem, 0));
   const int64_t grid = (int64_t)L.n_chunks * (L.nt / F::kCtaChains);
   if (grid > 0x7FFFFFFF) return fail(XZZX_EINVAL, "too many chains for one launch");
-  coop_chunks_kernel<Geo, NC, NP><<<(unsigned)grid, F::kThreads, smem, stream>>>(L);
+  coop_chunks_kernel<Geo, NC, NP, KB><<<(unsigned)grid, F::kThreads, smem, stream>>>(L);
   XZZX_CUDA_TRY(cudaGetLastError());
   return XZZX_OK;
 }
@@ -59,14 +59,16 @@ xzzx_status chunks_g(const batch::CoopLaunch& L, cudaStream_t stream) {
   xzzx_status st = sm_count(&n_sm);
   if (st) return st;
   // An occupancy cap (L.smem) is one of the plain form's CTAs.
-  return L.smem == 0 && producing<Geo>((int64_t)L.n_chunks * L.nt, n_sm) ? chunks_form<Geo, 1, 3>(L, stream)
-                                                                       : chunks_form<Geo, 4, 0>(L, stream);
+  const int kb = L.smem == 0 ? producing_kb<Geo>((int64_t)L.n_chunks * L.nt, n_sm) : 0;
+  return kb == 72   ? chunks_form<Geo, 1, 3, 72>(L, stream)
+         : kb == 52 ? chunks_form<Geo, 1, 3, 52>(L, stream)
+                    : chunks_form<Geo, 4, 0, 72>(L, stream);
 }
 
 template <class Geo>
 xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm) {
-  using F = Form<Geo, 4, 0>;
-  xzzx_status st = allow_shared(coop_chunks_kernel<Geo, 4, 0>);
+  using F = Form<Geo, 4, 0, 72>;
+  xzzx_status st = allow_shared(coop_chunks_kernel<Geo, 4, 0, 72>);
   if (st) return st;
   size_t smem = F::smem_bytes(n_classes);
   int dev = 0, per_sm_bytes = 0, reserved = 0, optin = 0;
@@ -78,7 +80,7 @@ xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm)
     const long pad = ((long)per_sm_bytes / cap - reserved) & ~15L;
     smem = std::max(smem, (size_t)std::min<long>(pad, optin));
   }
-  XZZX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_chunks_kernel<Geo, 4, 0>, F::kThreads, smem));
+  XZZX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_chunks_kernel<Geo, 4, 0, 72>, F::kThreads, smem));
   *smem_out = cap > 0 ? (int)smem : 0;
   return XZZX_OK;
 }
@@ -90,16 +92,22 @@ xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm)
 
 // Whether a launch of n_chains distance-d chains is faster with several lanes
 // per chain than with one thread per chain, whose time is that of one chain's
-// sweeps until its warps fill the GPU.  One thread / this kernel, ms, 400 sweeps
-// at p = 0.15, eta = 100: 0.71 / 0.47 at d = 5 and 3.75 / 2.04 at d = 15 for
-// 16,384 chains, 0.71 / 0.81 and 3.74 / 3.67 for 32,768; 3.45 / 2.10 at d = 17
-// and 10.3 / 4.4 at d = 31 for 8,192 chains, 3.47 / 4.03 and 10.3 / 8.3 for
-// 16,384 (a pair of rows per lane leaves up to 7 of 16 lanes idle at d >= 17).
+// sweeps until its warps fill the GPU.  The lanes' throughput is in proportion to
+// the share of them that hold rows, (d+1)/2 of a power of two.  One thread / this
+// kernel at 80, 120, 144, 180, 220 chains per SM (200 sweeps, p = 0.15, eta = 100):
+// d = 5 1.51, 1.36, 1.22, 0.93, 0.81; d = 7 1.81, 1.49, 1.49, 1.09, 0.94; d = 9 1.29, 1.07,
+// 1.00, 0.89, 0.73; d = 11 1.32, 1.12, 1.06, 0.93, 0.76; d = 15 1.52, 1.31, 1.29, 1.13, 0.93;
+// d = 17 1.28, 0.91, 0.99, 0.83; d = 25 1.44, 1.00, 1.26, 1.03; d = 31 1.66, 1.16, 1.44, 1.18;
+// d = 3 1.42, 1.41, 1.31, 1.31, 1.18, and 1.13 at 300 (its thread kernel spends a quarter
+// of a sweep on the table of thresholds).
 xzzx_status coop_is_faster(int d, int64_t n_chains, bool* yes) {
   int n_sm = 0;
   xzzx_status st = coop::sm_count(&n_sm);
   if (st) return st;
-  *yes = n_chains <= (int64_t)n_sm * (d <= 15 ? 144 : 80);
+  const int pairs = (d + 1) / 2;
+  int lanes = 2;
+  while (lanes < pairs) lanes *= 2;
+  *yes = n_chains <= (int64_t)n_sm * (d == 3 ? 280 : (d <= 15 ? 200 : 165) * pairs / lanes);
   return XZZX_OK;
 }
 

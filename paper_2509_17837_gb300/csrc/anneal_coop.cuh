@@ -523,14 +523,14 @@ struct PlanarLanes : LaneShape<D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 16 : 32, (D -
 // NP > 0: the producing warps draw every block of the next kSweeps sweeps and
 // write their tables while the sweeping warps run the current ones from shared
 // memory (two sets of each).
-template <class Geo, int NC, int NP>
+template <class Geo, int NC, int NP, int KB = 72>
 struct Form {
   static constexpr int kThreads = 32 * (NC + NP);
   static constexpr int kCtaChains = NC * Geo::kChains;
   static constexpr int kSets = NP ? 2 : 1;
-  // sweeps per set: as many as keep them within 72 KB (three CTAs per SM)
+  // sweeps per set: as many as keep them within KB kilobytes (72: three CTAs per SM, 52: four)
   static constexpr int kDrawBytes = NP ? NC * Geo::kBatches * kBatchWords * 4 : 0;
-  static constexpr int kFit = 72 * 1024 / (kSets * ((int)Geo::kTable + kDrawBytes));
+  static constexpr int kFit = KB * 1024 / (kSets * ((int)Geo::kTable + kDrawBytes));
   static constexpr int kSweeps = kFit >= 8 ? 8 : kFit >= 4 ? 4 : kFit >= 2 ? 2 : 1;
   static constexpr int kDrawWords = NP ? kSets * kSweeps * NC * Geo::kBatches * kBatchWords
                                        : NC * 2 * kBatchWords;
@@ -545,12 +545,12 @@ struct Form {
 
 // What a producing warp does for one set of sweeps [t0, t0 + ns): the draws of
 // every sweeping warp and the thresholds of the tables.
-template <class Geo, int NC, int NP>
+template <class Geo, int NC, int NP, int KB = 72>
 __device__ __forceinline__ void produce(int t0, int ns, const core::SaDraws (&base)[NC], const core::SweepTables& tab,
                                         const PhiloxKeys& K, uint32_t tables, const uint32_t* upd, int n_upd,
                                         uint32_t* draws, int pw, int lane) {
   const int k = lane & (Geo::G - 1);
-  constexpr int kSweeps = Form<Geo, NC, NP>::kSweeps;
+  constexpr int kSweeps = Form<Geo, NC, NP, KB>::kSweeps;
   for (int j = pw * 32 + lane; j < n_upd; j += NP * 32) {
     const uint32_t v = upd[j], a = tables + 8u * (v >> 16) + 4u;
     const uint32_t* T = tab.T + (size_t)t0 * tab.n_classes + (v & 0xFFFFu);
@@ -581,11 +581,11 @@ __device__ __forceinline__ void produce(int t0, int ns, const core::SaDraws (&ba
 // Anneal the n_chains (1 to kCtaChains) chains of a segment from chain first by
 // one CTA.  chain0, init0 and out0 are those of the segment's chain 0; groups
 // past n_chains run a copy of the last chain and write nothing.  smem: Form::smem_bytes(tab.n_classes) bytes.
-template <class Geo, int NC, int NP>
+template <class Geo, int NC, int NP, int KB = 72>
 __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ init0, uint64_t chain0, int64_t first,
                                                 int n_chains, const core::ChainOut& out0, const core::SweepTables& tab,
                                                 const PhiloxKeys& K, uint8_t* smem) {
-  using F = Form<Geo, NC, NP>;
+  using F = Form<Geo, NC, NP, KB>;
   constexpr int G = Geo::G, NW = Geo::NW, W = Geo::kW, kSweeps = F::kSweeps;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = lane & (G - 1);
   const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
@@ -605,13 +605,14 @@ __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ ini
   // where no draw can accept) follow per set of sweeps.
   if (tid == 0) n_upd_s[0] = 0;
   __syncthreads();
+  static_assert(kEntries % F::kThreads == 0, "whole warps in every pass");
   for (int e = tid; e < kEntries; e += F::kThreads) {
     const int src = Geo::sig_source(e);
     const int2 sg = src >= 0 ? __ldg(&tab.sig[src]) : make_int2(1, -1);
 #pragma unroll
     for (int s = 0; s < F::kSets * kSweeps; ++s)
       core::sts_u2(tables + (uint32_t)s * Geo::kTable + 8u * (uint32_t)e, make_uint2((uint32_t)sg.x, 0u));
-    if (sg.y >= 0) upd[atomicAdd(n_upd_s, 1)] = ((uint32_t)e << 16) | (uint32_t)sg.y;
+    core::append_entry(sg.y >= 0, ((uint32_t)e << 16) | (uint32_t)sg.y, upd, n_upd_s);
   }
   __syncthreads();
   const int n_upd = n_upd_s[0];
@@ -624,7 +625,7 @@ __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ ini
       base[w].init((uint32_t)ch, kTagSA | ((uint32_t)(ch >> 32) << 8), K);
     }
     for (int t0 = 0, set = 0; t0 < n_live; t0 += kSweeps, set ^= 1) {
-      produce<Geo, NC, NP>(t0, min(kSweeps, n_live - t0), base, tab, K, tables + (uint32_t)(set * kSweeps) * kTable, upd,
+      produce<Geo, NC, NP, KB>(t0, min(kSweeps, n_live - t0), base, tab, K, tables + (uint32_t)(set * kSweeps) * kTable, upd,
                            n_upd, draws + set * (F::kDrawWords / 2), warp - NC, lane);
       __syncthreads();
     }

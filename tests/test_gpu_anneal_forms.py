@@ -21,7 +21,7 @@ def test_thread_and_lane_forms_agree(env, d):
     X, torch = env
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
     restarts = 37  # 148 chains per shot: ragged warps and CTAs in every form
-    shots = (144 * n_sm) // (4 * restarts) + 2  # past the lane forms' range at every distance
+    shots = (280 * n_sm) // (4 * restarts) + 2  # past the lane forms' range at every distance
     code, noise = X.Code(d), X.noise_from_eta(0.17, 10.0)
     sched = X.Schedule(noise, 11, 0.05, 3.0)  # 11 sweeps: a partial set of tables
     _, syn = X.sample_errors(code, noise, 5, 7, shots)
@@ -67,7 +67,7 @@ def test_stopping_in_the_frozen_sweeps_changes_no_minimum(env, d, eta):
     X, torch = env
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
     restarts = 32
-    shots = (144 * n_sm) // (4 * restarts) + 1
+    shots = (280 * n_sm) // (4 * restarts) + 1
     code, noise = X.Code(d), X.noise_from_eta(0.15, eta)
     sched = X.Schedule(noise, 150, 0.1, 60.0)  # frozen from about a fifth of the sweeps
     _, T = sched.table()
