@@ -26,12 +26,8 @@ struct AnnealArgs {
   uint32_t* err;
 };
 
-// One chain per thread.  The pair path (d <= 15) is bounded to four 256-thread
-// CTAs per SM (64 registers); the row path keeps the compiler's choice for
-// 128-thread CTAs (about 120 registers up to d = 29, 160 at d = 31).
-template <int D>
+template <int D, int NT>
 __device__ __forceinline__ void anneal_body(const AnnealArgs& A) {
-  constexpr int NT = Shape<D>::kThreads;
   constexpr int W = Shape<D>::kW;
   extern __shared__ __align__(16) uint8_t smem[];
   const int64_t c_raw = (int64_t)blockIdx.x * NT + threadIdx.x;
@@ -54,43 +50,51 @@ __device__ __forceinline__ void anneal_body(const AnnealArgs& A) {
                     A.keys, smem);
 }
 
+// One chain per thread.  Full launches: 256-thread CTAs held to 64 registers (four
+// per SM) up to d = 15, 128-thread CTAs held to 128 registers (four per SM) above;
+// more chains in flight hide the sweep's dependent integer chain better than more
+// registers do.
 template <int D>
 __global__ void __launch_bounds__(Shape<D>::kThreads, 4) anneal_kernel(const __grid_constant__ AnnealArgs A) {
-  anneal_body<D>(A);
+  anneal_body<D, Shape<D>::kThreads>(A);
 }
+// Launches of up to 12 warps per SM at d <= 15, one warp per CTA: with wide CTAs
+// some SMs would hold one CTA more than others, or none (290 to 384 chains per SM:
+// 0.38 -> 0.32 ms at d = 5, 1.47 -> 1.21 ms at d = 11, 2.62 -> 2.09 ms at d = 15; 700 per
+// SM: 5 to 9% slower).  At d >= 17, with four-warp CTAs, it makes no difference.
+constexpr int kNarrowWarps = 12, kNarrowMaxD = 15;
 template <int D>
-__global__ void __launch_bounds__(Shape<D>::kThreads) anneal_kernel_rows(const __grid_constant__ AnnealArgs A) {
-  anneal_body<D>(A);
-}
-// d >= 29: held to 128 registers, four CTAs per SM instead of three (the
-// compiler's own choice is about 158); more chains in flight hide the sweep's
-// dependent integer chain better than the extra registers do.
-template <int D>
-__global__ void __launch_bounds__(Shape<D>::kThreads, 4) anneal_kernel_rows4(const __grid_constant__ AnnealArgs A) {
-  anneal_body<D>(A);
-}
-template <int D>
-constexpr auto anneal_kernel_of() {
-  if constexpr (D <= kPairMaxD) return &anneal_kernel<D>;
-  else if constexpr (D >= 29) return &anneal_kernel_rows4<D>;
-  else return &anneal_kernel_rows<D>;
+__global__ void __launch_bounds__(32, kNarrowWarps) anneal_narrow_kernel(const __grid_constant__ AnnealArgs A) {
+  anneal_body<D, 32>(A);
 }
 
-template <int D>
-xzzx_status launch_d(const AnnealArgs& A, cudaStream_t stream) {
-  constexpr int NT = Shape<D>::kThreads;
-  const size_t smem = smem_bytes<D, NT>();
-  static DeviceOnce once;
+template <int NT, typename F>
+xzzx_status launch_kernel(F kernel, DeviceOnce& once, size_t smem, const AnnealArgs& A, cudaStream_t stream) {
   xzzx_status st = once.run([&]() -> xzzx_status {
-    XZZX_CUDA_TRY(cudaFuncSetAttribute(anneal_kernel_of<D>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    XZZX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return XZZX_OK;
   });
   if (st) return st;
   const int64_t grid = (A.n_chains + NT - 1) / NT;
   if (grid > 0x7FFFFFFF) return fail(XZZX_EINVAL, "too many chains for one launch");
-  anneal_kernel_of<D>()<<<(unsigned)grid, NT, smem, stream>>>(A);
+  kernel<<<(unsigned)grid, NT, smem, stream>>>(A);
   XZZX_CUDA_TRY(cudaGetLastError());
   return XZZX_OK;
+}
+
+template <int D>
+xzzx_status launch_d(const AnnealArgs& A, cudaStream_t stream) {
+  constexpr int NT = Shape<D>::kThreads;
+  static DeviceOnce once;
+  if constexpr (D <= kNarrowMaxD) {
+    static DeviceOnce once_narrow;
+    int dev = 0, n_sm = 0;
+    XZZX_CUDA_TRY(cudaGetDevice(&dev));
+    XZZX_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    if (A.n_chains <= (int64_t)32 * kNarrowWarps * n_sm)
+      return launch_kernel<32>(anneal_narrow_kernel<D>, once_narrow, smem_bytes<D, 32>(), A, stream);
+  }
+  return launch_kernel<NT>(anneal_kernel<D>, once, smem_bytes<D, NT>(), A, stream);
 }
 
 }  // namespace

@@ -35,6 +35,23 @@ def test_thread_and_lane_forms_agree(env, d):
         assert torch.equal(thread[k][:1], few[k]), k
 
 
+@pytest.mark.parametrize("d", range(3, 16, 2))
+def test_one_warp_and_wide_ctas_agree(env, d):
+    """One thread per chain: CTAs of one warp up to 384 chains per SM, wide ones above."""
+    X, torch = env
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    restarts = 37
+    wide, narrow = (384 * n_sm) // (4 * restarts) + 1, (384 * n_sm) // (4 * restarts)
+    code, noise = X.Code(d), X.noise_from_eta(0.17, 10.0)
+    sched = X.Schedule(noise, 11, 0.05, 3.0)
+    _, syn = X.sample_errors(code, noise, 5, 7, wide)
+    init, _ = X.greedy_init(code, noise, 5, 7, syn, restarts)
+    kw = dict(want_cfg=True, want_final=True)
+    a, b = X.anneal(code, sched, 5, 7, init, **kw), X.anneal(code, sched, 5, 7, init[:narrow].contiguous(), **kw)
+    for k in a:
+        assert torch.equal(a[k][:narrow], b[k]), k
+
+
 @pytest.mark.parametrize("d", range(3, 32, 2))
 def test_planar_forms_agree(env, d):
     """On the planar lattice (d <= 15: one thread per chain, then several lanes;
