@@ -234,8 +234,8 @@ constexpr size_t reg_smem_bytes() {
 // Bound by the pipe of shifts and logic together with the wide multiplies of the
 // draws.  600 shots x 64 restarts, against three-row faces, a table rebuilt every
 // sweep and no frozen sweeps: 50 sweeps near the Nishimori temperature d = 9 1.65 ->
-// 1.53 ms, d = 15 5.58 -> 4.37 ms; 200 sweeps to 20 times it d = 9 4.95 -> 4.17 ms, d =
-// 15 18.7 -> 14.9 ms.  Held to seven CTAs per SM (72 registers) d = 9 takes 1.56 ms.
+// 1.49 ms, d = 15 5.58 -> 4.3 ms; 200 sweeps to 20 times it d = 9 4.95 -> 4.09 ms, d =
+// 15 18.7 -> 14.6 ms.  Held to seven CTAs per SM (72 registers) d = 9 takes 1.56 ms.
 template <int D>
 __global__ void __launch_bounds__(kRThreads, 1) anneal_planar_reg_kernel(const __grid_constant__ RegArgs A) {
   constexpr int G = PShape<D>::G;
