@@ -32,28 +32,44 @@ sys.path.insert(0, ROOT)
 D, ETA, PS, RESTARTS, SWEEPS, BETA0, BETA1, SCALE = 11, 100.0, (0.10, 0.13, 0.16, 0.19, 0.22), 64, 1000, 0.05, 20.0, 1024
 SEED = 0xD11
 I_ALG = 30  # integer instructions per move attempt in the algorithmic count
-# Counters of the current anneal_kernel<11> from one ncu capture (None until
-# the kernel has been captured since its last change): DRAM bytes (read +
-# write) per chain, ALU-pipe lane instructions per move attempt
+# Counters of anneal_kernel<11> from an ncu capture: DRAM bytes (read + write)
+# per chain, ALU-pipe lane instructions per move attempt
 # (sm__inst_executed_pipe_alu x 32 / attempts; the ALU pipe takes 16 lanes per
 # clock per SM sub-partition), all lane instructions per attempt
 # (smsp__inst_executed x 32 / attempts) and shared-memory bank conflicts per
-# shared wavefront.
-ANNEAL_DRAM_BYTES_PER_CHAIN = 8.399872e6 / 1.024e6
-ANNEAL_ALU_INST_PER_ATTEMPT = 12.12
-ANNEAL_MEASURED = {"inst_per_attempt": 20.51, "alu_inst_per_attempt": ANNEAL_ALU_INST_PER_ATTEMPT,
-                   "shared_bank_conflicts_per_wavefront": 1.2654e10 / 2.0863e10,
+# shared wavefront.  Attempts are those of the schedule; the warps whose chains
+# provably repeat stop in the frozen sweeps (thresholds all zero), so an executed
+# attempt costs more than these figures.
+ANNEAL_DRAM_BYTES_PER_CHAIN = 8.985344e6 / 1.024e6
+ANNEAL_ALU_INST_PER_ATTEMPT = 8.10
+ANNEAL_MEASURED = {"inst_per_attempt": 15.30, "alu_inst_per_attempt": ANNEAL_ALU_INST_PER_ATTEMPT,
+                   "shared_bank_conflicts_per_wavefront": 8.6816e9 / 1.42726e10,
                    "source": "ncu capture of one anneal_kernel<11> launch of 4000 shots, "
-                             "profiles/anneal_d11_ncu_full.md"}
-# The same counters for the d=31 row kernel of the large workload, taken on
-# its form before the group-by-group columns and the 128-register bound:
-# DRAM traffic is therefore not reported for the current kernel.
-ANNEAL_D31_DRAM_BYTES_PER_CHAIN = None
-ANNEAL_D31_MEASURED = {"inst_per_attempt": 18.83, "alu_inst_per_attempt": 11.69,
-                       "shared_bank_conflicts_per_wavefront": 5.7998e10 / 9.3272e10,
-                       "dram_bytes_per_chain": 4.580864e6 / (57 * 1024),
-                       "source": "ncu capture of one launch of the previous form of the d=31 row kernel "
-                                 "(158 registers, 3 CTAs per SM), profiles/anneal_d31_ncu_full.md"}
+                             "profiles/anneal_ncu_counters.md"}
+# The same counters for the d=31 row kernel of the large workload.
+ANNEAL_D31_DRAM_BYTES_PER_CHAIN = 5.614592e6 / (76 * 1024)
+ANNEAL_D31_MEASURED = {"inst_per_attempt": 15.95, "alu_inst_per_attempt": 9.91,
+                       "shared_bank_conflicts_per_wavefront": 3.2638e9 / 4.7895e9,
+                       "dram_bytes_per_chain": ANNEAL_D31_DRAM_BYTES_PER_CHAIN,
+                       "source": "ncu capture of one anneal_kernel<31> launch of 76 shots x 256 restarts x 500 "
+                                 "sweeps, profiles/anneal_ncu_counters.md"}
+ATTEMPTS_NOTE = ("attempts are those of the schedule; in its frozen sweeps (every acceptance threshold zero) a warp "
+                 "whose 32 chains have all returned to an earlier configuration stops, since no later sweep can "
+                 "change its minima; the roofline counts the attempts of the live sweeps only")
+
+
+def live_share(sched):
+    """Share of a schedule's sweeps up to the last with a threshold above zero."""
+    T = sched.table()[1]
+    live = [t for t in range(len(T)) if any(T[t])]
+    return (live[-1] + 1) / len(T) if live else 0.0
+
+
+def live_mean(segs):
+    """live_share of a batch's segments, weighted by their attempts."""
+    w = [len(sg["syndromes"]) * sg["restarts"] * sg["sched"].n_sweeps * sg["code"].n_stab for sg in segs]
+    share = {id(sg["sched"]): live_share(sg["sched"]) for sg in segs}
+    return sum(k * share[id(sg["sched"])] for k, sg in zip(w, segs)) / sum(w)
 
 
 def workload_config(shots_per_p, world):
@@ -163,11 +179,12 @@ def issue_peak(clocks, n_sm):
             "%d SMs x 4 SMSP x 32 lanes x %.0f MHz (median SM clock sampled in the timed region)" % (n_sm, f_mhz))
 
 
-def roofline_record(rate_attempts, clocks, n_sm, **extra):
+def roofline_record(rate_attempts, live, clocks, n_sm, **extra):
     peak, basis = issue_peak(clocks, n_sm)
-    achieved = rate_attempts * I_ALG / 1e12
+    achieved = rate_attempts * live * I_ALG / 1e12
     rec = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tinst/s",
-           "frac": (achieved / peak) if peak else None, "I_alg_per_attempt": I_ALG, "peak_basis": basis}
+           "frac": (achieved / peak) if peak else None, "I_alg_per_attempt": I_ALG, "live_share": live,
+           "attempts_note": ATTEMPTS_NOTE, "peak_basis": basis}
     rec.update(extra)
     return rec
 
@@ -459,7 +476,7 @@ def run_uneven(args):
                    "segments": info["n_segments"], "chunks": info["n_chunks"],
                    "tuned_cfg": form_rec("tuned")["cfg"],
                    "modes": "0 persistent (one chain per thread, chunk queue), 1 one launch per distance, 2 per "
-                            "distance with one warp per chain, 3 per-distance launches on forked streams, 4 one "
+                            "distance with several lanes per chain, 3 per-distance launches on forked streams, 4 one "
                             "persistent launch per distance class on forked streams; 0, 3 and 4 replayed as "
                             "captured CUDA graphs",
                    "autotune": {"batch_shots": int(sum(int(sg["syndromes"].shape[0]) for sg in tune_segs)),
@@ -469,7 +486,7 @@ def run_uneven(args):
         "move_attempts_per_s": att, "forms": {name: form_rec(name) for name in forms},
         "speedup_vs_plain": ms["plain"] / ms["tuned"], "identical_outputs": bool(same),
         "logical_failures": fails, "clocks": clocks,
-        "roofline": roofline_record(att, clocks, props.multi_processor_count, traffic=None,
+        "roofline": roofline_record(att, live_mean(segs), clocks, props.multi_processor_count, traffic=None,
                                     kernel="annealing launches of the tuned form (all distances)")}))
 
 
@@ -588,14 +605,14 @@ def run_large(args):
     att = shots * 4 * R * N * (d * d - 1) / (ms / 1e3)
     props = torch.cuda.get_device_properties(0)
 
-    # The same annealing launch (first p, step 1) with one warp per chain and
-    # colour-parallel lanes, against one thread per chain: identical chain
+    # The same annealing launch (first p, step 1) with several lanes per chain,
+    # against one thread per chain: identical chain
     # minima, and each mapping's rate.
     noise, sched, sd, err, syn = cases[0]
     init, _ = X.greedy_init(code, noise, sd, S, syn[S:2 * S], R)
     mapping = {}
     best = {}
-    for name, per_warp in (("thread_per_chain", False), ("warp_per_chain", True)):
+    for name, per_warp in (("thread_per_chain", False), ("lanes_per_chain", True)):
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(stream)
         a = X.anneal(code, sched, sd, S, init, want_cfg=False, per_warp=per_warp, stream=stream)
@@ -604,11 +621,11 @@ def run_large(args):
         best[name] = a["best_E"]
         mapping[name] = {"anneal_ms": e0.elapsed_time(e1),
                          "attempts_per_s": S * 4 * R * N * (d * d - 1) / (e0.elapsed_time(e1) / 1e3)}
-    mapping["identical_chain_minima"] = bool(torch.equal(best["thread_per_chain"], best["warp_per_chain"]))
+    mapping["identical_chain_minima"] = bool(torch.equal(best["thread_per_chain"], best["lanes_per_chain"]))
 
     # Occupancy sweep: the same shots with a given number of chains in flight
     # per SM (CTAs per SM x chains per CTA), one chain per thread as one
-    # persistent launch, then one chain per warp.  Decisions must equal the
+    # persistent launch, then several lanes per chain.  Decisions must equal the
     # plain decode of the same shots.
     ref = X.decode_batch(code, noise, sched, sd, S, syn[S:2 * S], R, true_errors=err[S:2 * S], stream=stream)
     occupancy = []
@@ -633,7 +650,7 @@ def run_large(args):
                               "attempts_per_s": info["move_attempts"] / (e0.elapsed_time(e1) / 1e3),
                               "identical_decisions": bool(same)})
             b.close()
-        # One warp per chain (mode 2, 4 chains per CTA): resident CTAs per SM
+        # Several lanes per chain (mode 2; 16 lanes at d=31, 8 chains per CTA): resident CTAs per SM
         # capped by padding each CTA's shared memory (0 = the register limit).
         for cps in (2, 4, 8, 0):
             seg = dict(code=code, noise=noise, sched=sched, shot0=S, syndromes=syn[S:2 * S], restarts=R,
@@ -647,8 +664,8 @@ def run_large(args):
             o = b.outputs[0]
             same = all(torch.equal(o[k], ref[k]) for k in ("cls", "E4", "recovery", "fail"))
             info = b.info()
-            occupancy.append({"mapping": "warp_per_chain", "chains_per_cta": 4, "ctas_per_sm_cap": cps,
-                              "chains_in_flight_per_sm": 4 * info["warp_ctas_per_sm"],
+            occupancy.append({"mapping": "lanes_per_chain", "chains_per_cta": 8, "ctas_per_sm_cap": cps,
+                              "chains_in_flight_per_sm": 8 * info["warp_ctas_per_sm"],
                               "ms": e0.elapsed_time(e1),
                               "attempts_per_s": info["move_attempts"] / (e0.elapsed_time(e1) / 1e3),
                               "identical_decisions": bool(same)})
@@ -663,10 +680,10 @@ def run_large(args):
         "shots_per_s": shots / (ms / 1e3), "shots_timed": shots * args.steps,
         "logical_error_rates": [stats.ler_record(p, f, S * args.steps) for p, f in zip(LARGE_PS, fails)],
         "chain_mapping": mapping, "occupancy_sweep": occupancy, "clocks": clocks,
-        "roofline": roofline_record(att, clocks, props.multi_processor_count,
+        "roofline": roofline_record(att, statistics.fmean(live_share(c[1]) for c in cases), clocks, props.multi_processor_count,
                                     traffic=(None if ANNEAL_D31_DRAM_BYTES_PER_CHAIN is None
                                              else ANNEAL_D31_DRAM_BYTES_PER_CHAIN * S * R * 4),
-                                    kernel="anneal_kernel_rows4<31>", measured_per_attempt=ANNEAL_D31_MEASURED)}))
+                                    kernel="anneal_kernel<31>", measured_per_attempt=ANNEAL_D31_MEASURED)}))
 
 
 # --------------------------------------------------------------------------- logical error rate curves
@@ -903,7 +920,7 @@ def main():
         n_sm = props.multi_processor_count
         f_mhz = (clocks or {}).get("sm_mhz")
         roof = roofline_record(
-            anneal_rate, clocks, n_sm,
+            anneal_rate, statistics.fmean(live_share(c["sched"]) for c in cases), clocks, n_sm,
             traffic=None if ANNEAL_DRAM_BYTES_PER_CHAIN is None else ANNEAL_DRAM_BYTES_PER_CHAIN * S * RESTARTS * 4,
             kernel="anneal_kernel<11>",
             measured_per_attempt=ANNEAL_MEASURED,
