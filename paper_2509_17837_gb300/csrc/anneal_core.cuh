@@ -861,7 +861,7 @@ __device__ __forceinline__ void anneal_cta_rows(const uint32_t* __restrict__ ini
 }
 
 // Pair path.  Arguments as anneal_cta.
-template <int D, int NT, int U>
+template <int D, int NT, int U, bool KEEP>
 __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ init, uint64_t chain, int P_coset,
                                                  bool active, const ChainOut& out, const SweepTables& tab,
                                                  const PhiloxKeys& K, uint8_t* smem) {
@@ -906,17 +906,19 @@ __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ in
   int32_t E_best = E;
   uint32_t P[H][NW];
   rows_to_pairs<D, Row>(R, P);
+  auto put = [&] {  // the pair words into the chain's place in shared memory
 #pragma unroll
-  for (int j = 0; j < H; ++j)
+    for (int j = 0; j < H; ++j)
 #pragma unroll
-    for (int k = 0; k < NW; ++k) best[(j * NW + k) * NT + tid] = P[j][k];
+      for (int k = 0; k < NW; ++k) best[(j * NW + k) * NT + tid] = P[j][k];
+  };
+  if (KEEP) put();
   __syncwarp();
 
-#define XZZX_SNAPSHOT                                                                         \
-  if (E < E_best) {                                                                           \
-    E_best = E;                                                                               \
-    _Pragma("unroll") for (int j = 0; j < H; ++j)                                             \
-    _Pragma("unroll") for (int k = 0; k < NW; ++k) best[(j * NW + k) * NT + tid] = P[j][k];   \
+#define XZZX_SNAPSHOT   \
+  if (E < E_best) {     \
+    E_best = E;         \
+    if (KEEP) put();    \
   }
 #define XZZX_SWEEP(LIVE)                            \
   pair_phase<D, 0, LIVE>(P, E, Lb, dr, K, tab.err); \
@@ -942,16 +944,25 @@ __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ in
       __syncwarp();
     }
   }
-  // The frozen sweeps (see above).
-  uint32_t saved[H][NW];
+  // The frozen sweeps (see above).  Where no minimum is kept (KEEP = false) the
+  // saved configuration takes its place: in registers it made the persistent
+  // kernels, several distances under one bound, spill 264 to 504 bytes (batch mode
+  // 0, 4 shots x 32 restarts x 150 sweeps, ms, in registers / here: d = 11 0.81 /
+  // 0.57; d = 17, 21 2.83 / 2.00; d = 5 to 31 7.20 / 3.42; 250 shots each of d = 5 to
+  // 21 89 / 80).
+  uint32_t saved[KEEP ? H : 1][KEEP ? NW : 1];
   const bool may_stop = !out.final_E && !out.final_cfg;
   bool done = false;
   for (int t = n_live, i = 0; t < n_sweeps; ++t, ++i) {
     if ((i & (i + 1)) == 0) {
+      if constexpr (KEEP) {
 #pragma unroll
-      for (int j = 0; j < H; ++j)
+        for (int j = 0; j < H; ++j)
 #pragma unroll
-        for (int k = 0; k < NW; ++k) saved[j][k] = P[j][k];
+          for (int k = 0; k < NW; ++k) saved[j][k] = P[j][k];
+      } else {
+        put();
+      }
     }
     XZZX_SWEEP(false)
     if (may_stop) {
@@ -959,7 +970,7 @@ __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ in
 #pragma unroll
       for (int j = 0; j < H; ++j)
 #pragma unroll
-        for (int k = 0; k < NW; ++k) diff |= P[j][k] ^ saved[j][k];
+        for (int k = 0; k < NW; ++k) diff |= P[j][k] ^ (KEEP ? saved[KEEP ? j : 0][KEEP ? k : 0] : best[(j * NW + k) * NT + tid]);
       done |= diff == 0u;
       if (__all_sync(0xFFFFFFFFu, done)) break;
     }
@@ -974,7 +985,7 @@ __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ in
     pairs_to_rows<D, Row>(P, R);
     store_rows<D, Row>(R, out.final_cfg);
   }
-  if (out.best_cfg) {
+  if (KEEP && out.best_cfg) {
 #pragma unroll
     for (int j = 0; j < H; ++j)
 #pragma unroll
@@ -989,12 +1000,14 @@ __device__ __forceinline__ void anneal_cta_pairs(const uint32_t* __restrict__ in
 // chain: global chain id (Philox counter); P: coset index of L_P; inactive
 // threads run a copy of a real chain and write nothing.  smem: smem_bytes<D,
 // NT>() bytes of dynamic shared memory.  U: unroll factor of the sweep loop
-// (a tuning knob; results do not depend on it).
-template <int D, int NT, int U = 1>
+// (a tuning knob; results do not depend on it).  KEEP = false: out.best_cfg is
+// null and the minimum's configuration is not kept (the row path looks at the
+// pointer instead).
+template <int D, int NT, int U = 1, bool KEEP = true>
 __device__ __forceinline__ void anneal_cta(const uint32_t* __restrict__ init, uint64_t chain, int P, bool active,
                                            const ChainOut& out, const SweepTables& tab, const PhiloxKeys& K,
                                            uint8_t* smem) {
-  if constexpr (D <= kPairMaxD) anneal_cta_pairs<D, NT, U>(init, chain, P, active, out, tab, K, smem);
+  if constexpr (D <= kPairMaxD) anneal_cta_pairs<D, NT, U, KEEP>(init, chain, P, active, out, tab, K, smem);
   else anneal_cta_rows<D, NT, U>(init, chain, P, active, out, tab, K, smem);
 }
 

@@ -35,7 +35,7 @@ __device__ __forceinline__ void run_chunk(const ChunkDev& ch, const SegDev& sg, 
   out.best_cfg = nullptr;
   out.final_E = nullptr;
   out.final_cfg = nullptr;
-  core::anneal_cta<D, NT, U>(sg.init + (size_t)(c >> 2) * 2 * W, chain, (int)(c & 3), active, out, tab, K, smem);
+  core::anneal_cta<D, NT, U, false>(sg.init + (size_t)(c >> 2) * 2 * W, chain, (int)(c & 3), active, out, tab, K, smem);
 }
 
 // Threads per SM that a kernel of distances up to D is register-bounded for: 1024
