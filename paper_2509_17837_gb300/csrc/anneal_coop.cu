@@ -16,10 +16,10 @@ namespace {
 
 // Batched form: the chunks of one distance, each cut into CTAs of kCtaChains
 // chains (so a CTA's chains share a segment and its thresholds).
-template <class Geo, int NC, int NP, int KB>
-__global__ void __launch_bounds__(Form<Geo, NC, NP, KB>::kThreads, kMinCtas<NP, KB>)
+template <class Geo, int NC, int NP, int PER>
+__global__ void __launch_bounds__(Form<Geo, NC, NP, PER>::kThreads, PER)
     coop_chunks_kernel(const __grid_constant__ batch::CoopLaunch L) {
-  constexpr int kCta = Form<Geo, NC, NP, KB>::kCtaChains;
+  constexpr int kCta = Form<Geo, NC, NP, PER>::kCtaChains;
   extern __shared__ __align__(16) uint8_t smem[];
   const int per_chunk = L.nt / kCta;
   const batch::ChunkDev ch = L.chunks[L.chunk0 + blockIdx.x / per_chunk];
@@ -35,20 +35,20 @@ __global__ void __launch_bounds__(Form<Geo, NC, NP, KB>::kThreads, kMinCtas<NP, 
   for (int j = 0; j < 4; ++j) tab.W[j] = ch.W[j];
   tab.err = sg.code.err;
   const core::ChainOut out{sg.chain_E, nullptr, nullptr, nullptr};
-  anneal_coop_cta<Geo, NC, NP, KB>(sg.init, sg.shot0 * (uint64_t)sg.restarts * 4u, (int64_t)ch.first_chain + first,
+  anneal_coop_cta<Geo, NC, NP, PER>(sg.init, sg.shot0 * (uint64_t)sg.restarts * 4u, (int64_t)ch.first_chain + first,
                              min(kCta, ch.n_chains - first), out, tab, L.keys, smem);
 }
 
-template <class Geo, int NC, int NP, int KB>
+template <class Geo, int NC, int NP, int PER>
 xzzx_status chunks_form(const batch::CoopLaunch& L, cudaStream_t stream) {
-  using F = Form<Geo, NC, NP, KB>;
+  using F = Form<Geo, NC, NP, PER>;
   static DeviceOnce once;
-  xzzx_status st = once.run([] { return allow_shared(coop_chunks_kernel<Geo, NC, NP, KB>); });
+  xzzx_status st = once.run([] { return allow_shared(coop_chunks_kernel<Geo, NC, NP, PER>); });
   if (st) return st;
   const size_t smem = std::max(F::smem_bytes(L.n_classes), (size_t)std::max(L.smem, 0));
   const int64_t grid = (int64_t)L.n_chunks * (L.nt / F::kCtaChains);
   if (grid > 0x7FFFFFFF) return fail(XZZX_EINVAL, "too many chains for one launch");
-  coop_chunks_kernel<Geo, NC, NP, KB><<<(unsigned)grid, F::kThreads, smem, stream>>>(L);
+  coop_chunks_kernel<Geo, NC, NP, PER><<<(unsigned)grid, F::kThreads, smem, stream>>>(L);
   XZZX_CUDA_TRY(cudaGetLastError());
   return XZZX_OK;
 }
@@ -59,16 +59,16 @@ xzzx_status chunks_g(const batch::CoopLaunch& L, cudaStream_t stream) {
   xzzx_status st = sm_count(&n_sm);
   if (st) return st;
   // An occupancy cap (L.smem) is one of the plain form's CTAs.
-  const int kb = L.smem == 0 ? producing_kb<Geo>((int64_t)L.n_chunks * L.nt, n_sm) : 0;
-  return kb == 72   ? chunks_form<Geo, 1, 3, 72>(L, stream)
-         : kb == 52 ? chunks_form<Geo, 1, 3, 52>(L, stream)
-                    : chunks_form<Geo, 4, 0, 72>(L, stream);
+  const int per = L.smem == 0 ? producing_per_sm<Geo>((int64_t)L.n_chunks * L.nt, n_sm) : 0;
+  return per == 3   ? chunks_form<Geo, 1, 3, 3>(L, stream)
+         : per == 4 ? chunks_form<Geo, 1, 3, 4>(L, stream)
+                    : chunks_form<Geo, 4, 0, 4>(L, stream);
 }
 
 template <class Geo>
 xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm) {
-  using F = Form<Geo, 4, 0, 72>;
-  xzzx_status st = allow_shared(coop_chunks_kernel<Geo, 4, 0, 72>);
+  using F = Form<Geo, 4, 0, 4>;
+  xzzx_status st = allow_shared(coop_chunks_kernel<Geo, 4, 0, 4>);
   if (st) return st;
   size_t smem = F::smem_bytes(n_classes);
   int dev = 0, per_sm_bytes = 0, reserved = 0, optin = 0;
@@ -80,7 +80,7 @@ xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm)
     const long pad = ((long)per_sm_bytes / cap - reserved) & ~15L;
     smem = std::max(smem, (size_t)std::min<long>(pad, optin));
   }
-  XZZX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_chunks_kernel<Geo, 4, 0, 72>, F::kThreads, smem));
+  XZZX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_chunks_kernel<Geo, 4, 0, 4>, F::kThreads, smem));
   *smem_out = cap > 0 ? (int)smem : 0;
   return XZZX_OK;
 }

@@ -522,35 +522,41 @@ struct PlanarLanes : LaneShape<D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 16 : 32, (D -
 // need, and the CTA rebuilds the tables of the next kSweeps sweeps together.
 // NP > 0: the producing warps draw every block of the next kSweeps sweeps and
 // write their tables while the sweeping warps run the current ones from shared
-// memory (two sets of each).
-template <class Geo, int NC, int NP, int KB = 72>
+// memory (two sets of each).  PER: the CTAs that an SM holds at once, which the
+// sweeps per set and the launch's register bound are chosen for.
+constexpr size_t kSmShared = 228 * 1024, kCtaReserved = 1024;  // shared memory of an SM; taken by the system per CTA
+template <class Geo, int NC, int NP, int PER>
 struct Form {
-  static constexpr int kThreads = 32 * (NC + NP);
+  static constexpr int kThreads = 32 * (NC + NP), kPerSm = PER;
   static constexpr int kCtaChains = NC * Geo::kChains;
   static constexpr int kSets = NP ? 2 : 1;
-  // sweeps per set: as many as keep them within KB kilobytes (72: three CTAs per SM, 52: four)
-  static constexpr int kDrawBytes = NP ? NC * Geo::kBatches * kBatchWords * 4 : 0;
-  static constexpr int kFit = KB * 1024 / (kSets * ((int)Geo::kTable + kDrawBytes));
-  static constexpr int kSweeps = kFit >= 8 ? 8 : kFit >= 4 ? 4 : kFit >= 2 ? 2 : 1;
-  static constexpr int kDrawWords = NP ? kSets * kSweeps * NC * Geo::kBatches * kBatchWords
-                                       : NC * 2 * kBatchWords;
+  static constexpr int draw_words(int sweeps) {
+    return NP ? kSets * sweeps * NC * Geo::kBatches * kBatchWords : NC * 2 * kBatchWords;
+  }
   // Dynamic shared memory: alignment slack, the tables, the list of entries
   // with a threshold, the draws, the output staging of each chain and, for NP =
-  // 0, the raw thresholds of the next kSweeps sweeps.
-  static constexpr size_t smem_bytes(int n_classes) {
-    return 2048 + (size_t)kSets * kSweeps * Geo::kTable + Geo::kEntries * sizeof(uint32_t) + 16 + (size_t)kDrawWords * 4 +
-           (size_t)kCtaChains * 2 * Geo::kW * 4 + (NP ? 0 : (size_t)kSweeps * n_classes * 4);
+  // 0, the raw thresholds of the next set's sweeps.
+  static constexpr size_t bytes(int sweeps, int n_classes) {
+    return 2048 + (size_t)kSets * sweeps * Geo::kTable + Geo::kEntries * sizeof(uint32_t) + 16 +
+           (size_t)draw_words(sweeps) * 4 + (size_t)kCtaChains * 2 * Geo::kW * 4 +
+           (NP ? 0 : (size_t)sweeps * n_classes * 4);
   }
+  // PER CTAs fit on an SM (NP = 0: with schedules of up to 128 thresholds).
+  static constexpr bool fits(int sweeps) { return PER * (bytes(sweeps, 128) + kCtaReserved) <= kSmShared; }
+  static constexpr int kSweeps = fits(8) ? 8 : fits(4) ? 4 : fits(2) ? 2 : 1;
+  static_assert(fits(kSweeps), "the CTAs that the launch rules count on do not fit");
+  static constexpr int kDrawWords = draw_words(kSweeps);
+  static constexpr size_t smem_bytes(int n_classes) { return bytes(kSweeps, n_classes); }
 };
 
 // What a producing warp does for one set of sweeps [t0, t0 + ns): the draws of
 // every sweeping warp and the thresholds of the tables.
-template <class Geo, int NC, int NP, int KB = 72>
+template <class Geo, int NC, int NP, int PER>
 __device__ __forceinline__ void produce(int t0, int ns, const core::SaDraws (&base)[NC], const core::SweepTables& tab,
                                         const PhiloxKeys& K, uint32_t tables, const uint32_t* upd, int n_upd,
                                         uint32_t* draws, int pw, int lane) {
   const int k = lane & (Geo::G - 1);
-  constexpr int kSweeps = Form<Geo, NC, NP, KB>::kSweeps;
+  constexpr int kSweeps = Form<Geo, NC, NP, PER>::kSweeps;
   for (int j = pw * 32 + lane; j < n_upd; j += NP * 32) {
     const uint32_t v = upd[j], a = tables + 8u * (v >> 16) + 4u;
     const uint32_t* T = tab.T + (size_t)t0 * tab.n_classes + (v & 0xFFFFu);
@@ -581,11 +587,11 @@ __device__ __forceinline__ void produce(int t0, int ns, const core::SaDraws (&ba
 // Anneal the n_chains (1 to kCtaChains) chains of a segment from chain first by
 // one CTA.  chain0, init0 and out0 are those of the segment's chain 0; groups
 // past n_chains run a copy of the last chain and write nothing.  smem: Form::smem_bytes(tab.n_classes) bytes.
-template <class Geo, int NC, int NP, int KB = 72>
+template <class Geo, int NC, int NP, int PER>
 __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ init0, uint64_t chain0, int64_t first,
                                                 int n_chains, const core::ChainOut& out0, const core::SweepTables& tab,
                                                 const PhiloxKeys& K, uint8_t* smem) {
-  using F = Form<Geo, NC, NP, KB>;
+  using F = Form<Geo, NC, NP, PER>;
   constexpr int G = Geo::G, NW = Geo::NW, W = Geo::kW, kSweeps = F::kSweeps;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = lane & (G - 1);
   const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
@@ -625,7 +631,7 @@ __device__ __forceinline__ void anneal_coop_cta(const uint32_t* __restrict__ ini
       base[w].init((uint32_t)ch, kTagSA | ((uint32_t)(ch >> 32) << 8), K);
     }
     for (int t0 = 0, set = 0; t0 < n_live; t0 += kSweeps, set ^= 1) {
-      produce<Geo, NC, NP, KB>(t0, min(kSweeps, n_live - t0), base, tab, K, tables + (uint32_t)(set * kSweeps) * kTable, upd,
+      produce<Geo, NC, NP, PER>(t0, min(kSweeps, n_live - t0), base, tab, K, tables + (uint32_t)(set * kSweeps) * kTable, upd,
                            n_upd, draws + set * (F::kDrawWords / 2), warp - NC, lane);
       __syncthreads();
     }

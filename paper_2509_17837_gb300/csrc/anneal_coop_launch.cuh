@@ -42,19 +42,14 @@ inline Args make_args(const xzzx_code* code, const xzzx_schedule* sched, uint64_
   return A;
 }
 
-// Resident CTAs per SM the forms are register-bounded for (what their shared
-// memory allows).
-template <int NP, int KB>
-constexpr int kMinCtas = NP && KB > 52 ? 3 : 4;
-
-template <class Geo, int NC, int NP, int KB>
-__global__ void __launch_bounds__(Form<Geo, NC, NP, KB>::kThreads, kMinCtas<NP, KB>)
+template <class Geo, int NC, int NP, int PER>
+__global__ void __launch_bounds__(Form<Geo, NC, NP, PER>::kThreads, PER)
     anneal_coop_kernel(const __grid_constant__ Args A) {
-  constexpr int kCta = Form<Geo, NC, NP, KB>::kCtaChains;
+  constexpr int kCta = Form<Geo, NC, NP, PER>::kCtaChains;
   extern __shared__ __align__(16) uint8_t smem[];
   const int64_t first = (int64_t)blockIdx.x * kCta;
   const core::ChainOut out{A.best_E, A.best_cfg, A.final_E, A.final_cfg};
-  anneal_coop_cta<Geo, NC, NP, KB>(A.init, A.chain0, first, (int)min((int64_t)kCta, A.n_chains - first), out, A.tab,
+  anneal_coop_cta<Geo, NC, NP, PER>(A.init, A.chain0, first, (int)min((int64_t)kCta, A.n_chains - first), out, A.tab,
                                    A.keys, smem);
 }
 
@@ -65,29 +60,30 @@ xzzx_status sm_count(int* n_sm) {
   return XZZX_OK;
 }
 
-template <class Geo, int NC, int NP, int KB>
+template <class Geo, int NC, int NP, int PER>
 xzzx_status launch_form(const Args& A, cudaStream_t stream) {
-  using F = Form<Geo, NC, NP, KB>;
+  using F = Form<Geo, NC, NP, PER>;
   static DeviceOnce once;
-  xzzx_status st = once.run([] { return allow_shared(anneal_coop_kernel<Geo, NC, NP, KB>); });
+  xzzx_status st = once.run([] { return allow_shared(anneal_coop_kernel<Geo, NC, NP, PER>); });
   if (st) return st;
   const int64_t grid = (A.n_chains + F::kCtaChains - 1) / F::kCtaChains;
   if (grid > 0x7FFFFFFF) return fail(XZZX_EINVAL, "too many chains for one launch");
-  anneal_coop_kernel<Geo, NC, NP, KB><<<(unsigned)grid, F::kThreads, F::smem_bytes(A.tab.n_classes), stream>>>(A);
+  anneal_coop_kernel<Geo, NC, NP, PER><<<(unsigned)grid, F::kThreads, F::smem_bytes(A.tab.n_classes), stream>>>(A);
   XZZX_CUDA_TRY(cudaGetLastError());
   return XZZX_OK;
 }
-// The producing form runs while every CTA (one sweeping warp, kChains chains)
-// is resident at once: three per SM with sets of 72 KB, four with sets of 52 KB
-// (fewer sweeps each, so more barriers); past that its unconditional draws cost
-// more issue slots than they save, and four sweeping warps per CTA share the
-// tables.  400 sweeps at d = 11, producing / plain form, ms: 0.24 / 0.46 at 128
-// chains, 0.30 / 0.50 at 1024, 0.40 / 0.49 at 2048, 0.69 / 0.59 at 4096; one set of
-// 52 KB instead of 72: 0.26 at 128 chains.
+// CTAs per SM of the producing form for this launch, or 0.  It runs while every
+// CTA (one sweeping warp, kChains chains) is resident at once: sized for three
+// per SM, else for four (fewer sweeps per set, so more barriers); past that its
+// unconditional draws cost more issue slots than they save, and four sweeping
+// warps per CTA share the tables.  200 sweeps, CTAs per SM 1, 3, 4, 6, ms: d = 11
+// sized for three 0.088, 0.124, 0.191, 0.228, for four 0.093, 0.125, 0.145, 0.230,
+// plain form 0.204, 0.209, 0.212, 0.247; planar d = 25 0.251, 0.304, 0.525, 0.594;
+// 0.217, 0.276, 0.313, 0.559; 0.468, 0.469, 0.468, 0.583.
 template <class Geo>
-int producing_kb(int64_t n_chains, int n_sm) {
+int producing_per_sm(int64_t n_chains, int n_sm) {
   const int64_t ctas = (n_chains + Geo::kChains - 1) / Geo::kChains;
-  return ctas <= 3 * n_sm ? 72 : ctas <= 4 * n_sm ? 52 : 0;
+  return ctas <= 3 * n_sm ? 3 : ctas <= 4 * n_sm ? 4 : 0;
 }
 
 template <class Geo>
@@ -95,10 +91,10 @@ xzzx_status launch_g(const Args& A, cudaStream_t stream) {
   int n_sm = 0;
   xzzx_status st = sm_count(&n_sm);
   if (st) return st;
-  const int kb = producing_kb<Geo>(A.n_chains, n_sm);
-  return kb == 72   ? launch_form<Geo, 1, 3, 72>(A, stream)
-         : kb == 52 ? launch_form<Geo, 1, 3, 52>(A, stream)
-                    : launch_form<Geo, 4, 0, 72>(A, stream);
+  const int per = producing_per_sm<Geo>(A.n_chains, n_sm);
+  return per == 3   ? launch_form<Geo, 1, 3, 3>(A, stream)
+         : per == 4 ? launch_form<Geo, 1, 3, 4>(A, stream)
+                    : launch_form<Geo, 4, 0, 4>(A, stream);
 }
 
 }  // namespace

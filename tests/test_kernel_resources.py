@@ -23,3 +23,37 @@ def test_persistent_kernels_do_not_spill(tmp_path):
     for unit, text in zip(units, reports):
         spills = re.findall(r"(\d+) bytes spill stores, (\d+) bytes spill loads", text)
         assert spills and all(s == ("0", "0") for s in spills), (unit, spills)
+
+
+LANE_FORMS = r"""
+#include "anneal_coop.cuh"
+#include <cstdio>
+using namespace xzzx::coop;
+template <class G>
+void forms(const char* name, int d) {
+  const int per[3] = {Form<G, 1, 3, 3>::kPerSm, Form<G, 1, 3, 4>::kPerSm, Form<G, 4, 0, 4>::kPerSm};
+  const size_t bytes[3] = {Form<G, 1, 3, 3>::smem_bytes(64), Form<G, 1, 3, 4>::smem_bytes(64),
+                           Form<G, 4, 0, 4>::smem_bytes(64)};
+  for (int k = 0; k < 3; ++k) std::printf("%s %d %d %zu\n", name, d, per[k], bytes[k]);
+}
+template <int D>
+void upto() {
+  forms<RotLanes<D>>("rotated", D);
+  forms<PlanarLanes<D>>("planar", D);
+  if constexpr (D < 31) upto<D + 2>();
+}
+int main() { upto<3>(); }
+"""
+
+
+def test_lane_forms_fit_the_ctas_their_rules_count_on(tmp_path):
+    """The launch rule sizes the lane-parallel forms for so many CTAs per SM: that
+    many fit into an SM's 228 KB, with the kilobyte the system takes of each."""
+    (tmp_path / "forms.cu").write_text(LANE_FORMS)
+    exe = str(tmp_path / "forms")
+    subprocess.run([build.nvcc(), str(tmp_path / "forms.cu"), "-o", exe] + build.NVCC_FLAGS, check=True)
+    rows = [line.split() for line in subprocess.run([exe], capture_output=True, text=True, check=True).stdout.splitlines()]
+    assert len(rows) == 2 * 15 * 3
+    for lattice, d, per_sm, smem in rows:
+        taken = -(-int(smem) // 128) * 128 + 1024
+        assert int(per_sm) >= 3 and int(per_sm) * taken <= 228 * 1024, (lattice, d, per_sm, smem)
