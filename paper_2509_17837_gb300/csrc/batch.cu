@@ -276,7 +276,8 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
     d.restarts = s.restarts;
     d.randomised = s.randomised;
     const int big = greedy::is_large(d.code);
-    const greedy::Cut cut = greedy::cut_of<greedy::RotGeo>(d.code, s.restarts, rpw[big], few[big]);
+    const greedy::Cut cut = greedy::cut_of(d.code, big ? greedy::kLargeWarps : greedy::kSmallWarps, s.restarts,
+                                           s.randomised, rpw[big], few[big]);
     d.greedy_groups = cut.groups;
     d.greedy_cols = cut.cols;
     P.greedy_smem[big] = std::max(P.greedy_smem[big], cut.smem);

@@ -36,6 +36,11 @@ xzzx_status launch_g(const GreedyArgs& A, unsigned grid, size_t smem, cudaStream
   XZZX_CUDA_TRY(cudaGetLastError());
   return XZZX_OK;
 }
+template <class G>
+xzzx_status launch_w(const GreedyArgs& A, int warps, unsigned grid, size_t smem, cudaStream_t stream) {
+  return warps == kLargeWarps ? launch_g<G, kLargeWarps>(A, grid, smem, stream)
+                              : launch_g<G, kSmallWarps>(A, grid, smem, stream);
+}
 
 }  // namespace
 
@@ -50,14 +55,12 @@ xzzx_status launch_greedy(const xzzx_code* code, const xzzx_noise* noise, uint64
   A.n_shots = n_shots;
   A.restarts = restarts;
   A.randomised = randomised;
-  const bool large = is_large(code->dev);
-  const int warps = large ? kLargeWarps : kSmallWarps;
+  const int warps = choose_warps(A.code, n_shots, restarts, randomised);
   int rpw = 1;
   for (int r = kMaxRestartsPerWarp; r > 1 && rpw == 1; r >>= 1)
-    if ((int64_t)n_shots * greedy_groups(restarts, warps, r) >= min_ctas(large)) rpw = r;
+    if ((int64_t)n_shots * greedy_groups(restarts, warps, r) >= min_ctas(is_large(A.code))) rpw = r;
   const bool few = 2 * (int64_t)n_shots * greedy_groups(restarts, warps, 1) <= kFewCtas;
-  const Cut cut = code->layout == kLayoutPlanar ? cut_of<PlanarGeo>(A.code, restarts, rpw, few)
-                                                : cut_of<RotGeo>(A.code, restarts, rpw, few);
+  const Cut cut = cut_of(A.code, warps, restarts, randomised, rpw, few);
   A.groups = cut.groups;
   A.cols = cut.cols;
   A.Wt_x = noise->Wt_x;
@@ -67,11 +70,8 @@ xzzx_status launch_greedy(const xzzx_code* code, const xzzx_noise* noise, uint64
   A.cbits = cbits;
   const uint64_t grid = (uint64_t)n_shots * A.groups;
   if (grid > 0x7FFFFFFFull) return fail(XZZX_EINVAL, "too many shots x restarts for one launch");
-  if (code->layout == kLayoutPlanar)
-    return large ? launch_g<PlanarGeo, kLargeWarps>(A, (unsigned)grid, cut.smem, stream)
-                 : launch_g<PlanarGeo, kSmallWarps>(A, (unsigned)grid, cut.smem, stream);
-  return large ? launch_g<RotGeo, kLargeWarps>(A, (unsigned)grid, cut.smem, stream)
-               : launch_g<RotGeo, kSmallWarps>(A, (unsigned)grid, cut.smem, stream);
+  return code->layout == kLayoutPlanar ? launch_w<PlanarGeo>(A, warps, (unsigned)grid, cut.smem, stream)
+                                       : launch_w<RotGeo>(A, warps, (unsigned)grid, cut.smem, stream);
 }
 
 }  // namespace xzzx

@@ -126,12 +126,13 @@ __host__ __device__ inline int list_room(int faces_per_colour) {
 inline bool is_large(const DevCode& C) { return C.ns / 2 > kSmallFaces && list_room(C.ns / 2) > 0; }
 
 // Shared memory of a CTA: offsets in bytes; cols: colours whose lists are held at
-// once (1 or 2), each in a buffer of list_bytes and tie_bytes.
+// once (1 or 2), each in a buffer of list_bytes and tie_bytes; matched: false for
+// kInitBoundary, which has no pairs and needs none of that.
 struct Carve {
   int wb, nb, fa, fb, step, syn, defects, pq, wd, lists, ties, cur, pairs, free_, cfg, misc, total;
   int room, list_stride, list_bytes, tie_stride, tie_bytes, vmax;
 };
-__host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int cols, int restarts_per_cta) {
+__host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int cols, bool matched, int restarts_per_cta) {
   Carve c;
   int o = 0;
   auto take = [&](int bytes) {
@@ -141,7 +142,7 @@ __host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int col
   };
   const int half = ns / 2;      // faces per colour
   c.vmax = (half + 2 + 31) & ~31;  // vertices per colour, the virtual one too
-  c.room = list_room(half);
+  c.room = matched ? list_room(half) : 0;
   c.list_stride = c.room + 4;   // an odd number of words: lanes on different lists hit different banks
   c.tie_stride = c.room / 32 + 1;
   c.wb = take(4 * ns);
@@ -151,18 +152,18 @@ __host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int col
   c.step = take(ns);
   c.syn = take(4 * sw);
   c.defects = take(2 * 2 * c.vmax);
-  c.pq = take(2 * 4 * c.vmax);
-  c.wd = take(2 * 4 * c.vmax);
+  c.pq = take(matched ? 2 * 4 * c.vmax : 0);
+  c.wd = take(matched ? 2 * 4 * c.vmax : 0);
   // best and partner of each warp: beside the lists, or in their place when
   // the colour is scanned.
-  const int scan = c.vmax > c.room ? 4 * warps * c.vmax : 0, list = c.room * c.list_stride;
+  const int scan = matched && c.vmax > c.room ? 4 * warps * c.vmax : 0, list = c.room * c.list_stride;
   c.list_bytes = ((list > scan ? list : scan) + 15) & ~15;
   c.tie_bytes = (4 * c.room * c.tie_stride + 15) & ~15;
   c.lists = take(cols * c.list_bytes);
   c.ties = take(cols * c.tie_bytes);
   c.cur = take(warps * c.room);
   c.pairs = take(4 * warps * c.room);
-  c.free_ = take(4 * warps * (c.vmax / 32));
+  c.free_ = take(matched ? 4 * warps * (c.vmax / 32) : 0);
   c.cfg = take(4 * restarts_per_cta * 2 * w);
   c.misc = take(4 * (4 + restarts_per_cta));  // n_def[2], usable[2], walk_error[]
   c.total = o;
@@ -476,7 +477,7 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
   const int d = C.d, ns = C.ns, w = C.w;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int lo = (int)((int64_t)group * restarts / groups), hi = (int)((int64_t)(group + 1) * restarts / groups);
-  const Carve c = carve(ns, C.sw, w, kWarps, cols, hi - lo);
+  const Carve c = carve(ns, C.sw, w, kWarps, cols, mode != kInitBoundary, hi - lo);
   int32_t* wb = reinterpret_cast<int32_t*>(smem + c.wb);
   int16_t* nb = reinterpret_cast<int16_t*>(smem + c.nb);            // [4][ns]
   int8_t* fa = reinterpret_cast<int8_t*>(smem + c.fa);
@@ -669,22 +670,28 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
   }
 }
 
-// How a launch of n_shots x restarts of one code is cut: CTAs per shot, colours
-// held at once, shared memory.  n_ctas(r): the CTAs of the whole launch at r
-// restarts per warp (other segments' included).
+// How the shots of one code are cut at rpw restarts per warp: CTAs per shot,
+// colours held at once, shared memory.
 struct Cut {
   int groups = 1, cols = 2;
   size_t smem = 0;
 };
-template <class G>
-inline Cut cut_of(const DevCode& C, int restarts, int rpw, bool few) {
-  const bool large = is_large(C);
-  const int warps = large ? kLargeWarps : kSmallWarps;
+inline Cut cut_of(const DevCode& C, int warps, int restarts, int mode, int rpw, bool few) {
   Cut k;
   k.groups = few ? (restarts + warps / 2 - 1) / (warps / 2) : greedy_groups(restarts, warps, rpw);
   k.cols = C.ns / 2 > kSmallFaces && !few ? 1 : 2;
-  k.smem = (size_t)carve(C.ns, C.sw, C.w, warps, k.cols, (restarts + k.groups - 1) / k.groups).total;
+  k.smem =
+      (size_t)carve(C.ns, C.sw, C.w, warps, k.cols, mode != kInitBoundary, (restarts + k.groups - 1) / k.groups).total;
   return k;
+}
+
+// Warps per CTA of a launch.  Boundary references of a large code build no lists:
+// its wide CTAs only pay while all of them are resident (1000 shots x 1, us, 16
+// warps with the lists' memory / 8 without: rotated d = 21 54 / 32, d = 31 182 / 67).
+inline int choose_warps(const DevCode& C, int64_t n_shots, int restarts, int mode) {
+  if (!is_large(C)) return kSmallWarps;
+  return mode == kInitBoundary && n_shots * greedy_groups(restarts, kLargeWarps, 1) > min_ctas(true) ? kSmallWarps
+                                                                                                     : kLargeWarps;
 }
 
 }  // namespace greedy

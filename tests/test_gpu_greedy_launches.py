@@ -1,0 +1,42 @@
+"""Greedy references in the launches that take a way of their own: boundary
+references of large codes in narrow CTAs without lists.  Each equals the same
+shots a few at a time, and the oracle on a sample."""
+import numpy as np
+import pytest
+
+import oracle as O
+from layout import syn_words_to_bits, words_to_labels
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+
+    import paper_2509_17837_gb300 as X
+    return X, torch
+
+
+def check(env, layout, d, restarts, shots, mode, p, eta):
+    X, torch = env
+    code, noise = X.Code(d, layout), X.noise_from_eta(p, eta)
+    _, syn = X.sample_errors(code, noise, 4, 11, shots)
+    init, cbits = X.greedy_init(code, noise, 4, 11, syn, restarts, randomised=mode)
+    for first, n in ((0, 1), (shots - 1, 1), (shots // 2, 6)):
+        # more restarts than needed: another cut of the same references
+        a, c = X.greedy_init(code, noise, 4, 11 + first, syn[first:first + n].contiguous(), restarts + 7, randomised=mode)
+        assert torch.equal(a[:, :restarts], init[first:first + n]) and torch.equal(c[:, :restarts], cbits[first:first + n])
+    cid = O.planar(d) if layout else d
+    bits = syn_words_to_bits(syn.cpu().numpy(), code.n_stab)
+    for s in (0, shots - 1):
+        ref, _ = O.greedy(cid, (noise.px, noise.py, noise.pz), noise.scale, 4, 11 + s, restarts - 1, mode, bits[s])
+        assert np.array_equal(words_to_labels(init[s, restarts - 1].cpu().numpy(), code.n_qubits), ref)
+        assert int(cbits[s, restarts - 1]) == O.class_bits(cid, ref)
+    assert code.device_errors() == (0, 0)
+
+
+@pytest.mark.parametrize("layout,d,restarts,shots", [(0, 19, 1, 305), (0, 31, 1, 700), (0, 25, 40, 110), (1, 13, 3, 500),
+                                                     (1, 27, 64, 100), (1, 31, 1, 400)])
+def test_boundary_references_of_large_codes(env, layout, d, restarts, shots):
+    check(env, layout, d, restarts, shots, 2, 0.14, 5.0)
