@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kWarps * 32, 32 / kWarps)
   const int64_t local = b - G.cta_prefix[s];
   const int64_t k = local / sg.greedy_groups;
   const int group = (int)(local % sg.greedy_groups);
-  greedy::greedy_cta<greedy::RotGeo, kWarps>(sg.code, G.keys, sg.shot0 + (uint64_t)k, group, sg.greedy_groups, sg.greedy_cols, sg.restarts,
+  greedy::greedy_cta<greedy::RotGeo, kWarps>(sg.code, G.keys, sg.shot0 + (uint64_t)k, group, sg.greedy_groups, sg.greedy_cols, sg.greedy_room, sg.restarts,
                                      sg.randomised, sg.Wt_x, sg.Wt_z, sg.syndromes + (size_t)k * sg.code.sw,
                                      sg.init + (size_t)k * sg.restarts * 2 * sg.code.w, sg.cbits + (size_t)k * sg.restarts,
                                      smem);
@@ -277,9 +277,10 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
     d.randomised = s.randomised;
     const int big = greedy::is_large(d.code);
     const greedy::Cut cut = greedy::cut_of(d.code, big ? greedy::kLargeWarps : greedy::kSmallWarps, s.restarts,
-                                           s.randomised, rpw[big], few[big]);
+                                           s.randomised, rpw[big], few[big], false);
     d.greedy_groups = cut.groups;
     d.greedy_cols = cut.cols;
+    d.greedy_room = cut.room;
     P.greedy_smem[big] = std::max(P.greedy_smem[big], cut.smem);
     d.Wt_x = s.noise->Wt_x;
     d.Wt_z = s.noise->Wt_z;

@@ -14,7 +14,7 @@ constexpr int kNT = 128;  // default chains per CTA of the batched anneal launch
 struct SegDev {
   DevCode code;
   uint64_t shot0;
-  int n_shots, restarts, randomised, greedy_groups, greedy_cols;
+  int n_shots, restarts, randomised, greedy_groups, greedy_cols, greedy_room;
   int32_t Wt_x, Wt_z;
   const uint32_t* syndromes;
   const uint32_t* true_errors;

@@ -11,7 +11,7 @@ struct GreedyArgs {
   DevCode code;
   PhiloxKeys keys;
   uint64_t shot0;
-  int n_shots, restarts, randomised, groups, cols;
+  int n_shots, restarts, randomised, groups, cols, room;
   int32_t Wt_x, Wt_z;
   const uint32_t* syndromes;
   uint32_t* init;
@@ -22,8 +22,8 @@ template <class G, int kWarps>
 __global__ void __launch_bounds__(kWarps * 32, 32 / kWarps) greedy_kernel(const __grid_constant__ GreedyArgs A) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int k = blockIdx.x / A.groups;
-  greedy_cta<G, kWarps>(A.code, A.keys, A.shot0 + (uint64_t)k, blockIdx.x % A.groups, A.groups, A.cols, A.restarts,
-                        A.randomised, A.Wt_x, A.Wt_z, A.syndromes + (size_t)k * A.code.sw,
+  greedy_cta<G, kWarps>(A.code, A.keys, A.shot0 + (uint64_t)k, blockIdx.x % A.groups, A.groups, A.cols, A.room,
+                        A.restarts, A.randomised, A.Wt_x, A.Wt_z, A.syndromes + (size_t)k * A.code.sw,
                         A.init + (size_t)k * A.restarts * 2 * A.code.w, A.cbits + (size_t)k * A.restarts, smem);
 }
 
@@ -55,14 +55,16 @@ xzzx_status launch_greedy(const xzzx_code* code, const xzzx_noise* noise, uint64
   A.n_shots = n_shots;
   A.restarts = restarts;
   A.randomised = randomised;
-  const int warps = choose_warps(A.code, n_shots, restarts, randomised);
+  const bool scan = randomised != kInitBoundary && scans(A.code, *noise, restarts);
+  const int warps = choose_warps(A.code, n_shots, restarts, randomised, scan);
   int rpw = 1;
-  for (int r = kMaxRestartsPerWarp; r > 1 && rpw == 1; r >>= 1)
+  for (int r = kMaxRestartsPerWarp; r > 1 && rpw == 1 && !scan; r >>= 1)  // a scan has no lists to share
     if ((int64_t)n_shots * greedy_groups(restarts, warps, r) >= min_ctas(is_large(A.code))) rpw = r;
   const bool few = 2 * (int64_t)n_shots * greedy_groups(restarts, warps, 1) <= kFewCtas;
-  const Cut cut = cut_of(A.code, warps, restarts, randomised, rpw, few);
+  const Cut cut = cut_of(A.code, warps, restarts, randomised, rpw, few, scan);
   A.groups = cut.groups;
   A.cols = cut.cols;
+  A.room = cut.room;
   A.Wt_x = noise->Wt_x;
   A.Wt_z = noise->Wt_z;
   A.syndromes = syndromes;

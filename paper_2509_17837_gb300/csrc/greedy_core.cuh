@@ -39,6 +39,8 @@
 // ms.
 #pragma once
 
+#include <cmath>
+
 #include "anneal_core.cuh"
 #include "internal.h"
 #include "philox.cuh"
@@ -125,14 +127,28 @@ __host__ __device__ inline int list_room(int faces_per_colour) {
 
 inline bool is_large(const DevCode& C) { return C.ns / 2 > kSmallFaces && list_room(C.ns / 2) > 0; }
 
+// Whether a launch scans every colour: without lists, or with so few restarts
+// that the scan of a colour which has outgrown its list would leave most of a
+// large CTA's warps idle, where the noise says that most colours will (1000 shots x
+// 1, planar d = 27, p = 0.14: 8.6 -> 3.4 ms).
+inline bool scans(const DevCode& C, const xzzx_noise& noise, int restarts) {
+  const double a = 1.0 - 2.0 * (noise.px + noise.py), b = 1.0 - 2.0 * (noise.pz + noise.py);
+  const double p = 0.5 * (1.0 - a * a * b * b), n = C.ns / 2 * p;  // defects of a colour of four-qubit faces
+  const int room = list_room(C.ns / 2);
+  return room == 0 || (restarts <= 4 && n + std::sqrt(n * (1.0 - p)) > room);
+}
+
 // Shared memory of a CTA: offsets in bytes; cols: colours whose lists are held at
-// once (1 or 2), each in a buffer of list_bytes and tie_bytes; matched: false for
-// kInitBoundary, which has no pairs and needs none of that.
+// once (1 or 2), each in a buffer of list_bytes and tie_bytes; room: vertices a
+// list has room for (0: every colour is scanned); matched: false for
+// kInitBoundary, which has no pairs and needs none of that.  The boundary
+// distances wb give way to the lists once they are in wd.
 struct Carve {
   int wb, nb, fa, fb, step, syn, defects, pq, wd, lists, ties, cur, pairs, free_, cfg, misc, total;
-  int room, list_stride, list_bytes, tie_stride, tie_bytes, vmax;
+  int list_stride, list_bytes, tie_stride, tie_bytes, vmax;
 };
-__host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int cols, bool matched, int restarts_per_cta) {
+__host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int cols, int room, bool matched,
+                                       int restarts_per_cta) {
   Carve c;
   int o = 0;
   auto take = [&](int bytes) {
@@ -142,10 +158,8 @@ __host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int col
   };
   const int half = ns / 2;      // faces per colour
   c.vmax = (half + 2 + 31) & ~31;  // vertices per colour, the virtual one too
-  c.room = matched ? list_room(half) : 0;
-  c.list_stride = c.room + 4;   // an odd number of words: lanes on different lists hit different banks
-  c.tie_stride = c.room / 32 + 1;
-  c.wb = take(4 * ns);
+  c.list_stride = room + 4;     // an odd number of words: lanes on different lists hit different banks
+  c.tie_stride = room / 32 + 1;
   c.nb = take(4 * 2 * ns);
   c.fa = take(ns);
   c.fb = take(ns);
@@ -155,14 +169,16 @@ __host__ __device__ inline Carve carve(int ns, int sw, int w, int warps, int col
   c.pq = take(matched ? 2 * 4 * c.vmax : 0);
   c.wd = take(matched ? 2 * 4 * c.vmax : 0);
   // best and partner of each warp: beside the lists, or in their place when
-  // the colour is scanned.
-  const int scan = matched && c.vmax > c.room ? 4 * warps * c.vmax : 0, list = c.room * c.list_stride;
-  c.list_bytes = ((list > scan ? list : scan) + 15) & ~15;
-  c.tie_bytes = (4 * c.room * c.tie_stride + 15) & ~15;
-  c.lists = take(cols * c.list_bytes);
+  // the colour is scanned (without lists one area serves both colours: a warp
+  // works on one at a time).
+  const int scan = matched && c.vmax > room ? 4 * warps * c.vmax : 0, list = room * c.list_stride;
+  c.list_bytes = room ? ((list > scan ? list : scan) + 15) & ~15 : 0;
+  c.tie_bytes = (4 * room * c.tie_stride + 15) & ~15;
+  const int lists = room ? cols * c.list_bytes : scan;
+  c.wb = c.lists = take(lists > 4 * ns ? lists : 4 * ns);
   c.ties = take(cols * c.tie_bytes);
-  c.cur = take(warps * c.room);
-  c.pairs = take(4 * warps * c.room);
+  c.cur = take(warps * room);
+  c.pairs = take(4 * warps * room);
   c.free_ = take(matched ? 4 * warps * (c.vmax / 32) : 0);
   c.cfg = take(4 * restarts_per_cta * 2 * w);
   c.misc = take(4 * (4 + restarts_per_cta));  // n_def[2], usable[2], walk_error[]
@@ -471,13 +487,13 @@ __device__ __forceinline__ bool match(const Vertices& V, const Carve& c, const u
 // bytes for at least that many restarts.
 template <class G, int kWarps>
 __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K, uint64_t shot, int group, int groups,
-                                           int cols, int restarts, int mode, int32_t Wt_x, int32_t Wt_z,
+                                           int cols, int room, int restarts, int mode, int32_t Wt_x, int32_t Wt_z,
                                            const uint32_t* __restrict__ syn, uint32_t* __restrict__ init,
                                            uint8_t* __restrict__ cbits, uint8_t* smem) {
   const int d = C.d, ns = C.ns, w = C.w;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int lo = (int)((int64_t)group * restarts / groups), hi = (int)((int64_t)(group + 1) * restarts / groups);
-  const Carve c = carve(ns, C.sw, w, kWarps, cols, mode != kInitBoundary, hi - lo);
+  const Carve c = carve(ns, C.sw, w, kWarps, cols, room, mode != kInitBoundary, hi - lo);
   int32_t* wb = reinterpret_cast<int32_t*>(smem + c.wb);
   int16_t* nb = reinterpret_cast<int16_t*>(smem + c.nb);            // [4][ns]
   int8_t* fa = reinterpret_cast<int8_t*>(smem + c.fa);
@@ -493,7 +509,7 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
   int* walk_error = n_def + 4;                                      // [hi - lo]
   Work W;
   W.free_ = reinterpret_cast<uint32_t*>(smem + c.free_) + warp * (c.vmax / 32);
-  W.cur = smem + c.cur + warp * c.room;
+  W.cur = smem + c.cur + warp * room;
 
   // Faces, their neighbours, and distances over the boundary edges alone.
   for (int f = tid; f < ns; f += blockDim.x) {
@@ -590,14 +606,14 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
         pq[colour * c.vmax + x] = (G::zpos(fa[f], fb[f]) + 256) | ((G::xpos(fa[f], fb[f]) + 256) << 16);
         wd[colour * c.vmax + x] = wb[f];
       }
-    if (tid < 2) usable[tid] = n_def[tid] + (n_def[tid] & 1) <= c.room;
+    if (tid < 2) usable[tid] = n_def[tid] + (n_def[tid] & 1) <= room;
     __syncthreads();
   }
   PairKeys pk(shot, K);
   for (int first = 0; first < 2 && mode != kInitBoundary; first += cols) {
     for (int slot = 0; slot < cols; ++slot) {  // candidate lists, every warp of the CTA building some
       const Vertices V = vertices(first + slot);
-      if (V.nv > c.room) continue;
+      if (V.nv > room) continue;
       bool fits = true;
       for (int x = warp; x < V.nv; x += kWarps) {
         uint8_t* Lx = smem + c.lists + slot * c.list_bytes + x * c.list_stride;
@@ -610,14 +626,14 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
       if (lane == 0 && !fits) usable[first + slot] = 0;
     }
     __syncthreads();
-    for (int it = warp; it < cols * (hi - lo); it += kWarps) {
-      const int slot = it % cols, i = lo + it / cols;
+    for (int it = warp; it < cols * (hi - lo); it += kWarps) {  // both colours of a warp's restarts, not one of more
+      const int slot = it >= hi - lo, i = lo + it - slot * (hi - lo);
       const Vertices V = vertices(first + slot);
       if (V.nv == 0) continue;
       const bool listed = usable[first + slot] != 0;
       const uint8_t* lists = smem + c.lists + slot * c.list_bytes;
       const uint32_t* ties = reinterpret_cast<const uint32_t*>(smem + c.ties + slot * c.tie_bytes);
-      const int len = listed ? c.room : c.vmax;  // per warp: best, then partner
+      const int len = listed ? room : c.vmax;  // per warp: best, then partner
       W.best = reinterpret_cast<int16_t*>(smem + (listed ? c.pairs : c.lists + slot * c.list_bytes)) + warp * 2 * len;
       W.partner = W.best + len;
       __syncwarp();  // the warp's previous matching is walked
@@ -671,25 +687,26 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
 }
 
 // How the shots of one code are cut at rpw restarts per warp: CTAs per shot,
-// colours held at once, shared memory.
+// colours held at once, room of the lists, shared memory.
 struct Cut {
-  int groups = 1, cols = 2;
+  int groups = 1, cols = 2, room = 0;
   size_t smem = 0;
 };
-inline Cut cut_of(const DevCode& C, int warps, int restarts, int mode, int rpw, bool few) {
+inline Cut cut_of(const DevCode& C, int warps, int restarts, int mode, int rpw, bool few, bool scan) {
   Cut k;
+  const bool matched = mode != kInitBoundary;
+  k.room = matched && !scan ? list_room(C.ns / 2) : 0;
   k.groups = few ? (restarts + warps / 2 - 1) / (warps / 2) : greedy_groups(restarts, warps, rpw);
-  k.cols = C.ns / 2 > kSmallFaces && !few ? 1 : 2;
-  k.smem =
-      (size_t)carve(C.ns, C.sw, C.w, warps, k.cols, mode != kInitBoundary, (restarts + k.groups - 1) / k.groups).total;
+  k.cols = C.ns / 2 > kSmallFaces && k.room && !few ? 1 : 2;
+  k.smem = (size_t)carve(C.ns, C.sw, C.w, warps, k.cols, k.room, matched, (restarts + k.groups - 1) / k.groups).total;
   return k;
 }
 
 // Warps per CTA of a launch.  Boundary references of a large code build no lists:
 // its wide CTAs only pay while all of them are resident (1000 shots x 1, us, 16
 // warps with the lists' memory / 8 without: rotated d = 21 54 / 32, d = 31 182 / 67).
-inline int choose_warps(const DevCode& C, int64_t n_shots, int restarts, int mode) {
-  if (!is_large(C)) return kSmallWarps;
+inline int choose_warps(const DevCode& C, int64_t n_shots, int restarts, int mode, bool scan) {
+  if (!is_large(C) || scan) return kSmallWarps;
   return mode == kInitBoundary && n_shots * greedy_groups(restarts, kLargeWarps, 1) > min_ctas(true) ? kSmallWarps
                                                                                                      : kLargeWarps;
 }

@@ -1,5 +1,5 @@
 """Greedy references in the launches that take a way of their own: boundary
-references of large codes in narrow CTAs without lists.  Each equals the same
+references of large codes in narrow CTAs without lists, and launches that scan every colour.  Each equals the same
 shots a few at a time, and the oracle on a sample."""
 import numpy as np
 import pytest
@@ -40,3 +40,13 @@ def check(env, layout, d, restarts, shots, mode, p, eta):
                                                      (1, 27, 64, 100), (1, 31, 1, 400)])
 def test_boundary_references_of_large_codes(env, layout, d, restarts, shots):
     check(env, layout, d, restarts, shots, 2, 0.14, 5.0)
+
+
+@pytest.mark.parametrize("layout,d,restarts,shots,p", [(1, 27, 1, 300, 0.17), (1, 27, 4, 60, 0.17), (1, 25, 2, 160, 0.25),
+                                                       (1, 27, 4, 60, 0.06), (1, 29, 1, 300, 0.12), (1, 31, 9, 40, 0.12),
+                                                       (1, 31, 64, 20, 0.04)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_scans(env, layout, d, restarts, shots, p, mode):
+    """Planar d >= 29, and d = 25, 27 with few restarts where the noise fills the
+    colours (p = 0.06: lists)."""
+    check(env, layout, d, restarts, shots, mode, p, 5.0)
