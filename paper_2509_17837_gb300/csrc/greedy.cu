@@ -38,8 +38,9 @@ xzzx_status launch_g(const GreedyArgs& A, unsigned grid, size_t smem, cudaStream
 }
 template <class G>
 xzzx_status launch_w(const GreedyArgs& A, int warps, unsigned grid, size_t smem, cudaStream_t stream) {
-  return warps == kLargeWarps ? launch_g<G, kLargeWarps>(A, grid, smem, stream)
-                              : launch_g<G, kSmallWarps>(A, grid, smem, stream);
+  return warps == kLargeWarps   ? launch_g<G, kLargeWarps>(A, grid, smem, stream)
+         : warps == kSmallWarps ? launch_g<G, kSmallWarps>(A, grid, smem, stream)
+                                : launch_g<G, kFewWarps>(A, grid, smem, stream);
 }
 
 }  // namespace

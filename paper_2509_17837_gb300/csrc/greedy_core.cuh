@@ -48,10 +48,11 @@
 namespace xzzx {
 namespace greedy {
 
-// Warps of a CTA: 8 for codes of up to 150 faces per decoding-graph colour
-// (rotated d <= 17, planar d <= 11), 16 above, where the lists take long to build
-// and most of the shared memory.
-constexpr int kSmallWarps = 8, kLargeWarps = 16, kSmallFaces = 150;
+// Warps of a CTA (choose_warps): 8 for codes of up to 150 faces per
+// decoding-graph colour (rotated d <= 17, planar d <= 11), 16 above, where the lists
+// take long to build and most of the shared memory, 4 where there is too little
+// for 8 to do.
+constexpr int kFewWarps = 4, kSmallWarps = 8, kLargeWarps = 16, kSmallFaces = 150;
 // A launch of no more CTAs than this gives each restart two warps, one per colour.
 constexpr int64_t kFewCtas = 152;
 // A launch takes the largest restarts-per-warp count (8, 4, 2 or 1) that still
@@ -579,7 +580,6 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
     }
     step[f] = (uint8_t)st;
   }
-  __syncthreads();
 
   auto vertices = [&](int colour) {
     Vertices V;
@@ -591,6 +591,7 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
     return V;
   };
   if (mode == kInitBoundary) {
+    __syncthreads();
     // Each defect joined to the nearer boundary of its decoding graph.
     for (int i = lo + warp; i < hi; i += kWarps)
       for (int colour = 0; colour < 2; ++colour) {
@@ -613,7 +614,7 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
   for (int first = 0; first < 2 && mode != kInitBoundary; first += cols) {
     for (int slot = 0; slot < cols; ++slot) {  // candidate lists, every warp of the CTA building some
       const Vertices V = vertices(first + slot);
-      if (V.nv > room) continue;
+      if (V.nv <= 2 || V.nv > room) continue;  // two vertices match each other
       bool fits = true;
       for (int x = warp; x < V.nv; x += kWarps) {
         uint8_t* Lx = smem + c.lists + slot * c.list_bytes + x * c.list_stride;
@@ -638,9 +639,14 @@ __device__ __forceinline__ void greedy_cta(const DevCode& C, const PhiloxKeys& K
       W.partner = W.best + len;
       __syncwarp();  // the warp's previous matching is walked
       if (mode == kInitGreedyRandom) pk.restart(i, K);
-      const bool good =
-          listed ? match<true>(V, c, lists, ties, W, mode == kInitGreedyRandom, pk, K, Wt_x, Wt_z, C.err, lane)
-                 : match<false>(V, c, lists, ties, W, mode == kInitGreedyRandom, pk, K, Wt_x, Wt_z, C.err, lane);
+      bool good = true;
+      if (V.nv == 2) {
+        if (lane < 2) W.partner[lane] = (int16_t)(1 - lane);
+        __syncwarp();
+      } else {
+        good = listed ? match<true>(V, c, lists, ties, W, mode == kInitGreedyRandom, pk, K, Wt_x, Wt_z, C.err, lane)
+                      : match<false>(V, c, lists, ties, W, mode == kInitGreedyRandom, pk, K, Wt_x, Wt_z, C.err, lane);
+      }
       uint32_t* cfg = cfgs + (i - lo) * 2 * w;
       bool ok = good;
       // Join every kept pair.
@@ -702,11 +708,20 @@ inline Cut cut_of(const DevCode& C, int warps, int restarts, int mode, int rpw, 
   return k;
 }
 
-// Warps per CTA of a launch.  Boundary references of a large code build no lists:
-// its wide CTAs only pay while all of them are resident (1000 shots x 1, us, 16
-// warps with the lists' memory / 8 without: rotated d = 21 54 / 32, d = 31 182 / 67).
+// Warps per CTA of a launch.
 inline int choose_warps(const DevCode& C, int64_t n_shots, int restarts, int mode, bool scan) {
+  const int half = C.ns / 2;
+  // Past one wave of eight-warp CTAs, where a shot has not enough to keep them
+  // busy, narrow ones hold twice the shots on an SM (p = 0.14, us, 8 warps / 4: 1000
+  // shots x 1 restart d = 3 13.8 / 8.5, d = 9 28.5 / 20.8, d = 17 91 / 87; 1000 x 3 d = 5
+  // 19.1 / 17.3, d = 17 98 / 114; 300 x 64 d = 3 34.7 / 30.2).
+  if (half <= kSmallFaces && !scan && n_shots * greedy_groups(restarts, kSmallWarps, 1) > 608 &&
+      (half <= 6 || restarts <= 2 || (restarts == 3 && (half <= 12 || mode == kInitBoundary))))
+    return kFewWarps;
   if (!is_large(C) || scan) return kSmallWarps;
+  // Boundary references of a large code build no lists: its wide CTAs only pay
+  // while all of them are resident (1000 shots x 1, us, 16 warps with the lists'
+  // memory / 8 without: rotated d = 21 54 / 32, d = 31 182 / 67).
   return mode == kInitBoundary && n_shots * greedy_groups(restarts, kLargeWarps, 1) > min_ctas(true) ? kSmallWarps
                                                                                                      : kLargeWarps;
 }

@@ -1,5 +1,6 @@
 """Greedy references in the launches that take a way of their own: boundary
-references of large codes in narrow CTAs without lists, and launches that scan every colour.  Each equals the same
+references of large codes in narrow CTAs without lists, launches that scan every
+colour, and small codes in CTAs of four warps.  Each equals the same
 shots a few at a time, and the oracle on a sample."""
 import numpy as np
 import pytest
@@ -49,4 +50,13 @@ def test_boundary_references_of_large_codes(env, layout, d, restarts, shots):
 def test_scans(env, layout, d, restarts, shots, p, mode):
     """Planar d >= 29, and d = 25, 27 with few restarts where the noise fills the
     colours (p = 0.06: lists)."""
+    check(env, layout, d, restarts, shots, mode, p, 5.0)
+
+
+@pytest.mark.parametrize("layout,d,restarts,shots", [(0, 3, 8, 700), (0, 3, 3, 609), (0, 5, 3, 800), (0, 9, 1, 700),
+                                                     (0, 17, 2, 650), (1, 3, 20, 400), (1, 11, 1, 700)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("p", [0.02, 0.15])
+def test_narrow_launches_of_small_codes(env, layout, d, restarts, shots, mode, p):
+    """Four-warp CTAs; at the low rate most colours have no more than two vertices."""
     check(env, layout, d, restarts, shots, mode, p, 5.0)
