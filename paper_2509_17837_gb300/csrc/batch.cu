@@ -370,22 +370,24 @@ namespace {
 struct BlobLayout {
   size_t segs, lpt, byd, bycls, cta, shot, chain, head, total;
 };
-BlobLayout blob_layout(const Plan& p) {
+BlobLayout blob_layout(size_t n_segs, size_t n_chunks) {
   BlobLayout L;
-  const size_t nc = std::max<size_t>(p.lpt.size(), 1);
+  const size_t nc = std::max<size_t>(n_chunks, 1);
   L.segs = 0;
-  L.lpt = align256(L.segs + sizeof(SegDev) * p.segs.size());
+  L.lpt = align256(L.segs + sizeof(SegDev) * n_segs);
   L.byd = align256(L.lpt + sizeof(ChunkDev) * nc);
   L.bycls = align256(L.byd + sizeof(ChunkDev) * nc);
   L.cta = align256(L.bycls + sizeof(ChunkDev) * nc);
-  L.shot = align256(L.cta + sizeof(int64_t) * p.cta_prefix.size());
-  L.chain = align256(L.shot + sizeof(int64_t) * p.shot_prefix.size());
-  L.head = align256(L.chain + sizeof(int64_t) * p.chain_prefix.size());
+  L.shot = align256(L.cta + sizeof(int64_t) * (n_segs + 1));
+  L.chain = align256(L.shot + sizeof(int64_t) * (n_segs + 1));
+  L.head = align256(L.chain + sizeof(int64_t) * (n_segs + 1));
   L.total = align256(L.head + sizeof(int) * (1 + kNumClasses));
   return L;
 }
+BlobLayout blob_layout(const Plan& p) { return blob_layout(p.segs.size(), p.lpt.size()); }
 }  // namespace
 
+size_t descriptor_bytes(size_t n_segs, size_t n_chunks) { return blob_layout(n_segs, n_chunks).total; }
 size_t descriptor_bytes(const Plan& p) { return blob_layout(p).total; }
 
 PlanDev descriptor_layout(const Plan& p, char* base) {

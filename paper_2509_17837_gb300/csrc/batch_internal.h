@@ -105,6 +105,7 @@ struct PlanDev {
 xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int order, char* ws_base, Plan& out,
                        int nt = kNT, int unroll = 1);
 // Bytes of the descriptor blob and the layout of PlanDev inside it.
+size_t descriptor_bytes(size_t n_segs, size_t n_chunks);
 size_t descriptor_bytes(const Plan& p);
 PlanDev descriptor_layout(const Plan& p, char* dev_base);
 void pack_descriptors(const Plan& p, char* host_blob);

@@ -49,7 +49,8 @@ struct Class {
   xzzx_schedule* sched = nullptr;
   xzzx_noise noise{};
   int d = 0, group = 0;
-  size_t bytes = 0;      // conservative device bytes per request
+  size_t bytes = 0;      // conservative device bytes of one request, for the check at start
+  size_t chunks = 0, syn = 0, workspace = 0;  // a request's chunks, and its bytes of syndrome and workspace
   int64_t regs = 0;      // registers per request while resident
 };
 
@@ -77,6 +78,17 @@ struct Slot {
 };
 
 constexpr size_t kOutStride = 512;  // bytes per request result in the output area
+
+inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// What a batch takes of its slot, laid out as [descriptors | syndromes | outputs |
+// workspace], the first two of them staged in pinned host memory.
+struct Need {
+  size_t n = 0, chunks = 0, syn = 0, workspace = 0;
+  Need plus(const Class& c) const { return {n + 1, chunks + c.chunks, syn + c.syn, workspace + c.workspace}; }
+  size_t staging() const { return align256(align256(batch::descriptor_bytes(n, chunks)) + syn); }
+  size_t device() const { return align256(staging() + n * kOutStride) + workspace; }
+};
 
 }  // namespace serve
 }  // namespace xzzx
@@ -110,8 +122,6 @@ struct xzzx_server {
 namespace xzzx {
 namespace serve {
 namespace {
-
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 void CUDART_CB on_complete(void* p) {
   Slot* s = (Slot*)p;
@@ -232,15 +242,16 @@ void harvest(xzzx_server* sv) {
 bool form_batch(xzzx_server* sv, Slot& slot) {
   if (sv->pending.empty()) return false;
   const int group = sv->classes[sv->pending.front().cls].d;
-  size_t bytes = 4096;
+  Need need;
   int64_t regs = 0;
   std::vector<size_t> take;
   for (size_t i = 0; i < sv->pending.size() && (int)take.size() < sv->cfg.max_batch; ++i) {
     const Class& c = sv->classes[sv->pending[i].cls];
     if (c.d != group) continue;
-    if (bytes + c.bytes > sv->slot_bytes) break;
+    const Need with = need.plus(c);
+    if (with.device() > sv->slot_bytes || with.staging() > sv->staging_bytes) break;
     if (sv->regs_in_use + regs + c.regs > sv->regs_total && !(take.empty() && sv->regs_in_use == 0)) break;
-    bytes += c.bytes;
+    need = with;
     regs += c.regs;
     take.push_back(i);
   }
@@ -398,10 +409,11 @@ xzzx_status xzzx_serve_add_class(xzzx_server* sv, int d, const xzzx_noise* noise
   }
   const size_t R = (size_t)sv->cfg.restarts, w = (size_t)c.code->w;
   // descriptors (segment + chunks + prefixes), workspace, syndrome, output row
-  const size_t chunks = (4 * R + batch::kNT - 1) / batch::kNT;
-  c.bytes = sizeof(batch::SegDev) + chunks * 2 * sizeof(batch::ChunkDev) + 2 * sizeof(int64_t) +
-            align256(sizeof(uint32_t) * R * 2 * w) + align256(R) + align256(sizeof(int32_t) * 4 * R) +
-            align256(sizeof(uint32_t) * c.code->sw) + kOutStride;
+  c.chunks = (4 * R + batch::kNT - 1) / batch::kNT;
+  c.syn = align256(sizeof(uint32_t) * c.code->sw);
+  c.workspace = align256(sizeof(uint32_t) * R * 2 * w) + align256(R) + align256(sizeof(int32_t) * 4 * R);
+  c.bytes = sizeof(batch::SegDev) + c.chunks * 2 * sizeof(batch::ChunkDev) + 2 * sizeof(int64_t) + c.workspace + c.syn +
+            kOutStride;
   c.regs = 0;  // filled at start, from the kernel's register use
   *class_id = (int)sv->classes.size();
   sv->classes.push_back(c);
@@ -432,11 +444,14 @@ xzzx_status xzzx_serve_start(xzzx_server* sv) {
   sv->staging_bytes = ((size_t)64 << 10) + (size_t)sv->cfg.max_batch * 1024;
   // Every class must fit one request into an empty slot (memory and staging),
   // or requests of that class could never be dispatched.
-  for (const Class& c : sv->classes)
-    if (4096 + c.bytes > sv->slot_bytes || 4096 + c.bytes > sv->staging_bytes)
-      return fail(XZZX_ENOMEM, "one request of distance " + std::to_string(c.d) + " needs " +
-                                   std::to_string(4096 + c.bytes) + " bytes but a slot holds " +
-                                   std::to_string(sv->slot_bytes) + " (raise hbm_budget_bytes or lower n_slots)");
+  for (const Class& c : sv->classes) {
+    const Need one = Need().plus(c);
+    const size_t dev = std::max(4096 + c.bytes, one.device()), staged = std::max(4096 + c.bytes, one.staging());
+    if (dev > sv->slot_bytes || staged > sv->staging_bytes)
+      return fail(XZZX_ENOMEM, "one request of distance " + std::to_string(c.d) + " needs " + std::to_string(dev) +
+                                   " bytes but a slot holds " + std::to_string(sv->slot_bytes) +
+                                   " (raise hbm_budget_bytes or lower n_slots)");
+  }
   // One device error area for every class's code, so that each batch's flags
   // can be read back with its results.
   XZZX_CUDA_TRY(cudaMalloc((void**)&sv->d_err, 256));
