@@ -331,15 +331,14 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
   P.workspace_bytes = ws;
   P.byd = chunks;  // grouped by distance already (segments are)
   P.lpt = chunks;
-  auto work = [](const ChunkDev& c) { return (int64_t)c.n_sweeps * (c.d * c.d - 1); };
   if (order_policy == 0)
     std::stable_sort(P.lpt.begin(), P.lpt.end(),
-                     [&](const ChunkDev& x, const ChunkDev& y) { return work(x) > work(y); });
+                     [](const ChunkDev& x, const ChunkDev& y) { return chunk_work(x) > chunk_work(y); });
   P.bycls = chunks;
   std::stable_sort(P.bycls.begin(), P.bycls.end(), [&](const ChunkDev& x, const ChunkDev& y) {
     const int cx = class_of(x.d), cy = class_of(y.d);
     if (cx != cy) return cx < cy;
-    return order_policy == 0 && work(x) > work(y);
+    return order_policy == 0 && chunk_work(x) > chunk_work(y);
   });
   for (int c = 0, k = 0; c < kNumClasses; ++c) {
     ClassRange r;

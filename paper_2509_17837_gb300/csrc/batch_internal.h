@@ -42,6 +42,15 @@ struct ChunkDev {
   int32_t W[4];
 };
 
+// Attempts a chain of a chunk takes, for the order of the queue: the sweeps with
+// a threshold above zero, then about kRepeatSweeps until the chains of a warp all
+// repeat (at d = 5 to 21, eta = 1 to 100; the rest of the schedule is not run).
+constexpr int kRepeatSweeps = 60;
+inline int64_t chunk_work(const ChunkDev& c) {
+  const int live = c.n_live + kRepeatSweeps;
+  return (int64_t)(live < c.n_sweeps ? live : c.n_sweeps) * (c.d * c.d - 1);
+}
+
 struct AnnealLaunch {
   PhiloxKeys keys;
   const SegDev* segs;
