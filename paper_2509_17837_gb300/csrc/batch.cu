@@ -18,6 +18,7 @@
 // plans into memory it allocated up front.
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <numeric>
 #include <vector>
@@ -478,7 +479,10 @@ struct xzzx_batch {
   cudaGraphExec_t graph_exec = nullptr;
   int graph_mode = 0;
   int class_grid[xzzx::batch::kNumClasses] = {0, 0, 0};  // mode 4: persistent grid of each class
-  int warp_per_sm = 0;  // mode 2: resident CTAs of the lane-parallel kernel per SM (fewest over the distances)
+  // Mode 2: resident CTAs per SM of the lane-parallel kernel where every warp
+  // sweeps, fewest over the distances (0: not asked for yet).
+  mutable std::mutex lanes_mu;
+  mutable int warp_per_sm = 0;
   // modes 3 and 4: one side stream and one completion event per distance (or
   // class), and the fork event, created on first use
   std::vector<cudaStream_t> side;
@@ -496,6 +500,19 @@ void free_batch(xzzx_batch* b) {
   if (b->fork) cudaEventDestroy(b->fork);
   if (b->dev_block) cudaFree(b->dev_block);
   delete b;
+}
+// The fewest resident CTAs per SM of the lane-parallel kernels of a batch's
+// distances; cap: as configure_coop_chunks, whose shared memory goes to each
+// range.
+xzzx_status configure_lanes(std::vector<xzzx::batch::DistanceRange>& ranges, int cap, int* fewest) {
+  *fewest = 0;
+  for (xzzx::batch::DistanceRange& r : ranges) {
+    int per_sm = 0;
+    xzzx_status st = xzzx::batch::configure_coop_chunks(r.d, cap, r.n_classes, &r.coop_smem, &per_sm);
+    if (st) return st;
+    *fewest = *fewest ? std::min(*fewest, per_sm) : per_sm;
+  }
+  return XZZX_OK;
 }
 xzzx_status ensure_side_streams(xzzx_batch* b, size_t n) {
   while (b->side.size() < n) {
@@ -634,14 +651,11 @@ xzzx_status xzzx_batch_create(const xzzx_segment* segs, int n_segs, uint64_t see
     if (cfg && cfg->ctas_per_sm > 0) cls_per_sm = std::min(cls_per_sm, cfg->ctas_per_sm);
     b->class_grid[r.cls] = n_sm * cls_per_sm;
   }
-  b->warp_per_sm = 0;
-  for (DistanceRange& r : b->plan.ranges) {
-    int w_per_sm = 0;
-    if ((st = configure_coop_chunks(r.d, cfg ? cfg->ctas_per_sm : 0, r.n_classes, &r.coop_smem, &w_per_sm))) {
-      free_batch(b);
-      return st;
-    }
-    b->warp_per_sm = b->warp_per_sm ? std::min(b->warp_per_sm, w_per_sm) : w_per_sm;
+  // Without a cap mode 2 needs no preparation, and its kernels are loaded (21 ms
+  // in a process that has not used them) when it runs or its occupancy is asked for.
+  if (cfg && cfg->ctas_per_sm > 0 && (st = configure_lanes(b->plan.ranges, cfg->ctas_per_sm, &b->warp_per_sm))) {
+    free_batch(b);
+    return st;
   }
   b->graph_mode = cfg ? cfg->graph_mode : 0;
   if (b->graph_mode != 0 && b->graph_mode != 3 && b->graph_mode != 4) {
@@ -707,6 +721,16 @@ xzzx_status xzzx_batch_get_info(const xzzx_batch* b, xzzx_batch_info* out) {
   out->total_shots = b->plan.total_shots;
   out->chains_per_cta = b->plan.nt;
   out->sweep_unroll = b->plan.unroll;
+  std::lock_guard<std::mutex> lk(b->lanes_mu);
+  if (b->warp_per_sm == 0) {
+    int cur = -1;
+    XZZX_CUDA_TRY(cudaGetDevice(&cur));
+    if (cur != b->device) XZZX_CUDA_TRY(cudaSetDevice(b->device));
+    std::vector<DistanceRange> ranges = b->plan.ranges;
+    const xzzx_status st = configure_lanes(ranges, 0, &b->warp_per_sm);
+    if (cur != b->device) XZZX_CUDA_TRY(cudaSetDevice(cur));
+    if (st) return st;
+  }
   out->warp_ctas_per_sm = b->warp_per_sm;
   return XZZX_OK;
 }
