@@ -13,7 +13,6 @@ struct AnnealArgs {
   PhiloxKeys keys;
   uint64_t chain0;  // global id of local chain 0
   int64_t n_chains;
-  int restarts;
   int n_sweeps, n_classes, n_live;
   int32_t W[4];
   const uint32_t* T;
@@ -125,7 +124,6 @@ xzzx_status launch_anneal(const xzzx_code* code, const xzzx_schedule* sched, uin
   A.keys = philox_keys(seed);
   A.chain0 = shot0 * (uint64_t)restarts * 4u;
   A.n_chains = (int64_t)n_shots * restarts * 4;
-  A.restarts = restarts;
   A.n_sweeps = sched->n_sweeps;
   A.n_classes = sched->n_classes;
   A.n_live = sched->n_live[kLayoutRotated];

@@ -258,8 +258,7 @@ __device__ __forceinline__ void colour_phase(Row (&R)[D], int32_t& E, const uint
     const Row m_top = (Row)0x6u << s;  // X on TL, Z on TR
     const Row m_bot = (Row)0x9u << s;  // Z on BL, X on BR
     // Group by group (the faces that share one Philox block): a group's
-    // lookups, draw and moves finish before the next group's lookups.  Against
-    // loading the whole column first this is 2% faster at d = 17, 21 and lets
+    // lookups, draw and moves finish before the next group's lookups, which lets
     // d = 29, 31 fit 128 registers without spills.
 #pragma unroll
     for (int g = 0; g < NG; ++g) {

@@ -247,7 +247,6 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
   P.segs.resize(n_segs);
   P.cta_prefix.assign(n_segs + 1, 0);
   P.shot_prefix.assign(n_segs + 1, 0);
-  P.chain_prefix.assign(n_segs + 1, 0);
   size_t ws = 0;
   std::vector<ChunkDev> chunks;
   // Restarts per greedy warp of the small and of the large distances: the
@@ -297,16 +296,9 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
     ws = align256(ws + n * R);
     d.chain_E = (int32_t*)(ws_base ? ws_base + ws : nullptr);
     ws = align256(ws + sizeof(int32_t) * n * R * 4);
-    d.T = s.sched->d_T;
-    d.sig = s.sched->d_sig;
-    d.n_sweeps = s.sched->n_sweeps;
-    d.n_classes = s.sched->n_classes;
-    d.n_live = s.sched->n_live[kLayoutRotated];
-    for (int k = 0; k < 4; ++k) d.W[k] = s.sched->noise.W[k];
     P.cta_prefix[j + 1] = P.cta_prefix[j] + (int64_t)s.n_shots * d.greedy_groups;
     if (!big) P.small_cta_end = P.cta_prefix[j + 1];
     P.shot_prefix[j + 1] = P.shot_prefix[j] + s.n_shots;
-    P.chain_prefix[j + 1] = P.chain_prefix[j] + (int64_t)s.n_shots * s.restarts * 4;
     P.dmax = std::max(P.dmax, s.code->d);
     const int64_t nch = (int64_t)s.n_shots * s.restarts * 4;
     if (nch > 0x7FFFFFFFll) return fail(XZZX_EINVAL, "segment too large");
@@ -368,7 +360,7 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
 
 namespace {
 struct BlobLayout {
-  size_t segs, lpt, byd, bycls, cta, shot, chain, head, total;
+  size_t segs, lpt, byd, bycls, cta, shot, head, total;
 };
 BlobLayout blob_layout(size_t n_segs, size_t n_chunks) {
   BlobLayout L;
@@ -379,8 +371,7 @@ BlobLayout blob_layout(size_t n_segs, size_t n_chunks) {
   L.bycls = align256(L.byd + sizeof(ChunkDev) * nc);
   L.cta = align256(L.bycls + sizeof(ChunkDev) * nc);
   L.shot = align256(L.cta + sizeof(int64_t) * (n_segs + 1));
-  L.chain = align256(L.shot + sizeof(int64_t) * (n_segs + 1));
-  L.head = align256(L.chain + sizeof(int64_t) * (n_segs + 1));
+  L.head = align256(L.shot + sizeof(int64_t) * (n_segs + 1));
   L.total = align256(L.head + sizeof(int) * (1 + kNumClasses));
   return L;
 }
@@ -399,7 +390,6 @@ PlanDev descriptor_layout(const Plan& p, char* base) {
   d.bycls = (ChunkDev*)(base + L.bycls);
   d.cta_prefix = (int64_t*)(base + L.cta);
   d.shot_prefix = (int64_t*)(base + L.shot);
-  d.chain_prefix = (int64_t*)(base + L.chain);
   d.head = (int*)(base + L.head);
   return d;
 }
@@ -415,7 +405,6 @@ void pack_descriptors(const Plan& p, char* blob) {
   }
   std::memcpy(blob + L.cta, p.cta_prefix.data(), sizeof(int64_t) * p.cta_prefix.size());
   std::memcpy(blob + L.shot, p.shot_prefix.data(), sizeof(int64_t) * p.shot_prefix.size());
-  std::memcpy(blob + L.chain, p.chain_prefix.data(), sizeof(int64_t) * p.chain_prefix.size());
 }
 
 xzzx_status configure_plan_kernels(int dmax, int nt, int unroll, int* ctas_per_sm) {

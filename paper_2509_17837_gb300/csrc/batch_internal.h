@@ -25,15 +25,10 @@ struct SegDev {
   uint32_t* init;     // workspace: n_shots x restarts x 2w words
   uint8_t* cbits;     // workspace: n_shots x restarts
   int32_t* chain_E;   // workspace: n_shots x restarts x 4
-  // schedule (also carried by every chunk of the segment)
-  const uint32_t* T;
-  const int2* sig;
-  int n_sweeps, n_classes, n_live;
-  int32_t W[4];
 };
 
 // Up to NT (the plan's chains per CTA) consecutive chains of one segment (one
-// CTA's work).
+// CTA's work), with the segment's schedule.
 struct ChunkDev {
   int seg, d, first_chain, n_chains;
   const uint32_t* T;
@@ -86,7 +81,7 @@ struct Plan {
   std::vector<SegDev> segs;
   std::vector<ChunkDev> lpt, byd, bycls;  // longest first; by distance; by class, longest first
   std::vector<ClassRange> classes;
-  std::vector<int64_t> cta_prefix, shot_prefix, chain_prefix;
+  std::vector<int64_t> cta_prefix, shot_prefix;
   std::vector<DistanceRange> ranges;
   int dmax = 0;
   double attempts = 0;
@@ -104,7 +99,6 @@ struct PlanDev {
   ChunkDev* bycls;
   int64_t* cta_prefix;
   int64_t* shot_prefix;
-  int64_t* chain_prefix;
   int* head;  // 1 + kNumClasses queue heads: mode 0's, then one per class (mode 4)
 };
 
