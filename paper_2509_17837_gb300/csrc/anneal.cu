@@ -87,9 +87,9 @@ xzzx_status launch_d(const AnnealArgs& A, cudaStream_t stream) {
   static DeviceOnce once;
   if constexpr (D <= kNarrowMaxD) {
     static DeviceOnce once_narrow;
-    int dev = 0, n_sm = 0;
-    XZZX_CUDA_TRY(cudaGetDevice(&dev));
-    XZZX_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    int n_sm = 0;
+    xzzx_status st = sm_count(&n_sm);
+    if (st) return st;
     if (A.n_chains <= (int64_t)32 * kNarrowWarps * n_sm)
       return launch_kernel<32>(anneal_narrow_kernel<D>, once_narrow, smem_bytes<D, 32>(), A, stream);
   }

@@ -102,7 +102,7 @@ xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm)
 // of a sweep on the table of thresholds).
 xzzx_status coop_is_faster(int d, int64_t n_chains, bool* yes) {
   int n_sm = 0;
-  xzzx_status st = coop::sm_count(&n_sm);
+  xzzx_status st = sm_count(&n_sm);
   if (st) return st;
   const int pairs = (d + 1) / 2;
   int lanes = 2;

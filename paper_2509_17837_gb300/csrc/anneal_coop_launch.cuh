@@ -53,13 +53,6 @@ __global__ void __launch_bounds__(Form<Geo, NC, NP, PER>::kThreads, PER)
                                    A.keys, smem);
 }
 
-xzzx_status sm_count(int* n_sm) {
-  int dev = 0;
-  XZZX_CUDA_TRY(cudaGetDevice(&dev));
-  XZZX_CUDA_TRY(cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev));
-  return XZZX_OK;
-}
-
 template <class Geo, int NC, int NP, int PER>
 xzzx_status launch_form(const Args& A, cudaStream_t stream) {
   using F = Form<Geo, NC, NP, PER>;

@@ -11,7 +11,7 @@ namespace xzzx {
 // = 9, 1.05 / 0.41 at d = 15; 32,768 chains 0.12 / 0.19, 0.53 / 0.96, 1.39 / 1.40.
 xzzx_status coop_planar_is_faster(int d, int64_t n_chains, bool* yes) {
   int n_sm = 0;
-  xzzx_status st = coop::sm_count(&n_sm);
+  xzzx_status st = sm_count(&n_sm);
   if (st) return st;
   *yes = d > 15 || n_chains <= (int64_t)n_sm * (d <= 11 ? 64 : 128);
   return XZZX_OK;

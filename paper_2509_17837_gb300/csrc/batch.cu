@@ -249,6 +249,8 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
   P.shot_prefix.assign(n_segs + 1, 0);
   size_t ws = 0;
   std::vector<ChunkDev> chunks;
+  int n_sm = 0;
+  XZZX_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device));
   // Restarts per greedy warp of the small and of the large distances: the
   // largest count that leaves each launch enough CTAs.
   int rpw[2] = {1, 1};
@@ -263,8 +265,8 @@ xzzx_status build_plan(const xzzx_segment* segs, int n_segs, int device, int ord
       return n;
     };
     for (int r = greedy::kMaxRestartsPerWarp; r > 1 && rpw[big] == 1; r >>= 1)
-      if (ctas(r) >= greedy::min_ctas(big == 1)) rpw[big] = r;
-    few[big] = 2 * ctas(1) <= greedy::kFewCtas;
+      if (ctas(r) >= greedy::min_ctas(big == 1, n_sm)) rpw[big] = r;
+    few[big] = greedy::few_ctas(ctas(1), n_sm);
   }
   for (int j = 0; j < n_segs; ++j) {
     const xzzx_segment& s = segs[order[j]];

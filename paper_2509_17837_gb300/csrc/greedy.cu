@@ -56,12 +56,15 @@ xzzx_status launch_greedy(const xzzx_code* code, const xzzx_noise* noise, uint64
   A.n_shots = n_shots;
   A.restarts = restarts;
   A.randomised = randomised;
+  int n_sm = 0;
+  xzzx_status st = sm_count(&n_sm);
+  if (st) return st;
   const bool scan = randomised != kInitBoundary && scans(A.code, *noise, restarts);
-  const int warps = choose_warps(A.code, n_shots, restarts, randomised, scan);
+  const int warps = choose_warps(A.code, n_shots, restarts, randomised, scan, n_sm);
   int rpw = 1;
   for (int r = kMaxRestartsPerWarp; r > 1 && rpw == 1 && !scan; r >>= 1)  // a scan has no lists to share
-    if ((int64_t)n_shots * greedy_groups(restarts, warps, r) >= min_ctas(is_large(A.code))) rpw = r;
-  const bool few = 2 * (int64_t)n_shots * greedy_groups(restarts, warps, 1) <= kFewCtas;
+    if ((int64_t)n_shots * greedy_groups(restarts, warps, r) >= min_ctas(is_large(A.code), n_sm)) rpw = r;
+  const bool few = few_ctas((int64_t)n_shots * greedy_groups(restarts, warps, 1), n_sm);
   const Cut cut = cut_of(A.code, warps, restarts, randomised, rpw, few, scan);
   A.groups = cut.groups;
   A.cols = cut.cols;

@@ -53,15 +53,16 @@ namespace greedy {
 // take long to build and most of the shared memory, 4 where there is too little
 // for 8 to do.
 constexpr int kFewWarps = 4, kSmallWarps = 8, kLargeWarps = 16, kSmallFaces = 150;
-// A launch of no more CTAs than this gives each restart two warps, one per colour.
-constexpr int64_t kFewCtas = 152;
+// A launch of at most one CTA per two SMs gives each restart two warps, one per colour.
+inline bool few_ctas(int64_t n, int n_sm) { return 2 * n <= n_sm; }
 // A launch takes the largest restarts-per-warp count (8, 4, 2 or 1) that still
 // gives it enough CTAs: large launches then share each CTA's setup across more
 // restarts, small ones keep their CTAs.  Lists of small codes cost little next
-// to a restart, and several waves of CTAs fill the launch's tail; the lists of
-// larger codes cost about as much as one restart, so two CTAs per SM are enough.
+// to a restart, and several waves of CTAs (13 per SM) fill the launch's tail; the
+// lists of larger codes cost about as much as one restart, so two CTAs per SM are
+// enough.
 constexpr int kMaxRestartsPerWarp = 8;
-inline int64_t min_ctas(bool large) { return large ? 304 : 2048; }
+inline int64_t min_ctas(bool large, int n_sm) { return (int64_t)n_sm * (large ? 2 : 13); }
 // CTAs of a shot's restarts at rpw restarts per warp.
 inline int greedy_groups(int restarts, int warps, int rpw) { return (restarts + warps * rpw - 1) / (warps * rpw); }
 // Reference modes: greedy matching with lexicographic ties (Alg. 5), with
@@ -709,20 +710,20 @@ inline Cut cut_of(const DevCode& C, int warps, int restarts, int mode, int rpw, 
 }
 
 // Warps per CTA of a launch.
-inline int choose_warps(const DevCode& C, int64_t n_shots, int restarts, int mode, bool scan) {
+inline int choose_warps(const DevCode& C, int64_t n_shots, int restarts, int mode, bool scan, int n_sm) {
   const int half = C.ns / 2;
   // Past one wave of eight-warp CTAs, where a shot has not enough to keep them
   // busy, narrow ones hold twice the shots on an SM (p = 0.14, us, 8 warps / 4: 1000
   // shots x 1 restart d = 3 13.8 / 8.5, d = 9 28.5 / 20.8, d = 17 91 / 87; 1000 x 3 d = 5
   // 19.1 / 17.3, d = 17 98 / 114; 300 x 64 d = 3 34.7 / 30.2).
-  if (half <= kSmallFaces && !scan && n_shots * greedy_groups(restarts, kSmallWarps, 1) > 608 &&
+  if (half <= kSmallFaces && !scan && n_shots * greedy_groups(restarts, kSmallWarps, 1) > 4 * n_sm &&
       (half <= 6 || restarts <= 2 || (restarts == 3 && (half <= 12 || mode == kInitBoundary))))
     return kFewWarps;
   if (!is_large(C) || scan) return kSmallWarps;
   // Boundary references of a large code build no lists: its wide CTAs only pay
   // while all of them are resident (1000 shots x 1, us, 16 warps with the lists'
   // memory / 8 without: rotated d = 21 54 / 32, d = 31 182 / 67).
-  return mode == kInitBoundary && n_shots * greedy_groups(restarts, kLargeWarps, 1) > min_ctas(true) ? kSmallWarps
+  return mode == kInitBoundary && n_shots * greedy_groups(restarts, kLargeWarps, 1) > min_ctas(true, n_sm) ? kSmallWarps
                                                                                                      : kLargeWarps;
 }
 

@@ -45,6 +45,13 @@ xzzx_status check_code(const xzzx_code* code) {
   return check_device(code->device);
 }
 
+xzzx_status sm_count(int* n_sm) {
+  int dev = 0;
+  XZZX_CUDA_TRY(cudaGetDevice(&dev));
+  XZZX_CUDA_TRY(cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev));
+  return XZZX_OK;
+}
+
 xzzx_status check_device(int device) {
   int cur = -1;
   XZZX_CUDA_TRY(cudaGetDevice(&cur));

@@ -203,5 +203,7 @@ namespace xzzx {
 // Validation helpers shared by the entry points.
 xzzx_status check_code(const xzzx_code* code);
 xzzx_status check_device(int device);
+// SMs of the current device.
+xzzx_status sm_count(int* n_sm);
 xzzx_status check_ptr(const void* p, const char* name);
 }  // namespace xzzx
