@@ -93,13 +93,22 @@ xzzx_status configure_g(int cap, int n_classes, int* smem_out, int* ctas_per_sm)
 // Whether a launch of n_chains distance-d chains is faster with several lanes
 // per chain than with one thread per chain, whose time is that of one chain's
 // sweeps until its warps fill the GPU.  The lanes' throughput is in proportion to
-// the share of them that hold rows, (d+1)/2 of a power of two.  One thread / this
-// kernel at 80, 120, 144, 180, 220 chains per SM (200 sweeps, p = 0.15, eta = 100):
-// d = 5 1.51, 1.36, 1.22, 0.93, 0.81; d = 7 1.81, 1.49, 1.49, 1.09, 0.94; d = 9 1.29, 1.07,
-// 1.00, 0.89, 0.73; d = 11 1.32, 1.12, 1.06, 0.93, 0.76; d = 15 1.52, 1.31, 1.29, 1.13, 0.93;
-// d = 17 1.28, 0.91, 0.99, 0.83; d = 25 1.44, 1.00, 1.26, 1.03; d = 31 1.66, 1.16, 1.44, 1.18;
-// d = 3 1.42, 1.41, 1.31, 1.31, 1.18, and 1.13 at 300 (its thread kernel spends a quarter
-// of a sweep on the table of thresholds).
+// the share of them that hold rows, (d+1)/2 of a power of two.  The line is where the
+// schedule with dense draws (50 sweeps near the Nishimori temperature; the first of
+// each pair) crosses; the one with sparse draws (200 sweeps to 20 times it) crosses
+// later.  Thread time / lane time at chains per SM:
+//   d     100         140         160         180         200         220
+//   5  1.18 1.29   1.08 1.19   1.09 1.19   0.79 0.83   0.73 0.80   0.73 0.80
+//   7  1.48 1.56   1.42 1.47   1.40 1.44   1.03 1.06   0.96 1.00   0.96 0.99
+//   9  1.07 1.21   0.96 1.04   0.91 0.97   0.79 0.91   0.71 0.80   0.67 0.75
+//  11  1.18 1.32   1.04 1.12   0.96 1.06   0.84 0.98   0.75 0.86   0.72 0.81
+//  15  1.51 1.45   1.36 1.37   1.27 1.27   1.10 1.18   0.99 1.03   0.94 0.97
+//  17  0.97 1.15   0.88 1.09   0.80 0.99   0.70 0.89   0.64 0.79   0.58 0.74
+//  21  1.04 1.22   0.96 1.21   0.88 1.09   0.77 0.96   0.70 0.87   0.64 0.80
+//  25  1.19 1.25   1.23 1.37   1.11 1.23   0.98 1.08   0.89 0.97   0.80 0.89
+//  29  1.29 1.30   1.33 1.44   1.20 1.29   1.05 1.14   0.96 1.02   0.87 0.94
+//  31  1.42 1.42   1.48 1.57   1.33 1.41   1.17 1.24   1.07 1.11   0.96 1.02
+// d = 3 stays above 0.97 up to 280.
 xzzx_status coop_is_faster(int d, int64_t n_chains, bool* yes) {
   int n_sm = 0;
   xzzx_status st = sm_count(&n_sm);
@@ -107,7 +116,7 @@ xzzx_status coop_is_faster(int d, int64_t n_chains, bool* yes) {
   const int pairs = (d + 1) / 2;
   int lanes = 2;
   while (lanes < pairs) lanes *= 2;
-  *yes = n_chains <= (int64_t)n_sm * (d == 3 ? 280 : (d <= 15 ? 200 : 165) * pairs / lanes);
+  *yes = n_chains <= (int64_t)n_sm * (d == 3 ? 280 : (d <= 15 ? 200 : d <= 23 ? 165 : 205) * pairs / lanes);
   return XZZX_OK;
 }
 

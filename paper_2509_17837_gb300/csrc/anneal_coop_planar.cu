@@ -6,14 +6,25 @@ namespace xzzx {
 // Whether a planar launch takes several lanes per chain.  d > 15: always (one
 // thread per chain with its rows in shared memory leaves room for two CTAs per SM:
 // 131,072 chains x 50 sweeps, 42.4 -> 11.8 ms at d = 17, 242 -> 20.8 ms at d =
-// 31).  Below, against the register-resident kernel, 50 sweeps near the
-// Nishimori temperature, ms: 8,192 chains 0.12 / 0.08 at d = 3, 0.42 / 0.29 at d
-// = 9, 1.05 / 0.41 at d = 15; 32,768 chains 0.12 / 0.19, 0.53 / 0.96, 1.39 / 1.40.
+// 31).  Below, against the register-resident kernel, by the share of the lanes that
+// hold rows (d of a power of two), at the crossing with dense draws.  Thread time /
+// lane time, 50 sweeps near the Nishimori temperature and 200 to 20 times it, at
+// chains per SM:
+//   d      60          80         100         150         180         200
+//   3  1.11 1.19   0.94 1.06   0.78 0.91   0.74 0.79   0.64 0.70   0.53 0.59
+//   5  1.41 1.44   1.19 1.22   0.83 0.91   0.72 0.80   0.60 0.69   0.57 0.64
+//   7  2.11 2.19   1.52 1.61   1.21 1.43   1.07 1.18   0.93 1.01   0.85 0.93
+//   9  1.29 1.59   1.03 1.23   0.81 1.01   0.73 0.93   0.61 0.78   0.56 0.72
+//  11  1.51 1.79   1.21 1.41   0.95 1.15   0.84 1.06   0.70 0.92   0.64 0.83
+//  13  1.90 2.10   1.52 1.65   1.19 1.35   1.05 1.29   0.88 1.10   0.80 1.00
+//  15  2.23 2.40   1.77 1.84   1.39 1.51   1.24 1.47   1.04 1.29   0.95 1.18
 xzzx_status coop_planar_is_faster(int d, int64_t n_chains, bool* yes) {
   int n_sm = 0;
   xzzx_status st = sm_count(&n_sm);
   if (st) return st;
-  *yes = d > 15 || n_chains <= (int64_t)n_sm * (d <= 11 ? 64 : 128);
+  int lanes = 4;
+  while (lanes < d) lanes *= 2;
+  *yes = d > 15 || n_chains <= (int64_t)n_sm * (d == 3 ? 64 : (8 * d > 6 * lanes ? 190 : 135) * d / lanes);
   return XZZX_OK;
 }
 
