@@ -31,7 +31,9 @@ sys.path.insert(0, ROOT)
 
 D, ETA, PS, RESTARTS, SWEEPS, BETA0, BETA1, SCALE = 11, 100.0, (0.10, 0.13, 0.16, 0.19, 0.22), 64, 1000, 0.05, 20.0, 1024
 SEED = 0xD11
-I_ALG = 30  # integer instructions per move attempt in the algorithmic count
+# Lane instructions that an executed move attempt cannot do without: signature,
+# load, compare, two updates and its share of a draw block.
+FLOOR_INST = 11
 # Counters of anneal_kernel<11> from an ncu capture: DRAM bytes (read + write)
 # per chain, ALU-pipe lane instructions per move attempt
 # (sm__inst_executed_pipe_alu x 32 / attempts; the ALU pipe takes 16 lanes per
@@ -55,7 +57,7 @@ ANNEAL_D31_MEASURED = {"inst_per_attempt": 15.95, "alu_inst_per_attempt": 9.91,
                                  "sweeps, profiles/anneal_ncu_counters.md"}
 ATTEMPTS_NOTE = ("attempts are those of the schedule; in its frozen sweeps (every acceptance threshold zero) a warp "
                  "whose 32 chains have all returned to an earlier configuration stops, since no later sweep can "
-                 "change its minima; the roofline counts the attempts of the live sweeps only")
+                 "change its minima")
 
 
 def live_share(sched):
@@ -179,12 +181,21 @@ def issue_peak(clocks, n_sm):
             "%d SMs x 4 SMSP x 32 lanes x %.0f MHz (median SM clock sampled in the timed region)" % (n_sm, f_mhz))
 
 
-def roofline_record(rate_attempts, live, clocks, n_sm, **extra):
+def roofline_record(rate_attempts, live, clocks, n_sm, measured=None, **extra):
+    """The integer issue peak's share.  measured: the kernel's counters (see
+    ANNEAL_MEASURED); achieved is then the lane instructions it executes, frac the
+    share of the issue slots they take.  Without counters achieved is the floor's:
+    the FLOOR_INST instructions of every attempt of the live sweeps."""
     peak, basis = issue_peak(clocks, n_sm)
-    achieved = rate_attempts * live * I_ALG / 1e12
+    floor = rate_attempts * live * FLOOR_INST / 1e12
+    achieved = rate_attempts * measured["inst_per_attempt"] / 1e12 if measured else floor
     rec = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tinst/s",
-           "frac": (achieved / peak) if peak else None, "I_alg_per_attempt": I_ALG, "live_share": live,
+           "frac": (achieved / peak) if peak else None,
+           "counted": "lane instructions executed" if measured else "lane instructions of the floor",
+           "floor_inst_per_live_attempt": FLOOR_INST, "floor_frac": (floor / peak) if peak else None, "live_share": live,
            "attempts_note": ATTEMPTS_NOTE, "peak_basis": basis}
+    if measured:
+        rec["measured_per_attempt"] = measured
     rec.update(extra)
     return rec
 
@@ -683,7 +694,7 @@ def run_large(args):
         "roofline": roofline_record(att, statistics.fmean(live_share(c[1]) for c in cases), clocks, props.multi_processor_count,
                                     traffic=(None if ANNEAL_D31_DRAM_BYTES_PER_CHAIN is None
                                              else ANNEAL_D31_DRAM_BYTES_PER_CHAIN * S * R * 4),
-                                    kernel="anneal_kernel<31>", measured_per_attempt=ANNEAL_D31_MEASURED)}))
+                                    kernel="anneal_kernel<31>", measured=ANNEAL_D31_MEASURED)}))
 
 
 # --------------------------------------------------------------------------- logical error rate curves
@@ -923,7 +934,7 @@ def main():
             anneal_rate, statistics.fmean(live_share(c["sched"]) for c in cases), clocks, n_sm,
             traffic=None if ANNEAL_DRAM_BYTES_PER_CHAIN is None else ANNEAL_DRAM_BYTES_PER_CHAIN * S * RESTARTS * 4,
             kernel="anneal_kernel<11>",
-            measured_per_attempt=ANNEAL_MEASURED,
+            measured=ANNEAL_MEASURED,
             secondary_alu_pipe=None if not (f_mhz and ANNEAL_ALU_INST_PER_ATTEMPT) else {
                 "alu_inst_per_attempt": ANNEAL_ALU_INST_PER_ATTEMPT,
                 "peak_attempts_per_s": n_sm * 4 * 16 * f_mhz * 1e6 / ANNEAL_ALU_INST_PER_ATTEMPT,
