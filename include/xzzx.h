@@ -305,8 +305,9 @@ typedef struct {
 } xzzx_segment;
 
 typedef struct {
-  int32_t ctas_per_sm;    /* persistent grid = SMs x this; 0 = the occupancy maximum.  Mode 2: resident
-                             four-warp CTAs per SM capped at this by padding each CTA's shared memory */
+  int32_t ctas_per_sm;    /* persistent grid = SMs x this; 0 = the occupancy maximum.  Mode 2: the form where
+                             every warp sweeps, its resident CTAs per SM capped at this by padding each CTA's
+                             shared memory */
   int32_t order;          /* chunk queue: 0 = longest chunks first, 1 = segment order */
   int32_t graph_mode;     /* the mode xzzx_batch_run_graph captures: 0, 3 or 4 */
   int32_t chains_per_cta; /* chains per CTA of the annealing launches (chunk size): 128 or 256; 0 = 128 */
@@ -321,7 +322,9 @@ typedef struct {
   int64_t total_shots;
   int32_t chains_per_cta, sweep_unroll;
   int32_t n_classes;     /* distance classes present (d <= 15, 17..21, 23..31): mode 4's launches */
-  int32_t warp_ctas_per_sm; /* mode 2: resident four-warp CTAs per SM, fewest over the distances */
+  int32_t warp_ctas_per_sm; /* mode 2: resident CTAs per SM of its four-warp form where every warp sweeps, fewest
+                               over the distances (small uncapped launches take CTAs of one sweeping warp and
+                               three that draw for it) */
 } xzzx_batch_info;
 
 typedef struct xzzx_batch xzzx_batch;

@@ -10,11 +10,11 @@
 //   mode 1 (plain):   the same three kernels once per distance;
 //   mode 2 (latency): as mode 1 with several lanes per chain.
 // Every chain uses the chain id it would get from xzzx_decode_batch on its
-// segment alone, so both modes, and per-segment calls, agree bit for bit.
+// segment alone, so every mode, and per-segment calls, agree bit for bit.
 //
 // xzzx_batch_* owns one allocation holding a plan's descriptors and
-// workspace; xzzx_batch_run_graph captures mode 0 into a CUDA graph on its
-// first call and replays it afterwards.  The decode server (serve.cu) builds
+// workspace; xzzx_batch_run_graph captures its graph mode (0, 3 or 4) into a CUDA
+// graph on its first call and replays it afterwards.  The decode server (serve.cu) builds
 // plans into memory it allocated up front.
 #include <algorithm>
 #include <cstring>

@@ -39,9 +39,9 @@ __device__ __forceinline__ void run_chunk(const ChunkDev& ch, const SegDev& sg, 
 }
 
 // Threads per SM that a kernel of distances up to D is register-bounded for: 1024
-// (64 registers) up to d = 15, 512 (128) up to d = 27, 384 (160) above.  Left
-// alone, the compiler takes up to 240 registers for the persistent kernels: two
-// CTAs per SM.
+// (64 registers) up to d = 15, 512 (128) up to d = 27, 384 (160) above; there a CTA
+// of 256 chains is the only one of its SM and the compiler's choice holds.  Left
+// alone, it takes up to 240 registers for the persistent kernels: two CTAs per SM.
 template <int D>
 constexpr int kSmThreads = D <= 15 ? 1024 : D <= 27 ? 512 : 384;
 
@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(NT, (DMAX <= 21 ? kSmThreads<DMAX> : 384) / NT
     dispatch_chunk<3, DMAX, NT, U>(ch, L.segs[ch.seg], L.keys, smem);
   }
 }
+
 // The largest shared memory of any distance the persistent kernel runs.
 template <int DMAX, int NT, int D = 3>
 constexpr size_t persistent_smem() {

@@ -34,8 +34,8 @@
 // code's own size, and one list buffer serves the two colours of a large code in
 // turn.  Against lists for rotated d <= 17 only and a fixed carve for d = 31
 // (identical references): 76 shots x 256 restarts at d = 31, p = 0.24 13.6 -> 2.85
-// ms; 4000 x 100 planar d = 9 7.59 -> 2.54 ms; 100 x 100 planar d = 21 3.82 ->
-// 1.24 ms; 4000 x 64 at d = 11 1.94 -> 1.77 ms; one shot x 32 at d = 25 0.58 -> 0.13
+// ms; 4000 x 100 planar d = 9 7.59 -> 2.35 ms; 100 x 100 planar d = 21 3.82 ->
+// 1.05 ms; 4000 x 64 at d = 11 1.94 -> 1.69 ms; one shot x 32 at d = 25 0.58 -> 0.12
 // ms.
 #pragma once
 
@@ -121,7 +121,7 @@ struct PlanarGeo {
 // at least 64 and at most 256 (list entries are bytes).  None for colours of
 // more than 800 faces (planar d >= 29), which mostly hold more than 256 defects:
 // the lists' memory would only lower the occupancy of the scan that then runs
-// (d = 31, p = 0.12: 4.96 against 4.26 ms).
+// (d = 31, p = 0.12: 4.96 against 4.26 ms, before three scanning CTAs fitted an SM).
 __host__ __device__ inline int list_room(int faces_per_colour) {
   const int n = (faces_per_colour * 35 / 64 + 31) / 32 * 32;
   return faces_per_colour > 800 ? 0 : n < 64 ? 64 : n > 256 ? 256 : n;
@@ -715,7 +715,8 @@ inline int choose_warps(const DevCode& C, int64_t n_shots, int restarts, int mod
   // Past one wave of eight-warp CTAs, where a shot has not enough to keep them
   // busy, narrow ones hold twice the shots on an SM (p = 0.14, us, 8 warps / 4: 1000
   // shots x 1 restart d = 3 13.8 / 8.5, d = 9 28.5 / 20.8, d = 17 91 / 87; 1000 x 3 d = 5
-  // 19.1 / 17.3, d = 17 98 / 114; 300 x 64 d = 3 34.7 / 30.2).
+  // 19.1 / 17.3, d = 17 98 / 114; 300 x 64 d = 3 34.7 / 30.2, with lists for two
+  // vertices too; without them 1000 x 8 at d = 3 19.0 -> 16.1).
   if (half <= kSmallFaces && !scan && n_shots * greedy_groups(restarts, kSmallWarps, 1) > 4 * n_sm &&
       (half <= 6 || restarts <= 2 || (restarts == 3 && (half <= 12 || mode == kInitBoundary))))
     return kFewWarps;
