@@ -17,7 +17,7 @@ namespace {
 // Batched form: the chunks of one distance, each cut into CTAs of kCtaChains
 // chains (so a CTA's chains share a segment and its thresholds).
 template <class Geo, int NC, int NP, int PER>
-__global__ void __launch_bounds__(Form<Geo, NC, NP, PER>::kThreads, PER)
+__global__ void __launch_bounds__(Form<Geo, NC, NP, PER>::kThreads, Form<Geo, NC, NP, PER>::kRegCtas)
     coop_chunks_kernel(const __grid_constant__ batch::CoopLaunch L) {
   constexpr int kCta = Form<Geo, NC, NP, PER>::kCtaChains;
   extern __shared__ __align__(16) uint8_t smem[];

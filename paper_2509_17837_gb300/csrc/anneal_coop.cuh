@@ -363,6 +363,7 @@ struct PlanarLanes : LaneShape<D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 16 : 32, (D -
   using S = LaneShape<D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 16 : 32, (D - 1) / 2, (D + 1) / 2, (D - 1) / 2, (D + 1) / 2, 0>;
   using Row = typename std::conditional<(D > 15), uint64_t, uint32_t>::type;
   static constexpr int NS = (D - 1) / 2;
+  static constexpr bool kByThree = D == 13 || D == 15;  // see sweeping_per_sm
   static constexpr int NR = sizeof(Row) / 4, NW = 2 * NR;
   static constexpr int kNQ = D * D + (D - 1) * (D - 1);
   static constexpr int kW = (kNQ + 31) / 32;
@@ -528,6 +529,7 @@ constexpr size_t kSmShared = 228 * 1024, kCtaReserved = 1024;  // shared memory 
 template <class Geo, int NC, int NP, int PER>
 struct Form {
   static constexpr int kThreads = 32 * (NC + NP), kPerSm = PER;
+  static constexpr int kRegCtas = NP ? PER : 4;  // CTAs per SM of the register bound (sweeping warps need no more than 128)
   static constexpr int kCtaChains = NC * Geo::kChains;
   static constexpr int kSets = NP ? 2 : 1;
   static constexpr int draw_words(int sweeps) {

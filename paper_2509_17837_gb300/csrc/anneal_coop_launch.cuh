@@ -43,7 +43,7 @@ inline Args make_args(const xzzx_code* code, const xzzx_schedule* sched, uint64_
 }
 
 template <class Geo, int NC, int NP, int PER>
-__global__ void __launch_bounds__(Form<Geo, NC, NP, PER>::kThreads, PER)
+__global__ void __launch_bounds__(Form<Geo, NC, NP, PER>::kThreads, Form<Geo, NC, NP, PER>::kRegCtas)
     anneal_coop_kernel(const __grid_constant__ Args A) {
   constexpr int kCta = Form<Geo, NC, NP, PER>::kCtaChains;
   extern __shared__ __align__(16) uint8_t smem[];
@@ -79,15 +79,29 @@ int producing_per_sm(int64_t n_chains, int n_sm) {
   return ctas <= 3 * n_sm ? 3 : ctas <= 4 * n_sm ? 4 : 0;
 }
 
+// CTAs per SM that the form where every warp sweeps is sized for.  Where that
+// changes its sweeps per set (planar: 8 at three, 4 at four) it is three while no more
+// are wanted -- fewer barriers -- and at d = 13, 15 where five or six would leave one
+// or two behind four.  Form sized for four / for three, ms, 30 sweeps near the
+// Nishimori temperature, d = 5: two CTAs per SM 0.050 / 0.045, four 0.079 / 0.100; 60
+// sweeps to 20 times it, d = 13: four 0.200 / 0.270, five 0.310 / 0.283, six 0.334 /
+// 0.317, eight 0.390 / 0.427.
+template <class Geo>
+int sweeping_per_sm(int64_t n_chains, int n_sm) {
+  const int64_t ctas = (n_chains + 4 * Geo::kChains - 1) / (4 * Geo::kChains), c = (ctas + n_sm - 1) / n_sm;
+  return c <= 3 || ((c == 5 || c == 6) && Geo::kByThree) ? 3 : 4;
+}
+
 template <class Geo>
 xzzx_status launch_g(const Args& A, cudaStream_t stream) {
   int n_sm = 0;
   xzzx_status st = sm_count(&n_sm);
   if (st) return st;
   const int per = producing_per_sm<Geo>(A.n_chains, n_sm);
-  return per == 3   ? launch_form<Geo, 1, 3, 3>(A, stream)
-         : per == 4 ? launch_form<Geo, 1, 3, 4>(A, stream)
-                    : launch_form<Geo, 4, 0, 4>(A, stream);
+  if (per) return per == 3 ? launch_form<Geo, 1, 3, 3>(A, stream) : launch_form<Geo, 1, 3, 4>(A, stream);
+  if constexpr (Form<Geo, 4, 0, 3>::kSweeps != Form<Geo, 4, 0, 4>::kSweeps)
+    if (sweeping_per_sm<Geo>(A.n_chains, n_sm) == 3) return launch_form<Geo, 4, 0, 3>(A, stream);
+  return launch_form<Geo, 4, 0, 4>(A, stream);
 }
 
 }  // namespace

@@ -44,6 +44,25 @@ def test_producing_forms_at_their_limits(env, planar, d):
                 assert torch.equal(many["best_E"][:take], few["best_E"])
 
 
+@pytest.mark.parametrize("d", [5, 7, 9, 13, 15, 17, 21, 31])
+def test_planar_sweeping_forms_at_their_limits(env, d):
+    """Every warp sweeping: two to six CTAs per SM and one more of each."""
+    X, torch = env
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    code, noise = X.Code(d, X.LAYOUT_PLANAR), X.noise_from_eta(0.15, 10.0)
+    shots = 70 * n_sm + 1
+    _, syn = X.sample_errors(code, noise, 5, 7, shots)
+    init, _ = X.greedy_init(code, noise, 5, 7, syn, 1)
+    sched = X.Schedule(noise, 37, 0.1, 60.0)
+    many = X.anneal(code, sched, 5, 7, init, want_cfg=True, want_final=True)
+    for per_sm in (2, 3, 4, 5, 6):
+        last = per_sm * n_sm * chains_per_cta(True, d)
+        for take in (last, last + 1):
+            few = X.anneal(code, sched, 5, 7, init[:take].contiguous(), want_cfg=True, want_final=True)
+            for k in many:
+                assert torch.equal(many[k][:take], few[k]), (k, take)
+
+
 @pytest.mark.parametrize("d", [7, 11, 17, 31])
 def test_batch_lane_forms_at_their_limits(env, d):
     """Batch mode 2, whose chunks of 128 chains are cut into the same forms."""

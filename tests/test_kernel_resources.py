@@ -31,10 +31,10 @@ LANE_FORMS = r"""
 using namespace xzzx::coop;
 template <class G>
 void forms(const char* name, int d) {
-  const int per[3] = {Form<G, 1, 3, 3>::kPerSm, Form<G, 1, 3, 4>::kPerSm, Form<G, 4, 0, 4>::kPerSm};
-  const size_t bytes[3] = {Form<G, 1, 3, 3>::smem_bytes(64), Form<G, 1, 3, 4>::smem_bytes(64),
-                           Form<G, 4, 0, 4>::smem_bytes(64)};
-  for (int k = 0; k < 3; ++k) std::printf("%s %d %d %zu\n", name, d, per[k], bytes[k]);
+  const int per[4] = {Form<G, 1, 3, 3>::kPerSm, Form<G, 1, 3, 4>::kPerSm, Form<G, 4, 0, 3>::kPerSm, Form<G, 4, 0, 4>::kPerSm};
+  const size_t bytes[4] = {Form<G, 1, 3, 3>::smem_bytes(64), Form<G, 1, 3, 4>::smem_bytes(64),
+                           Form<G, 4, 0, 3>::smem_bytes(64), Form<G, 4, 0, 4>::smem_bytes(64)};
+  for (int k = 0; k < 4; ++k) std::printf("%s %d %d %zu\n", name, d, per[k], bytes[k]);
 }
 template <int D>
 void upto() {
@@ -53,7 +53,7 @@ def test_lane_forms_fit_the_ctas_their_rules_count_on(tmp_path):
     exe = str(tmp_path / "forms")
     subprocess.run([build.nvcc(), str(tmp_path / "forms.cu"), "-o", exe] + build.NVCC_FLAGS, check=True)
     rows = [line.split() for line in subprocess.run([exe], capture_output=True, text=True, check=True).stdout.splitlines()]
-    assert len(rows) == 2 * 15 * 3
+    assert len(rows) == 2 * 15 * 4
     for lattice, d, per_sm, smem in rows:
         taken = -(-int(smem) // 128) * 128 + 1024
         assert int(per_sm) >= 3 and int(per_sm) * taken <= 228 * 1024, (lattice, d, per_sm, smem)
